@@ -1,14 +1,15 @@
 // Matrix-free stencil CG for the 19-point compact scheme (Section 2, eq. compact) and
 // the CG loop of Algorithm 1 (one step per pass of its WHILE loop).
 //
-// One CG step is two launches, both persistent over z-slab tiles of kTX x kTY columns:
+// One CG step is two launches (or two phases of a persistent one), both over tiles:
 //   k_dir_spmv_dot : p_new = r + beta p_old (p = r on the first step), q = A p_new,
 //                    partial sums of p.q; the last block forms alpha = r.r / p.q.
 //   k_update_dot   : x += alpha p, r -= alpha q, partial sums of r.r; the last block
 //                    forms beta, counts the step and applies the stopping test
 //                    ||r|| <= eps ||b|| (or the iteration cap).
-// The stencil marches in z through one shared-memory plane (with its x/y halo) at a
-// time: for each plane it forms per column
+// Float64 takes slabs whose 19-point sums run in block fixed point (fixed_slab.cuh).
+// Float32 tiles are kTX x kTY columns that march in z through one shared-memory plane (with
+// its x/y halo) at a time: for each plane a column forms
 //   C_k = c0 P + fx (P_{i-1}+P_{i+1}) + fy (P_{j-1}+P_{j+1}) + exy (4 xy-edge values)
 //   T_k = fz P + exz (P_{i-1}+P_{i+1}) + eyz (P_{j-1}+P_{j+1})
 // and (A p)_k = C_k + T_{k-1} + T_{k+1}: the z-face and z-edge terms of plane k are the
@@ -21,7 +22,9 @@
 
 #include <algorithm>
 
+#include "block_reduce.cuh"
 #include "excmg_internal.cuh"
+#include "fixed_slab.cuh"
 
 namespace excmg {
 
@@ -29,67 +32,6 @@ namespace {
 
 __device__ __forceinline__ double fmaT(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fmaT(float a, float b, float c) { return fmaf(a, b, c); }
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Sum over the block; the result is valid in thread 0.  Every thread must call.
-// float64 instructions are scarce on this GPU (2 per clock per SM, 64-clock latency), so
-// only warp 0 adds: every thread parks its value in shared memory, then each lane of
-// warp 0 sums blockDim/32 of them in a fixed order and the warp reduces by shuffles.
-// The order is fixed, so the result is deterministic.
-__device__ double block_sum(double v) {
-  __shared__ double s_v[kThreads];
-  const int lane = threadIdx.x & 31;
-  __syncthreads();
-  s_v[threadIdx.x] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x < 32) {
-    // kThreads / 32 values per lane as a pairwise tree (a short dependence chain)
-    double w[kThreads / 32];
-#pragma unroll
-    for (int u = 0; u < kThreads / 32; ++u) w[u] = s_v[lane + 32 * u];
-#pragma unroll
-    for (int d = 1; d < kThreads / 32; d *= 2)
-#pragma unroll
-      for (int u = 0; u + d < kThreads / 32; u += 2 * d) w[u] += w[u + d];
-    t = warp_sum(w[0]);
-  }
-  return t;
-}
-
-// Warp-0 sum of src[0 .. n) from global memory (through L2) in a fixed order: each lane
-// takes the values lane, lane + 32, ... in chunks of kSumChunk loads in flight, sums a
-// chunk as a pairwise tree, then the lanes reduce by shuffles.  Valid in lane 0.
-constexpr int kSumChunk = 8;
-__device__ __forceinline__ double warp0_sum_global(const double* src, int n) {
-  const int lane = threadIdx.x & 31;
-  double acc = 0.0;
-  for (int i0 = 0; i0 < n; i0 += 32 * kSumChunk) {
-    double w[kSumChunk];
-#pragma unroll
-    for (int u = 0; u < kSumChunk; ++u) {
-      const int i = i0 + lane + 32 * u;
-      w[u] = i < n ? __ldcg(src + i) : 0.0;
-    }
-#pragma unroll
-    for (int d = 1; d < kSumChunk; d *= 2)
-#pragma unroll
-      for (int u = 0; u + d < kSumChunk; u += 2 * d) w[u] += w[u + d];
-    acc += w[0];
-  }
-  return warp_sum(acc);
-}
-
-template <typename D>
-__device__ __forceinline__ int find_problem(const D* descs, int nprob, long long t, int p) {
-  while (p + 1 < nprob && t >= descs[p + 1].tile_begin) ++p;
-  return p;
-}
 
 struct TileXYZ {
   int x0, y0, z0, z1;
@@ -106,41 +48,6 @@ __device__ __forceinline__ TileXYZ tile_coords(const Grid3& g, const Tiling& tl,
   c.z0 = bz * tl.tz;
   c.z1 = min(c.z0 + tl.tz, g.nz + 1);
   return c;
-}
-
-// Publish this block's per-problem partial sums (NV values per problem) and let the
-// last block to arrive for problem p reduce the gridDim.x partials of p in index order
-// and call fin(p, sums).  The slot of problem p's state is descs[p].slot.
-template <int NV, typename Fin>
-__device__ void publish_and_finish(int nprob, const int* s_active, const double* s_part,
-                                   double* partials, unsigned* counters, const Fin& fin) {
-  __shared__ int s_last[kMaxProb];
-  const int G = gridDim.x;
-  for (int p = threadIdx.x; p < nprob; p += blockDim.x) {
-    s_last[p] = 0;
-    if (s_active[p]) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-        partials[((long long)p * NV + v) * G + blockIdx.x] = s_part[p * NV + v];
-      __threadfence();
-      const unsigned t = atomicAdd(&counters[p], 1u);
-      s_last[p] = (t == (unsigned)G - 1u);
-    }
-  }
-  __syncthreads();
-  for (int p = 0; p < nprob; ++p) {
-    if (!s_last[p]) continue;  // shared value: uniform across the block
-    __threadfence();
-    double sums[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-      sums[v] = threadIdx.x < 32 ? warp0_sum_global(partials + ((long long)p * NV + v) * G, G) : 0.0;
-    if (threadIdx.x == 0) {
-      fin(p, sums);
-      counters[p] = 0u;
-    }
-    __syncthreads();
-  }
 }
 
 template <typename T>
@@ -185,38 +92,6 @@ struct FinBeta {
     } else if (S.iter >= S.max_iter) {
       S.done = 1;
       S.status = S.fixed ? EXCMG_OK : EXCMG_ERR_NOT_CONVERGED;
-    }
-  }
-};
-
-struct FinRes {
-  const ResDesc* descs;
-  CGState* st;
-  __device__ void operator()(int p, const double* s) const {
-    const ResDesc& d = descs[p];
-    CGState& S = st[d.slot];
-    const double rr = s[0];
-    // s[1] = ||b||^2 (lift included), s[2] = ||RHS(f)||^2: the two readings of ||f_h||
-    const double bb = !d.want_b ? S.bb : (d.forcing && s[2] > 0.0) ? s[2] : s[1];
-    S.rr = rr;
-    S.rr0 = rr;
-    S.bb = bb;
-    S.alpha = 0.0;
-    S.beta = 0.0;
-    S.pq = 0.0;
-    S.iter = 0;
-    S.first = 1;
-    S.max_iter = d.max_iter;
-    S.fixed = d.fixed;
-    S.status = EXCMG_OK;
-    S.tol2 = d.fixed ? -1.0 : fmax(d.tol_b2 * bb, d.tol_r2 * rr);
-    if (d.hist && d.hist_len > 0) d.hist[0] = rr;
-    S.done = d.fixed ? (d.max_iter <= 0) : (rr <= S.tol2 || d.max_iter <= 0);
-    // no step allowed and the start does not pass the test: the level is unconverged
-    if (!d.fixed && d.max_iter <= 0 && !(rr <= S.tol2)) S.status = EXCMG_ERR_NOT_CONVERGED;
-    if (!isfinite(rr) || !isfinite(bb)) {
-      S.status = EXCMG_ERR_NONFINITE;
-      S.done = 1;
     }
   }
 };
@@ -332,6 +207,169 @@ __device__ __forceinline__ T spmv_tile(const CGDesc<T>& d, long long lt, bool fi
   return tacc;
 }
 
+// One slab of a float64 problem: p_new = r + beta p_old (p = r when first) and q = A p_new on
+// its interior nodes; adds this thread's share of p.q to acc.  p is formed on load (1.3
+// float64 FMA per node, halo included) and stored as integers for the sums; p.q is taken
+// from the integers (2^-56 of the group's largest p), so that no p stays in a register.
+// F64: the sums in float64.  Returns false, in every thread, when a group is not for fixed
+// point (the caller then takes the slab again with F64).  All threads of the block must call.
+// Measured, a whole CG step: 385 x 201 x 121 cells 0.517 ms with the sums in float64 (19
+// float64 instructions per node and step), 0.220 ms here (8; the FP64 pipe 63% busy);
+// 128^3 0.14 ms, 0.061 ms here.
+template <bool F64>
+__device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, bool first, double beta,
+                                       const double* __restrict__ pold, double* __restrict__ pnew, FxSmem& S,
+                                       double& acc_out) {
+  const int nx = d.g.nx, ny = d.g.ny, nz = d.g.nz;
+  const long long sy = d.g.sy, sz = d.g.sz;
+  const FxCols C(c);
+  long long o = C.i + C.j * sy + (c.z0 - 1) * sz;  // own node of the group's first plane
+  const bool own = C.i < nx && C.j < ny;
+  // the rim: boundary nodes (and nodes outside the grid) hold p = 0
+  long long ro[kRimT];
+  bool rim[kRimT];
+#pragma unroll
+  for (int m = 0; m < kRimT; ++m) {
+    rim[m] = C.rim_box[m] >= 0 && C.rim_x[m] > 0 && C.rim_x[m] < nx && C.rim_y[m] > 0 && C.rim_y[m] < ny;
+    ro[m] = C.rim_x[m] + C.rim_y[m] * sy + (c.z0 - 1 + C.rim_z[m]) * sz;
+  }
+  const double* __restrict__ r = d.r;
+  double* __restrict__ qout = d.q + (o + sz);
+  const FxWeights W = d.W;
+  double acc = 0.0;
+  FxMarch M;
+  F64March D;
+  int E1 = 0, scale = kFxMinExp;
+  for (int k0 = c.z0 - 1; k0 <= c.z1; k0 += kFxG) {
+    // planes of the group that hold p: 1 .. nz - 1 of the grid, up to the upper halo plane
+    const int lo = 1 - k0, hi = min(c.z1, nz - 1) - k0;
+    double p[kLoads];
+    {
+      double pv[kLoads];
+      const double* rr[kRimT];
+#pragma unroll
+      for (int m = 0; m < kRimT; ++m) rr[m] = r + ro[m];
+      load_group(p, r + o, own, rr, rim, C, sz, lo, hi, [](const double* a) { return ldv(a); });
+      if (!first) {
+#pragma unroll
+        for (int m = 0; m < kRimT; ++m) rr[m] = pold + ro[m];
+        load_group(pv, pold + o, own, rr, rim, C, sz, lo, hi, [](const double* a) { return ldv(a); });
+#pragma unroll
+        for (int n = 0; n < kLoads; ++n) p[n] = fma(beta, pv[n], p[n]);
+      }
+    }
+    if (own) {
+      double* pn = pnew + o;
+#pragma unroll
+      for (int n = 0; n < kOwn; ++n)
+        if (k0 + n >= c.z0 && k0 + n < c.z1) pn[n * sz] = p[n];
+    }
+    o += kFxG * sz;
+#pragma unroll
+    for (int m = 0; m < kRimT; ++m) ro[m] += kFxG * sz;
+    if (F64) {
+      __syncthreads();  // the box of the group before is read
+      store_box(reinterpret_cast<double*>(S.box), p, C, [](double v) { return v; });
+    } else {
+      warp_mag(p, S.mag[0]);
+      __syncthreads();
+      const int E = block_exp(S.mag[0]);
+      if (E < 0) return false;
+      const int sc = fx_group_scale(E, E1);
+      E1 = E;
+      if (sc != scale) M.rescale(scale - sc);
+      scale = sc;
+      store_box(S.box, p, C, [&](double v) { return fx_from_double<kFxBits>(v, sc); });
+    }
+    const int qL = fx_sum_exp(W.k, scale) - 1;  // A p = -L 2^qL
+    if (!F64 && (qL < -1000 || qL > 800)) return false;
+    __syncthreads();
+    double accg = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < kFxG; ++s) {
+      // this plane completes the sums of the one before
+      const bool out = k0 + s > c.z0 && k0 + s <= c.z1 && own;
+      if (F64)
+        D.plane(reinterpret_cast<const double*>(S.box) + s * kPlane + fx_corner(), d.A, [&](double pc, double qv) {
+          if (out) {
+            *qout = qv;
+            qout += sz;
+            accg = fma(pc, qv, accg);
+          }
+        });
+      else
+        M.plane(S.box + s * kPlane + fx_corner(), W, [&](long long pc, auto lhs2) {
+          if (out) {
+            const double v = (double)lhs2();  // -q 2^-qL
+            *qout = fx_scale_neg(v, qL);
+            qout += sz;
+            accg = fma(-(double)pc, v, accg);
+          }
+        });
+    }
+    // the scales of p and q
+    acc += F64 ? accg : accg * fx_pow2(scale - 1022 - kFxBits) * fx_pow2(qL);
+  }
+  acc_out += acc;
+  return true;
+}
+
+__device__ __forceinline__ double spmv_slab_any(const CGDesc<double>& d, long long lt, bool first, double beta,
+                                                const double* pold, double* pnew, FxSmem& S) {
+  const FxSlab c = fx_slab(d.g, d.t, lt);
+  double acc = 0.0;
+  if (d.float64 || !spmv_slab<false>(d, c, first, beta, pold, pnew, S, acc))
+    spmv_slab<true>(d, c, first, beta, pold, pnew, S, acc);
+  return acc;
+}
+
+// The update x += alpha p, r -= alpha q of one float64 slab (a column per thread); returns
+// this thread's share of r.r.
+__device__ __forceinline__ double update_slab(const CGDesc<double>& d, long long lt, double alpha,
+                                              const double* __restrict__ pn) {
+  const FxSlab c = fx_slab(d.g, d.t, lt);
+  const int i = c.x0 + (threadIdx.x & 31), j = c.y0 + (threadIdx.x >> 5);
+  if (i >= d.g.nx || j >= d.g.ny) return 0.0;
+  double* __restrict__ x = d.x;
+  double* __restrict__ r = d.r;
+  double acc = 0.0;
+  long long o = i + j * d.g.sy + c.z0 * d.g.sz;
+#pragma unroll 4
+  for (int k = c.z0; k < c.z1; ++k, o += d.g.sz) {
+    const double xv = fma(alpha, ldv(pn + o), ldv(x + o));
+    const double rv = fma(-alpha, ldv(d.q + o), ldv(r + o));
+    x[o] = xv;
+    r[o] = rv;
+    acc = fma(rv, rv, acc);
+  }
+  return acc;
+}
+
+// p_a, p_b and q of a float64 problem are zero on its boundary nodes (which the stencil
+// tiles neither read nor write, and the flat update runs over): zeroed by the blocks of
+// its team at the first step.
+__device__ __forceinline__ void zero_faces(const CGDesc<double>& d, int bl, int G) {
+  const Grid3 g = d.g;
+  const long long nz2 = 2 * (long long)(g.nx + 1) * (g.ny + 1), ny2 = 2 * (long long)(g.nx + 1) * (g.nz + 1),
+                  nx2 = 2 * (long long)(g.ny + 1) * (g.nz + 1);
+  for (long long t = (long long)bl * kThreads + threadIdx.x; t < nz2 + ny2 + nx2; t += (long long)G * kThreads) {
+    long long o;
+    if (t < nz2) {
+      const long long u = t >> 1;
+      o = u + (t & 1) * g.nz * g.sz;
+    } else if (t < nz2 + ny2) {
+      const long long u = (t - nz2) >> 1;
+      o = u % (g.nx + 1) + (u / (g.nx + 1)) * g.sz + ((t - nz2) & 1) * g.ny * g.sy;
+    } else {
+      const long long u = (t - nz2 - ny2) >> 1;
+      o = (u % (g.ny + 1)) * g.sy + (u / (g.ny + 1)) * g.sz + ((t - nz2 - ny2) & 1) * g.nx;
+    }
+    d.pa[o] = 0.0;
+    d.pb[o] = 0.0;
+    d.q[o] = 0.0;
+  }
+}
+
 // One update tile: x += alpha p, r -= alpha q on the tile's nodes; returns this thread's
 // share of r.r.
 template <typename T>
@@ -381,6 +419,11 @@ struct Vec<double> {
 __device__ __forceinline__ float4 ldv4(const float4* p) { return __ldcg(p); }
 __device__ __forceinline__ double2 ldv4(const double2* p) { return __ldcg(p); }
 
+// sigma r: the right-hand side's scale of the float32 engine's first step (float64 has none,
+// and no float64 multiply to spare on it).
+__device__ __forceinline__ float scaled(float sigma, float r) { return sigma * r; }
+__device__ __forceinline__ double scaled(double, double r) { return r; }
+
 // kRev: the blocks walk the chunks from the end of the array back to its start.  The
 // stencil phase before it walks its tiles forward, so the chunks this phase takes first
 // are the ones the stencil phase wrote last, still in L2 (and the chunks it takes last
@@ -404,7 +447,7 @@ __device__ __forceinline__ double update_flat(const CGDesc<T>& d, int bl, int G,
   if (bl == 0 && threadIdx.x < lead && threadIdx.x < n) {
     const long long o = threadIdx.x;
     const T xv = fmaT(alpha, ldv(pn + o), ldv(x + o));
-    const T rv = fmaT(-alpha, ldv(q + o), sigma * ldv(r + o));
+    const T rv = fmaT(-alpha, ldv(q + o), scaled(sigma, ldv(r + o)));
     x[o] = xv;
     r[o] = rv;
     acc += (double)(rv * rv);
@@ -429,7 +472,7 @@ __device__ __forceinline__ double update_flat(const CGDesc<T>& d, int bl, int G,
 #pragma unroll
         for (int e = 0; e < V; ++e) {
           xe[e] = fmaT(alpha, pe[e], xe[e]);
-          re[e] = fmaT(-alpha, qe[e], sigma * re[e]);
+          re[e] = fmaT(-alpha, qe[e], scaled(sigma, re[e]));
           tacc = fmaT(re[e], re[e], tacc);
         }
         *reinterpret_cast<VT*>(x + o) = xv;
@@ -438,7 +481,7 @@ __device__ __forceinline__ double update_flat(const CGDesc<T>& d, int bl, int G,
     } else {
       for (long long o = c0 + threadIdx.x; o < c1; o += kThreads) {
         const T xv = fmaT(alpha, ldv(pn + o), ldv(x + o));
-        const T rv = fmaT(-alpha, ldv(q + o), sigma * ldv(r + o));
+        const T rv = fmaT(-alpha, ldv(q + o), scaled(sigma, ldv(r + o)));
         x[o] = xv;
         r[o] = rv;
         tacc = fmaT(rv, rv, tacc);
@@ -475,18 +518,18 @@ __device__ __forceinline__ double update_flat(const CGDesc<T>& d, int bl, int G,
 #endif
 constexpr int kRT = EXCMG_TMA_ROWS;        // y-rows per thread (consecutive)
 constexpr int kTileY = kTY * kRT;          // y-rows of a tile of this engine
-constexpr int kBoxX = kTX + 8;
-constexpr int kBoxY = kTileY + 2;
+constexpr int kTmaBoxX = kTX + 8;
+constexpr int kTmaBoxY = kTileY + 2;
 constexpr int kStages = EXCMG_TMA_STAGES;
 constexpr int kZs = EXCMG_TMA_PLANES;  // planes per copy (the box's z extent)
-constexpr unsigned kBoxBytes = kBoxX * kBoxY * kZs * sizeof(float);
+constexpr unsigned kBoxBytes = kTmaBoxX * kTmaBoxY * kZs * sizeof(float);
 // a box's shared-memory slot, rounded up to 128 bytes so that every copy destination is
 // 128-byte aligned
 constexpr int kBoxSlot = ((kBoxBytes + 127) / 128) * 128 / sizeof(float);
 constexpr int kWarps = kThreads / 32;
 
 struct TmaRing {
-  float stage[kStages][2][kBoxSlot];      // r and p_old of kZs planes per stage (kZs x kBoxY x kBoxX)
+  float stage[kStages][2][kBoxSlot];      // r and p_old of kZs planes per stage (kZs x kTmaBoxY x kTmaBoxX)
   unsigned long long full[kStages];       // the stage's copies have landed
   unsigned long long empty[kStages];      // every warp is done reading the stage
   int abort;                              // a wait ran out: the block leaves the step
@@ -626,7 +669,7 @@ __device__ double spmv_tiles_tma(const CGDesc<float>& d, int bl, int G, bool fir
   bool stop = false;
   // this thread's neighbourhood in a plane of a stage: rows ty kRT .. ty kRT + kRT + 1,
   // columns tx + 3 .. tx + 5 (stage column c holds x = x0 - 4 + c, row r y = y0 - 1 + r)
-  const int base = ty * kRT * kBoxX + tx + 3;
+  const int base = ty * kRT * kTmaBoxX + tx + 3;
   for (long long t = bl; t < T && !stop; t += G) {
     const TileXYZ c = tma_tile_coords(g, tl, t);
     const int i = c.x0 + tx, j0 = c.y0 + ty * kRT;
@@ -646,14 +689,14 @@ __device__ double spmv_tiles_tma(const CGDesc<float>& d, int bl, int G, bool fir
       const int np = min(kZs, c.z1 + 1 - k0);  // planes of this box that the tile uses
 #pragma unroll 1
       for (int pz = 0; pz < np; ++pz) {
-        const float* rs = &R.stage[slot][0][pz * kBoxY * kBoxX + base];
-        const float* ps = &R.stage[slot][1][pz * kBoxY * kBoxX + base];
+        const float* rs = &R.stage[slot][0][pz * kTmaBoxY * kTmaBoxX + base];
+        const float* ps = &R.stage[slot][1][pz * kTmaBoxY * kTmaBoxX + base];
         float v[kRT + 2][3];
 #pragma unroll
         for (int a = 0; a < kRT + 2; ++a)
 #pragma unroll
           for (int b = 0; b < 3; ++b)
-            v[a][b] = first ? sigma * rs[a * kBoxX + b] : fmaf(beta, ps[a * kBoxX + b], rs[a * kBoxX + b]);
+            v[a][b] = first ? sigma * rs[a * kTmaBoxX + b] : fmaf(beta, ps[a * kTmaBoxX + b], rs[a * kTmaBoxX + b]);
         const int kc = k0 + pz - 1;
         const bool emit = kc >= c.z0 && ownx;
         const bool zin = kc > 0 && kc < g.nz;
@@ -723,10 +766,12 @@ __device__ double spmv_tiles_tma(const CGDesc<float>& d, int bl, int G, bool fir
 // K1: p_new = r + beta p_old, q = A p_new, sum p.q
 // ---------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kFxBlocks : 1)
     k_dir_spmv_dot(int nprob, const CGDesc<T>* __restrict__ descs, long long total_tiles,
                    CGState* st, double* partials, unsigned* counters) {
-  __shared__ T sp[2][kTY + 2][kTX + 2];
+  constexpr bool kFx = sizeof(T) == 8;  // float64: fixed-point slabs
+  __shared__ __align__(16) unsigned char fx_smem[kFx ? sizeof(FxSmem) : 16];
+  __shared__ T sp[kFx ? 1 : 2][kFx ? 1 : kTY + 2][kFx ? 1 : kTX + 2];
   __shared__ int s_active[kMaxProb];
   __shared__ double s_part[kMaxProb];
   for (int p = threadIdx.x; p < nprob; p += blockDim.x) {
@@ -750,8 +795,12 @@ __global__ void __launch_bounds__(kThreads)
     const CGDesc<T>& d = descs[p];
     const CGState& S = st[d.slot];
     const int it = S.iter;
-    acc += (double)spmv_tile<T>(d, t - d.tile_begin, S.first != 0, (T)S.beta,
-                                (it & 1) ? d.pb : d.pa, (it & 1) ? d.pa : d.pb, sp, buf);
+    const T* pold = (it & 1) ? d.pb : d.pa;
+    T* pnew = (it & 1) ? d.pa : d.pb;
+    if constexpr (kFx)
+      acc += spmv_slab_any(d, t - d.tile_begin, S.first != 0, S.beta, pold, pnew, *reinterpret_cast<FxSmem*>(fx_smem));
+    else
+      acc += (double)spmv_tile<T>(d, t - d.tile_begin, S.first != 0, (T)S.beta, pold, pnew, sp, buf);
   }
   if (cur >= 0) {
     const double s = block_sum(acc);
@@ -791,7 +840,11 @@ __global__ void __launch_bounds__(kThreads)
     const CGDesc<T>& d = descs[p];
     const CGState& S = st[d.slot];
     const int it = S.iter;
-    acc += (double)update_tile<T>(d, t - d.tile_begin, (T)S.alpha, (it & 1) ? d.pa : d.pb);
+    const T* pn = (it & 1) ? d.pa : d.pb;
+    if constexpr (sizeof(T) == 8)
+      acc += update_slab(d, t - d.tile_begin, S.alpha, pn);
+    else
+      acc += (double)update_tile<T>(d, t - d.tile_begin, (T)S.alpha, pn);
   }
   if (cur >= 0) {
     const double s = block_sum(acc);
@@ -869,7 +922,7 @@ __device__ double sum_partials_all(const double* part, int n) {
 template <typename T, bool kTma>
 __device__ bool cg_team(const CGDesc<T>& d, int p, int bl, CGState* st, double* partials,
                         unsigned* bars, T (*sp)[kTY + 2][kTX + 2], double& s_scalar, int& buf,
-                        TmaRing* R, RingPhases& phases, unsigned long long wait_ns) {
+                        TmaRing* R, RingPhases& phases, FxSmem* fx, unsigned long long wait_ns) {
   const int G = d.blk_count;
   CGState* S = st + d.slot;
   if (S->done) return false;  // same value in every block of this team
@@ -916,6 +969,9 @@ __device__ bool cg_team(const CGDesc<T>& d, int p, int bl, CGState* st, double* 
         if (threadIdx.x == 0) atomicExch(err, 1);
         break;
       }
+    } else if constexpr (sizeof(T) == 8) {
+      if (first) zero_faces(d, bl, G);
+      for (long long t = bl; t < total_tiles; t += G) acc += spmv_slab_any(d, t, first, beta, pold, pnew, *fx);
     } else {
       for (long long t = bl; t < total_tiles; t += G)
         acc += (double)spmv_tile<T>(d, t, first, (T)beta, pold, pnew, sp, buf);
@@ -944,7 +1000,10 @@ __device__ bool cg_team(const CGDesc<T>& d, int p, int bl, CGState* st, double* 
       acc = update_flat<T, kTma>(d, bl, G, (T)alpha, pnew, sigma);
     } else {
       for (long long t = bl; t < total_tiles; t += G)
-        acc += (double)update_tile<T>(d, t, (T)alpha, pnew, sigma);
+        if constexpr (sizeof(T) == 8)
+          acc += update_slab(d, t, alpha, pnew);
+        else
+          acc += (double)update_tile<T>(d, t, (T)alpha, pnew, sigma);
     }
     bs = block_sum(acc);
     if (threadIdx.x == 0) partB[bl] = bs;
@@ -1000,16 +1059,19 @@ __device__ bool cg_team(const CGDesc<T>& d, int p, int bl, CGState* st, double* 
 #define EXCMG_PERSIST_TMA_MIN_BLOCKS 2
 #endif
 template <typename T, bool kTma>
-__global__ void __launch_bounds__(kThreads, kTma ? EXCMG_PERSIST_TMA_MIN_BLOCKS : EXCMG_PERSIST_MIN_BLOCKS)
+__global__ void __launch_bounds__(kThreads, kTma            ? EXCMG_PERSIST_TMA_MIN_BLOCKS
+                                            : sizeof(T) == 8 ? kFxBlocks
+                                                             : EXCMG_PERSIST_MIN_BLOCKS)
     k_cg_persistent(int nprob, const CGDesc<T>* __restrict__ descs, CGState* st,
                     double* partials, unsigned* bars, unsigned long long wait_ns) {
   __shared__ double s_scalar;
   __shared__ int s_slot;
   T(*sp)[kTY + 2][kTX + 2] = nullptr;
   TmaRing* R = nullptr;
+  FxSmem* fx = nullptr;
   if constexpr (kTma) {
-    extern __shared__ __align__(128) unsigned char dyn_smem[];  // sizeof(TmaRing) bytes
-    TmaRing& ring = *reinterpret_cast<TmaRing*>(dyn_smem);
+    extern __shared__ __align__(128) unsigned char dyn_persist[];  // sizeof(TmaRing) bytes
+    TmaRing& ring = *reinterpret_cast<TmaRing*>(dyn_persist);
     R = &ring;
     if (threadIdx.x == 0) {
       for (int k = 0; k < kStages; ++k) {
@@ -1029,6 +1091,9 @@ __global__ void __launch_bounds__(kThreads, kTma ? EXCMG_PERSIST_TMA_MIN_BLOCKS 
         asm volatile("prefetch.tensormap [%0];" ::"l"(&m->pb) : "memory");
       }
     }
+  } else if constexpr (sizeof(T) == 8) {
+    __shared__ FxSmem slab;
+    fx = &slab;
   } else {
     __shared__ T stage[2][kTY + 2][kTX + 2];
     sp = stage;
@@ -1048,249 +1113,12 @@ __global__ void __launch_bounds__(kThreads, kTma ? EXCMG_PERSIST_TMA_MIN_BLOCKS 
     while (p < nprob && !(slot >= descs[p].blk_begin && slot < descs[p].blk_begin + descs[p].blk_count)) ++p;
     if (p >= nprob) return;  // unreachable: every slot below total_slots has a team
     if (cg_team<T, kTma>(descs[p], p, slot - descs[p].blk_begin, st, partials, bars, sp, s_scalar,
-                         buf, R, phases, wait_ns))
+                         buf, R, phases, fx, wait_ns))
       return;  // the copy ring was abandoned: this block takes no further work
   }
 }
 
 
-
-// ---------------------------------------------------------------------------------
-// K3: r = LHS(u) - RHS(f) = b - A u_I (float64), sums r.r and b.b, CG state init
-// ---------------------------------------------------------------------------------
-#ifndef EXCMG_RES_MINB
-#define EXCMG_RES_MINB 3  // one row per thread: 24 warps per SM, measured faster than 16
-#endif
-#ifndef EXCMG_RES_MINB_WIDE
-// four rows per thread share the W + E sums of their neighbourhood (2 row sums per node
-// instead of 3) and need 128 registers: 16 warps per SM (at 80 registers they spill)
-#define EXCMG_RES_MINB_WIDE 2
-#endif
-
-// A residual tile: kTX columns along x (one warp) x kTY * R rows along y (each thread
-// takes R adjacent rows) x tz planes, covering nodes 0 .. n per direction.
-// (Tiles of the interior nodes 1 .. n, with the index-0 boundary nodes written by their
-// neighbours, hold no padding for power-of-two grids but measured 40% slower.)
-template <int R>
-__device__ __forceinline__ TileXYZ res_tile_coords(const Grid3& g, const Tiling& tl, long long lt) {
-  TileXYZ c;
-  const int bx = (int)(lt % tl.ntx);
-  const long long r = lt / tl.ntx;
-  const int by = (int)(r % tl.nty);
-  const int bz = (int)(r / tl.nty);
-  c.x0 = bx * kTX;
-  c.y0 = by * kTY * R;
-  c.z0 = bz * tl.tz;
-  c.z1 = min(c.z0 + tl.tz, g.nz + 1);
-  return c;
-}
-
-// The Dirichlet lift of node (i, j, k) next to an x or y boundary face: the part of its
-// 19-point sum over boundary nodes, grouped as the sum itself is (in-plane part of
-// plane k, plus the out-of-plane parts of planes k - 1 and k + 1, which are whole
-// boundary planes when k - 1 = 0 or k + 1 = nz).  Direct loads: about 3% of the nodes.
-__device__ double perim_lift(const double* __restrict__ u, const Grid3& g, const Coef& A, int i,
-                             int j, int k) {
-  const bool bxm = (i - 1 == 0), bxp = (i + 1 == g.nx), bym = (j - 1 == 0), byp = (j + 1 == g.ny);
-  auto at = [&](int x, int y, int z) { return __ldg(u + x + (long long)y * g.sy + (long long)z * g.sz); };
-  // out-of-plane part of plane kk: whole plane if it is a boundary plane, else its
-  // boundary columns
-  auto lt = [&](int kk) -> double {
-    if (kk == 0 || kk == g.nz) {
-      const double SX = at(i - 1, j, kk) + at(i + 1, j, kk), SY = at(i, j - 1, kk) + at(i, j + 1, kk);
-      return fma(A.fz, at(i, j, kk), fma(A.exz, SX, A.eyz * SY));
-    }
-    const double mSX = (bxm ? at(i - 1, j, kk) : 0.0) + (bxp ? at(i + 1, j, kk) : 0.0);
-    const double mSY = (bym ? at(i, j - 1, kk) : 0.0) + (byp ? at(i, j + 1, kk) : 0.0);
-    return fma(A.exz, mSX, A.eyz * mSY);
-  };
-  const double mSX = (bxm ? at(i - 1, j, k) : 0.0) + (bxp ? at(i + 1, j, k) : 0.0);
-  const double mSY = (bym ? at(i, j - 1, k) : 0.0) + (byp ? at(i, j + 1, k) : 0.0);
-  const double mEXY = ((bxm || bym) ? at(i - 1, j - 1, k) : 0.0) + ((bxp || bym) ? at(i + 1, j - 1, k) : 0.0) +
-                      ((bxm || byp) ? at(i - 1, j + 1, k) : 0.0) + ((bxp || byp) ? at(i + 1, j + 1, k) : 0.0);
-  const double LC = fma(A.fx, mSX, fma(A.fy, mSY, A.exy * mEXY));
-  return (LC + lt(k - 1)) + lt(k + 1);
-}
-
-// Twice the right-hand side of eq. (compact) at interior node (i, j, k): 6 f_c + the 6
-// face values of f (the face values are re-read through L1 by the neighbouring threads),
-// or the value an earlier pass kept, or -2 b when b is given directly.  o is the node's
-// offset.
-__device__ __forceinline__ double res_rhs2(const ResDesc& d, int i, int j, int k, long long o) {
-  if (d.rhs2 != nullptr) return d.rhs2[o];
-  if (d.src != nullptr) return -2.0 * d.src[o];
-  const View& F = d.f;
-  return fma(6.0, F.at(i, j, k), ((F.at(i - 1, j, k) + F.at(i + 1, j, k)) +
-                                  (F.at(i, j - 1, k) + F.at(i, j + 1, k)) +
-                                  (F.at(i, j, k - 1) + F.at(i, j, k + 1))));
-}
-
-// The residual's block sums of one problem (r.r, ||b||^2 with the lift, ||RHS(f)||^2)
-// added to its three partials in shared memory.  Called at problem switches only; kept
-// out of line so that it adds no registers to the plane loop.
-__device__ __noinline__ void residual_flush(double acc_r, double acc_b, double acc_b4, double* part) {
-  const double s1 = block_sum(acc_r);
-  const double s2 = block_sum(fma(0.25, acc_b4, acc_b));
-  const double s3 = block_sum(0.25 * acc_b4);
-  if (threadIdx.x == 0) {
-    part[0] += s1;
-    part[1] += s2;
-    part[2] += s3;
-  }
-}
-
-// Each thread marches its R rows of one x-column through the tile's planes.  Per
-// plane it loads the (R + 2) x 3 neighbourhood (through the read-only cache:
-// neighbouring threads share the lines; no staging, no block barrier) and forms, per row,
-// the in-plane part C = c0 P + fx S_x + fy S_y + exy E_xy and the out-of-plane part
-// T = fz P + exz S_x + eyz S_y of the 19-point sum, with S_x = W + E computed once per
-// loaded row and shared by the rows above and below (E_xy of row j = S_x(j-1) + S_x(j+1),
-// the same grouping as (SW + SE) + (NW + NE)); the sum at plane k is C_k + T_{k-1} +
-// T_{k+1}.  The first and last plane of a tile contribute T only.  b (for ||b||) is
-// -RHS away from the boundary; next to a z-boundary plane its lift is that plane's T;
-// next to a y boundary face it is formed by perim_lift (the whole warp is such a row).
-// Next to an x boundary face only one lane of the warp is such a node: those nodes are
-// left out of the plane loop and formed after it, one lane per plane, so a warp issues
-// the lift once for up to 32 planes instead of once per plane for one lane.
-template <typename TR, int R>
-__global__ void __launch_bounds__(kThreads, R > 1 ? EXCMG_RES_MINB_WIDE : EXCMG_RES_MINB)
-    k_residual(int nprob, const ResDesc* __restrict__ descs, long long total_tiles,
-               CGState* st, double* partials, unsigned* counters) {
-  static_assert(kTX == 32, "one warp per x-run of a residual tile row");
-  __shared__ int s_active[kMaxProb];
-  __shared__ double s_part[3 * kMaxProb];
-  for (int p = threadIdx.x; p < nprob; p += blockDim.x) {
-    s_active[p] = 1;
-    s_part[3 * p] = 0.0;
-    s_part[3 * p + 1] = 0.0;
-    s_part[3 * p + 2] = 0.0;
-  }
-  __syncthreads();
-  const int tx = threadIdx.x % kTX, ty = threadIdx.x / kTX;
-  int cur = -1, p = 0;
-  // acc_b4 sums (2 RHS)^2 over every interior node: ||RHS(f)||^2 = acc_b4 / 4 is the
-  // forcing reading of ||f_h||.  b = -RHS - lift, and the lift is nonzero only next to
-  // the boundary, so ||b||^2 = acc_b4 / 4 + acc_b with acc_b summing b^2 - RHS^2 =
-  // lift (lift + 2 RHS) over those nodes (the lift reading).
-  double acc_r = 0.0, acc_b = 0.0, acc_b4 = 0.0;
-  auto flush = [&](int q) { residual_flush(acc_r, acc_b, acc_b4, s_part + 3 * q); };
-  for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-    p = find_problem(descs, nprob, t, p);
-    if (p != cur) {
-      if (cur >= 0) flush(cur);
-      acc_r = acc_b = acc_b4 = 0.0;
-      cur = p;
-    }
-    const ResDesc& d = descs[p];
-    const Grid3 g = d.g;
-    const double* __restrict__ u = d.u;
-    TR* __restrict__ rout = reinterpret_cast<TR*>(d.r);
-    // output strides: the padded float32 layout, or the grid's own for float64
-    const long long osy = sizeof(TR) == 4 ? d.osy : g.sy, osz = sizeof(TR) == 4 ? d.osz : g.sz;
-    const TileXYZ c = res_tile_coords<R>(g, d.t, t - d.tile_begin);
-    const int i = c.x0 + tx, jb = c.y0 + R * ty;  // rows jb .. jb + R - 1
-    if (c.x0 >= g.nx || c.y0 >= g.ny || c.z0 >= g.nz) {
-      // a tile of boundary nodes only (the last column, row or plane of the grid and the
-      // padding beyond it): r = 0, no arithmetic
-      for (int kc = c.z0; kc < c.z1; ++kc)
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-          const int j = jb + q;
-          if (i < osy && j <= g.ny) rout[i + j * osy + (long long)kc * osz] = (TR)0.0;
-        }
-      continue;
-    }
-    const bool colx = (i > 0) && (i < g.nx);
-    const bool want_b = d.want_b != 0;
-    const Coef A = d.A;
-    double Cm1[R], Tm1[R], Tm2[R];
-#pragma unroll
-    for (int q = 0; q < R; ++q) Cm1[q] = Tm1[q] = Tm2[q] = 0.0;
-    for (int kk = c.z0 - 1; kk <= c.z1; ++kk) {
-      const bool need_c = (kk >= c.z0) && (kk < c.z1);  // C of the tile's own planes only
-      // the neighbourhood: rows jb - 1 .. jb + R (index y = row - jb + 1), columns i - 1,
-      // i, i + 1; zero outside the grid
-      double Pv[R + 2], SXv[R + 2];
-      const bool kin = kk >= 0 && kk <= g.nz;
-      const double* pl = u + (long long)kk * g.sz;
-#pragma unroll
-      for (int y = 0; y < R + 2; ++y) {
-        const int gj = jb - 1 + y;
-        const bool rin = kin && gj >= 0 && gj <= g.ny;
-        const double* row = pl + (long long)gj * g.sy;
-        const double W = (rin && i - 1 >= 0 && i - 1 <= g.nx) ? __ldg(row + i - 1) : 0.0;
-        const double E = (rin && i + 1 <= g.nx) ? __ldg(row + i + 1) : 0.0;
-        Pv[y] = (rin && i <= g.nx) ? __ldg(row + i) : 0.0;
-        SXv[y] = W + E;
-      }
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const int y = q + 1, j = jb + q;
-        const double SX = SXv[y], SY = Pv[y - 1] + Pv[y + 1], P = Pv[y];
-        double Ck = 0.0;
-        if (need_c) Ck = fma(A.c0, P, fma(A.fx, SX, fma(A.fy, SY, A.exy * (SXv[y - 1] + SXv[y + 1]))));
-        const double Tk = fma(A.fz, P, fma(A.exz, SX, A.eyz * SY));
-        const int kc = kk - 1;
-        if (kc >= c.z0 && i <= g.nx && j <= g.ny) {
-          const long long o = i + j * g.sy + (long long)kc * g.sz;
-          double rv = 0.0;
-          if (colx && j > 0 && j < g.ny && kc > 0 && kc < g.nz) {
-            // twice the right-hand side (kept as it is for the later passes); the factor
-            // 1/2 is applied inside the fused multiply-add below, exactly
-            const double rhs2 = res_rhs2(d, i, j, kc, o);
-            if (d.rhs_out) d.rhs_out[o] = rhs2;
-            // LHS(u) - RHS = -(A-stencil of u over all 19 nodes) - RHS
-            rv = fma(-0.5, rhs2, -((Cm1[q] + Tm2[q]) + Tk));
-            acc_r = fma(rv, rv, acc_r);
-            if (want_b) {
-              acc_b4 = fma(rhs2, rhs2, acc_b4);
-              const bool yface = (j == 1 || j == g.ny - 1), xface = (i == 1 || i == g.nx - 1);
-              if ((yface || !xface) && (yface || kc < 2 || kc > g.nz - 2)) {
-                const double lift = yface ? perim_lift(u, g, A, i, j, kc)
-                                          : (kc == 1 ? Tm2[q] : 0.0) + (kc == g.nz - 1 ? Tk : 0.0);
-                acc_b = fma(lift, lift + rhs2, acc_b);
-              }  // next to an x face only: after the plane loop; elsewhere b = -RHS
-            }
-          }
-          rout[i + j * osy + (long long)kc * osz] = (TR)rv;
-        } else if (sizeof(TR) == 4 && kc >= c.z0 && i > g.nx && i < osy && j <= g.ny) {
-          rout[i + j * osy + (long long)kc * osz] = (TR)0.0;  // padding column
-        }
-        Tm2[q] = Tm1[q];
-        Tm1[q] = Tk;
-        Cm1[q] = Ck;
-      }
-    }
-    if (want_b) {
-      // b of the tile's nodes next to an x face and no y face (columns 1 and nx - 1, rows
-      // 2 .. ny - 2): the warp of such a row takes them one lane per plane.  A warp is one
-      // x-run of 32 columns (kTX = 32), so its columns are c.x0 .. c.x0 + 31 in every row.
-      const int lane = threadIdx.x & 31;
-      const int k_lo = max(c.z0, 1), k_hi = min(c.z1, g.nz);  // interior planes of the tile
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const int j = jb + q;
-        if (j < 2 || j > g.ny - 2) continue;
-        for (int side = 0; side < 2; ++side) {
-          const int xi = side == 0 ? 1 : g.nx - 1;
-          if (side == 1 && xi == 1) break;  // nx = 2: a single interior column
-          if (xi < c.x0 || xi >= c.x0 + kTX) continue;
-          for (int k0 = k_lo; k0 < k_hi; k0 += 32) {
-            const int kc = k0 + lane;
-            if (kc < k_hi) {
-              const long long o = xi + j * g.sy + (long long)kc * g.sz;
-              const double lift = perim_lift(u, g, A, xi, j, kc);
-              acc_b = fma(lift, lift + res_rhs2(d, xi, j, kc, o), acc_b);
-            }
-          }
-        }
-      }
-    }
-  }
-  if (cur >= 0) flush(cur);
-  __syncthreads();
-  publish_and_finish<3>(nprob, s_active, s_part, partials, counters, FinRes{descs, st});
-}
 
 // MIXED refinement: u += e / scale (the float32 correction of the scaled system), then
 // e = 0 for the next inner solve.  e has the padded float32 layout, u the unpadded
@@ -1379,29 +1207,21 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 int g_max_grid = 0;
-int g_coop_grid[2] = {0, 0};  // co-resident blocks of k_cg_persistent<double>, <float>
-int g_coop_grid_tma = 0;      // the same for the float32 tensor-copy engine
 
 }  // namespace
 
-// Dynamic shared memory of a k_cg_persistent launch (the tensor-copy ring).
-template <bool kTma>
-size_t persistent_smem() {
-  return kTma ? sizeof(TmaRing) : 0;
-}
-
+// Co-resident blocks of k_cg_persistent, -1 without cooperative launches.
 template <typename T, bool kTma>
-int coop_blocks(int& cached) {
+int coop_blocks() {
+  static int cached = 0;
   if (cached == 0) {
     int dev = 0, sms = 0, occ = 0, coop = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (kTma)
-      cudaFuncSetAttribute(k_cg_persistent<T, kTma>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)persistent_smem<kTma>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_persistent<T, kTma>, kThreads,
-                                                  persistent_smem<kTma>());
+    const size_t smem = kTma ? sizeof(TmaRing) : 0;
+    if (kTma) cudaFuncSetAttribute(k_cg_persistent<T, kTma>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_persistent<T, kTma>, kThreads, smem);
     cached = (coop && sms > 0 && occ > 0) ? std::min(sms * occ, kMaxGrid) : -1;
   }
   return cached;
@@ -1409,12 +1229,12 @@ int coop_blocks(int& cached) {
 
 template <typename T>
 int persistent_cg_blocks() {
-  return coop_blocks<T, false>(g_coop_grid[sizeof(T) == 8 ? 0 : 1]);
+  return coop_blocks<T, false>();
 }
 template int persistent_cg_blocks<double>();
 template int persistent_cg_blocks<float>();
 
-int persistent_cg_blocks_tma() { return coop_blocks<float, true>(g_coop_grid_tma); }
+int persistent_cg_blocks_tma() { return coop_blocks<float, true>(); }
 
 template <typename T>
 cudaError_t launch_cg_persistent(int nprob, const CGDesc<T>* descs, int grid, CGState* st,
@@ -1427,7 +1247,7 @@ cudaError_t launch_cg_persistent(int nprob, const CGDesc<T>* descs, int grid, CG
   if constexpr (sizeof(T) == 4) {
     if (tma) {
       fn = (const void*)k_cg_persistent<float, true>;
-      smem = persistent_smem<true>();
+      smem = sizeof(TmaRing);
     }
   }
   return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kThreads), args, smem, s);
@@ -1481,7 +1301,7 @@ bool encode_plane_map(CUtensorMap* m, float* base, const Grid3& g32) {
   // x extent nx + 1: the padding columns are outside the map and read as zeros
   const cuuint64_t dims[3] = {(cuuint64_t)g32.nx + 1, (cuuint64_t)g32.ny + 1, (cuuint64_t)g32.nz + 1};
   const cuuint64_t strides[2] = {(cuuint64_t)g32.sy * sizeof(float), (cuuint64_t)g32.sz * sizeof(float)};
-  const cuuint32_t box[3] = {(cuuint32_t)kBoxX, (cuuint32_t)kBoxY, (cuuint32_t)kZs};
+  const cuuint32_t box[3] = {(cuuint32_t)kTmaBoxX, (cuuint32_t)kTmaBoxY, (cuuint32_t)kZs};
   const cuuint32_t estr[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1503,28 +1323,6 @@ int persistent_grid(long long total_tiles) {
   return g < 1 ? 1 : (int)g;
 }
 
-static int g_res_grid[2] = {0, 0};
-
-int residual_grid(long long total_tiles, int rows) {
-  const int w = rows > 1 ? 1 : 0;
-  if (g_res_grid[w] == 0) {
-    int dev = 0, sms = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (w)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_residual<double, kResRowsWide>, kThreads, 0);
-    else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_residual<double, 1>, kThreads, 0);
-    if (sms <= 0) sms = 1;
-    if (occ <= 0) occ = 1;
-    g_res_grid[w] = sms * occ;
-    // the residual publishes 3 partials per block into room for 2 x kMaxGrid
-    if (g_res_grid[w] > 2 * kMaxGrid / 3) g_res_grid[w] = 2 * kMaxGrid / 3;
-  }
-  long long g = total_tiles < g_res_grid[w] ? total_tiles : g_res_grid[w];
-  return g < 1 ? 1 : (int)g;
-}
-
 template <typename T>
 cudaError_t launch_cg_step(int nprob, const CGDesc<T>* descs, long long total_tiles, int grid,
                            CGState* st, double* partials, unsigned* counters, cudaStream_t s,
@@ -1543,25 +1341,11 @@ template cudaError_t launch_cg_step<float>(int, const CGDesc<float>*, long long,
                                            double*, unsigned*, cudaStream_t, cudaEvent_t,
                                            cudaEvent_t, cudaEvent_t);
 
-cudaError_t launch_residual(bool out_float, int nprob, const ResDesc* descs, long long total_tiles,
-                            int grid, CGState* st, double* partials, unsigned* counters,
-                            cudaStream_t s, int rows) {
-  if (rows != 1 && rows != kResRowsWide) return cudaErrorInvalidValue;
-  if (out_float && rows > 1)
-    k_residual<float, kResRowsWide><<<grid, kThreads, 0, s>>>(nprob, descs, total_tiles, st, partials, counters);
-  else if (out_float)
-    k_residual<float, 1><<<grid, kThreads, 0, s>>>(nprob, descs, total_tiles, st, partials, counters);
-  else if (rows > 1)
-    k_residual<double, kResRowsWide><<<grid, kThreads, 0, s>>>(nprob, descs, total_tiles, st, partials, counters);
-  else
-    k_residual<double, 1><<<grid, kThreads, 0, s>>>(nprob, descs, total_tiles, st, partials, counters);
-  return cudaGetLastError();
-}
-
-// Zeros of p_a, p_b and q on the far boundary faces of a padded float32 grid: the
+// Zeros of p_a, p_b, q and r on the far boundary faces of a padded float32 grid: the
 // columns nx .. sy - 1 of every row, the row ny and the plane nz.  The tensor-copy CG
-// engine never writes these nodes (its tiles end at n - 1) and reads them as halo.
-__global__ void k_zero_far_faces(Grid3 g, float* a, float* b, float* c) {
+// engine never writes these nodes (its tiles end at n - 1) and reads them as halo; the
+// residual writes no padding columns.
+__global__ void k_zero_far_faces(Grid3 g, float* a, float* b, float* c, float* r) {
   const long long rows = (long long)(g.ny + 1) * (g.nz + 1);
   const int cx = g.sy - g.nx;  // columns nx .. sy - 1
   const long long n1 = rows * cx, n2 = (long long)g.sy * (g.nz + 1), n3 = (long long)g.sy * (g.ny + 1);
@@ -1582,6 +1366,7 @@ __global__ void k_zero_far_faces(Grid3 g, float* a, float* b, float* c) {
     a[o] = 0.f;
     b[o] = 0.f;
     c[o] = 0.f;
+    r[o] = 0.f;
   }
 }
 
@@ -1601,7 +1386,7 @@ cudaError_t launch_zero_far_faces(const CGDesc<float>& d, cudaStream_t s) {
   const long long n = (long long)(d.g.ny + 1) * (d.g.nz + 1) * (d.g.sy - d.g.nx) +
                       (long long)d.g.sy * (d.g.nz + d.g.ny + 2);
   const long long blocks = std::min<long long>((n + kThreads - 1) / kThreads, 4096);
-  k_zero_far_faces<<<(int)std::max<long long>(blocks, 1), kThreads, 0, s>>>(d.g, d.pa, d.pb, d.q);
+  k_zero_far_faces<<<(int)std::max<long long>(blocks, 1), kThreads, 0, s>>>(d.g, d.pa, d.pb, d.q, d.r);
   return cudaGetLastError();
 }
 

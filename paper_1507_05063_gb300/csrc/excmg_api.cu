@@ -57,38 +57,6 @@ Tiling make_tiling(const Grid3& g, int tz) {
   return t;
 }
 
-// Slab depth of the residual kernel: among 1..64 the one minimising (rounds of the tiles
-// that hold interior nodes over the residual grid) x (planes per tile, halo included).
-// Tiles of boundary nodes only cost nothing (k_residual writes zeros there), and every
-// block of a round waits for the slowest, so a deep slab that leaves blocks idle loses
-// to a thin one that fills every block.
-int choose_res_tz(const Grid3& g, int grid_blocks, int requested, int rows) {
-  if (requested > 0) return requested;
-  int best = 16;
-  double best_cost = 1e300;
-  const int cands[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64};
-  for (int tz : cands) {
-    const long long tiles = (long long)((g.nx + kTX - 1) / kTX) *
-                            ((g.ny + kTY * rows - 1) / (kTY * rows)) * ((g.nz + tz - 1) / tz);
-    const long long rounds = (tiles + grid_blocks - 1) / grid_blocks;
-    const double cost = (double)rounds * (std::min(tz, g.nz + 1) + 2);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = tz;
-    }
-  }
-  return best;
-}
-
-Tiling make_res_tiling(const Grid3& g, int tz, int rows) {
-  Tiling t = make_tiling(g, tz);
-  t.nty = (g.ny + 1 + kTY * rows - 1) / (kTY * rows);
-  return t;
-}
-
-int res_rows_model(const Grid3& g) { return g.nodes() >= kResWideMinNodes ? kResRowsWide : 1; }
-
-
 // Slab depth: among 1..64 the one minimising (waves of tiles) x (planes staged per tile),
 // a model of the stencil kernel's time when every block runs at the same rate.  Large
 // grids get deep slabs (little halo re-staging); small, latency-bound grids get thin
@@ -174,7 +142,7 @@ bool options_ok(const excmg_options* o) {
     return false;
   if (o->test_phantom_blocks < 0 || o->test_phantom_blocks > 64) return false;
   if (o->autotune < -1 || o->autotune > 1) return false;
-  if (o->res_rows != 0 && o->res_rows != 1 && o->res_rows != kResRowsWide) return false;
+  if (o->res_rows != 0 && o->res_rows != 1 && o->res_rows != 4) return false;
   return true;
 }
 
@@ -226,7 +194,7 @@ struct ProbLayout {
   size_t coarse_off[EXCMG_MAX_LEVELS];  // u of levels 0 .. L-2 (float64)
   size_t r, pa, pb, q;                  // float64 CG vectors (finest size)
   size_t r32, pa32, pb32, q32, e32;     // float32 CG vectors (MIXED)
-  size_t rhs64;                         // MIXED: 2 RHS(f) of the level being refined
+  size_t rhs64;                         // MIXED: RHS(f) of the level being refined
   size_t s0, s1;                        // resident CG: s by step parity (its grids' size)
   size_t bytes;
 };
@@ -700,7 +668,7 @@ struct Item {
   ResDesc res;
   CGDesc<double> d64;
   CGDesc<float> d32;
-  double* rhs_cache;    // MIXED: 2 RHS(f) kept between refinement residuals (NULL: none)
+  double* rhs_cache;    // MIXED: RHS(f) kept between refinement residuals (NULL: none)
   double eps;           // stop at ||r|| <= eps ||b||
   long long nodes;
   // results
@@ -708,14 +676,13 @@ struct Item {
   double relres;
 };
 
-ResDesc make_res(const Grid3& g, int tile_z, int slot, const double* x, View f,
-                 const double* src, int rows) {
+ResDesc make_res(const Grid3& g, int slot, const double* x, View f, const double* src) {
   ResDesc r;
   memset(&r, 0, sizeof(r));
   r.g = g;
   r.A = make_coef(g);
-  r.rows = rows;
-  r.t = make_res_tiling(g, choose_res_tz(g, residual_grid(1LL << 40, rows), tile_z, rows), rows);
+  r.W = make_fx_weights(g);
+  r.t = make_fx_tiling(g, choose_fx_tz(&g, 1));
   r.slot = slot;
   r.u = x;
   r.f = f;
@@ -762,20 +729,18 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
   std::vector<CGState> hs;
   std::vector<ResDesc> hr;
   long long tiles = 0, rtiles = 0;  // CG tiles, residual tiles
-  // one residual launch serves every problem: they share its rows per thread (one
-  // row unless all of them take more)
-  int rows = kResRowsWide;
-  for (auto& it : items) rows = std::min(rows, it.res.rows);
+  // one launch serves every problem: they share the depth of their fixed-point slabs
+  std::vector<Grid3> grids;
+  for (const Item& it : items)
+    if (!it.d64.direct) grids.push_back(it.res.g);
+  const int fx_tz = choose_fx_tz(grids.data(), (int)grids.size());
   for (int a = 0; a < n; ++a) {
     Item& it = items[a];
     it.iters = it.refs = 0;
     it.status = EXCMG_OK;
     it.relres = 0.0;
-    if (it.res.rows != rows) {
-      it.res.t = make_res_tiling(it.res.g, it.res.t.tz, rows);
-      it.res.rows = rows;
-    }
     ResDesc r = it.res;
+    r.t = it.d64.t = make_fx_tiling(r.g, fx_tz);
     r.tile_begin = rtiles;
     if (!it.d64.direct) rtiles += r.t.count();  // DSOLVE levels form their own b
     it.d64.tile_begin = tiles;
@@ -797,6 +762,7 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
       r.tol_b2 = it.eps * it.eps;
       r.tol_r2 = 0.0;
       r.fixed = fixed ? 1 : 0;
+      r.float64 = it.d64.float64 = !fixed && it.eps < kFloat64Eps;
       r.max_iter = fixed ? fixed[a] : o->max_iter;
     }
     it.res = r;
@@ -821,8 +787,7 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
     if (nres > 0) {
       CK(cudaMemcpyAsync(c.resd(), hr.data(), sizeof(ResDesc) * nres, cudaMemcpyHostToDevice, c.s));
       CK(c.timed(EXCMG_K_RESIDUAL, res_nodes, [&] {
-        return launch_residual(false, nres, c.resd(), rtiles, residual_grid(rtiles, rows), c.st(),
-                               c.partials(), c.counters(), c.s, rows);
+        return launch_residual(false, nres, c.resd(), rtiles, c.st(), c.partials(), c.counters(), c.s);
       }));
     }
     // DSOLVE levels: one direct solve each (their states are done with 0 steps, so the
@@ -870,9 +835,9 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
       rt += r.t.count();
       if (items[a].rhs_cache && !r.src) {
         if (pass == 0) {
-          r.rhs_out = items[a].rhs_cache;  // keep 2 RHS(f) for the later passes
+          r.rhs_out = items[a].rhs_cache;  // keep RHS(f) for the later passes
         } else {
-          r.rhs2 = items[a].rhs_cache;     // r = LHS(u) - RHS(f) without recomputing RHS
+          r.rhs_in = items[a].rhs_cache;   // r = LHS(u) - RHS(f) without recomputing RHS
           r.want_b = 0;                    // ||b|| is already in the state
         }
       }
@@ -883,8 +848,7 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
     for (int a : cur) rnodes += (double)items[a].nodes;
     CK(cudaMemcpyAsync(c.resd(), rr.data(), sizeof(ResDesc) * nr, cudaMemcpyHostToDevice, c.s));
     CK(c.timed(EXCMG_K_RESIDUAL, rnodes, [&] {
-      return launch_residual(true, nr, c.resd(), rt, residual_grid(rt, rows), c.st(), c.partials(),
-                             c.counters(), c.s, rows);
+      return launch_residual(true, nr, c.resd(), rt, c.st(), c.partials(), c.counters(), c.s);
     }));
     excmg_status e = read_states(c, nslots, hs);
     if (e != EXCMG_OK) return e;
@@ -964,23 +928,17 @@ bool level_f32(const Grid3& g, bool dsolve_level, const excmg_options* o) {
 // Launch shapes of a level: the caller's tile_z, else the tuned ones (options.autotune
 // >= 0 and a cache entry), else the models.
 struct Shapes {
-  int res_tz, cg_tz, tma_tz, res_rows;
+  int cg_tz, tma_tz;
 };
 Shapes level_shapes(const Grid3& g, bool dsolve_level, const excmg_options* o) {
   Shapes sh;
   const int tz = choose_tz(g, persistent_grid(1LL << 40), o->tile_z);
   sh.cg_tz = tz;
   sh.tma_tz = o->tile_z > 0 ? tz : tma_slab_depth(tz);
-  sh.res_rows = o->res_rows > 0 ? o->res_rows : res_rows_model(g);
-  sh.res_tz = choose_res_tz(g, residual_grid(1LL << 40, sh.res_rows), o->tile_z, sh.res_rows);
   excmg_tuning t;
   if (o->tile_z == 0 && o->autotune >= 0 && tune_lookup(g, level_f32(g, dsolve_level, o), &t)) {
     // an entry's cg_tz is 0 where the single solve's engine for the grid is not tiled
     // (resident or cluster): the model's depth stays for the tiled engines of a batch
-    if (t.res_tz > 0 && (o->res_rows == 0 || o->res_rows == t.res_rows)) {
-      sh.res_tz = t.res_tz;
-      if (t.res_rows > 0) sh.res_rows = t.res_rows;
-    }
     if (t.cg_tz > 0) {
       if (level_f32(g, dsolve_level, o))
         sh.tma_tz = t.cg_tz;
@@ -1001,12 +959,13 @@ Item make_item(Prob& p, int l, int slot, const excmg_options* o) {
   const double ratio = o->eps_ratio > 0 ? o->eps_ratio : 1.0;
   it.eps = (l < 2) ? o->eps_coarse : o->eps * std::pow(ratio, (double)((int)p.lv.size() - 1 - l));
   it.nodes = g.nodes();
-  it.res = make_res(g, sh.res_tz, slot, p.level_u(l), p.fview(l), nullptr, sh.res_rows);
+  it.res = make_res(g, slot, p.level_u(l), p.fview(l), nullptr);
   it.res.forcing = o->rhs_norm == EXCMG_RHS_NORM_FORCING;
   CGDesc<double>& d = it.d64;
   d.g = g;
   d.A = it.res.A;
-  d.t = t;
+  d.W = it.res.W;
+  d.t = it.res.t;
   d.slot = slot;
   d.x = p.level_u(l);
   d.r = reinterpret_cast<double*>(p.base + p.L.r);
@@ -1044,12 +1003,11 @@ Item make_item(Prob& p, int l, int slot, const excmg_options* o) {
 }
 
 // The tuning pass of options.autotune = 1 (single solves): for every level from 2 up
-// without a cache entry, time the residual at candidate slab depths and, where the
-// level's CG engine is tiled (the persistent float64 engine above kResidentMaxNodes
-// nodes, or the float32 tensor-copy engine), three CG steps at candidate slab depths;
-// each candidate runs on the level's own solution array (overwritten by the solve
-// afterwards: boundary = g, interior = 0 at every start) with CUDA events around every
-// launch.  The fastest of each, and the model's choice with its time, go to the cache.
+// without a cache entry, time the residual and, where the level's CG engine has a slab
+// depth (the float32 tensor-copy engine), three CG steps at candidate depths; each candidate runs on the level's own
+// solution array (overwritten by the solve afterwards: boundary = g, interior = 0 at every
+// start) with CUDA events around every launch.  The fastest depth, and the model's with its
+// time, go to the cache.
 excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
   for (int l = 2; l < (int)p.lv.size(); ++l) {
     const Grid3 g = p.grid(l);
@@ -1065,13 +1023,12 @@ excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
     om.max_refine = 1;
     om.inner_tol = 1e-30;
     const Shapes model = level_shapes(g, false, &om);
-    const bool cg_tiled = f32 || g.nodes() > kResidentMaxNodes;
-    // one run: residual + three CG steps at slab depth tz for both, the residual with
-    // `rows` rows per thread; returns the mean residual launch and the mean CG step (ms)
-    auto run = [&](int tz, int rows, double& res_ms, double& step_ms) -> excmg_status {
+    const bool cg_tiled = f32;
+    // one run: residual + three CG steps at slab depth tz; returns the mean residual launch
+    // and the mean CG step (ms)
+    auto run = [&](int tz, double& res_ms, double& step_ms) -> excmg_status {
       excmg_options ot = om;
       ot.tile_z = tz;
-      ot.res_rows = rows;
       Ctx c = c0;
       c.defer = false;
       c.hist = nullptr;
@@ -1104,43 +1061,33 @@ excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
     t.N[1] = g.ny;
     t.N[2] = g.nz;
     t.f32 = f32 ? 1 : 0;
-    t.res_tz = t.res_tz_model = model.res_tz;
-    t.res_rows = t.res_rows_model = model.res_rows;
+    t.res_tz = t.res_tz_model = choose_fx_tz(&g, 1);  // one model for the fixed-point slabs
+    t.res_rows = t.res_rows_model = 1;
     t.cg_tz = t.cg_tz_model = cg_tiled ? (f32 ? model.tma_tz : model.cg_tz) : 0;
     double best_res = 1e300, best_cg = 1e300;
     std::vector<int> cands = {2, 4, 6, 8, 10, 12, 16, 20, 24, 32, 48};
     for (int& c : cands)
       if (f32 && cg_tiled) c = tma_slab_depth(c);  // CG candidates for the tensor-copy engine
-    cands.push_back(model.res_tz);
     cands.push_back(f32 ? model.tma_tz : model.cg_tz);
     std::sort(cands.begin(), cands.end());
     cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
-    // the CG engine's depths are timed in the one-row runs; the residual's over both
-    // row counts
-    const int row_cands[] = {1, kResRowsWide};
-    for (int rows : row_cands)
-      for (int tz : cands) {
-        if (tz < 1 || tz > g.nz + 1) continue;
-        double rm = 0.0, sm = 0.0;
-        excmg_status e = run(tz, rows, rm, sm);
-        if (e != EXCMG_OK) return e;
-        if (rm > 0 && rm < best_res) {
-          best_res = rm;
-          t.res_tz = tz;
-          t.res_rows = rows;
+    if (!cg_tiled) cands.resize(1);  // one run times the residual
+    for (int tz : cands) {
+      if (cg_tiled && (tz < 1 || tz > g.nz + 1)) continue;
+      double rm = 0.0, sm = 0.0;
+      excmg_status e = run(tz, rm, sm);
+      if (e != EXCMG_OK) return e;
+      if (rm > 0) best_res = std::min(best_res, rm);
+      if (cg_tiled && sm > 0) {
+        if (sm < best_cg) {
+          best_cg = sm;
+          t.cg_tz = tz;
         }
-        if (tz == model.res_tz && rows == model.res_rows) t.res_ms_model = rm;
-        if (rows == 1 && cg_tiled && sm > 0) {
-          if (sm < best_cg) {
-            best_cg = sm;
-            t.cg_tz = tz;
-          }
-          if (tz == t.cg_tz_model) t.cg_ms_model = sm;
-        }
+        if (tz == t.cg_tz_model) t.cg_ms_model = sm;
       }
-    t.res_ms = best_res < 1e300 ? best_res : 0.0;
+    }
+    t.res_ms = t.res_ms_model = best_res < 1e300 ? best_res : 0.0;
     t.cg_ms = best_cg < 1e300 ? best_cg : 0.0;
-    if (t.res_ms_model == 0.0) t.res_ms_model = t.res_ms;
     tune_store(g, f32, t);
   }
   return EXCMG_OK;
@@ -1657,13 +1604,11 @@ excmg_status excmg_residual(const excmg_grid* grid, const double* f, const doubl
   c.H = header_layout(1);
   c.s = static_cast<cudaStream_t>(stream);
   const Grid3 g = make_grid(grid->Nx, grid->Ny, grid->Nz, grid->Lx, grid->Ly, grid->Lz);
-  const int rows = res_rows_model(g);
-  ResDesc d = make_res(g, 0, 0, u, View{f, 1, g.sy, g.sz}, nullptr, rows);
+  ResDesc d = make_res(g, 0, u, View{f, 1, g.sy, g.sz}, nullptr);
   d.r = r;
   CK(cudaMemsetAsync(c.counters(), 0, sizeof(unsigned), c.s));
   CK(cudaMemcpyAsync(c.resd(), &d, sizeof(d), cudaMemcpyHostToDevice, c.s));
-  CK(launch_residual(false, 1, c.resd(), d.t.count(), residual_grid(d.t.count(), rows), c.st(),
-                     c.partials(), c.counters(), c.s, rows));
+  CK(launch_residual(false, 1, c.resd(), d.t.count(), c.st(), c.partials(), c.counters(), c.s));
   std::vector<CGState> hs;
   excmg_status e = read_states(c, 1, hs);
   if (e != EXCMG_OK) return e;

@@ -19,15 +19,15 @@ constexpr int kMaxProb = 128;    // problems per batched launch
 constexpr int kThreads = 256;    // threads of every tiled kernel
 constexpr int kTX = 32;          // x-width of a stencil tile (one warp)
 constexpr int kTY = 8;           // y-rows of a stencil tile
-// y-rows per thread of the residual kernel: 1 or kResRowsWide, per launch (ResDesc.rows).
-// Four rows share their W + E sums (7% faster on 1024x512x512) but run 16 warps per SM
-// instead of 24 (17% slower on 512x256x128); the tuning cache decides per level grid,
-// else grids of at least EXCMG_RES_WIDE_MIN_NODES nodes take four.
-constexpr int kResRowsWide = 4;
-#ifndef EXCMG_RES_WIDE_MIN_NODES
-#define EXCMG_RES_WIDE_MIN_NODES (1LL << 26)
-#endif
-constexpr long long kResWideMinNodes = EXCMG_RES_WIDE_MIN_NODES;
+// Nodes of a fixed-point stencil slab along y (fixed_slab.cuh; kTX along x).
+constexpr int kFxSlabY = 8;
+// Blocks per SM of the fixed-point stencil kernels (80 registers): the residual of
+// 320 x 255 x 257 cells takes 375 us with three, 620 with four (64 registers, spills).
+constexpr int kFxBlocks = 3;
+// Float64 solves with a stopping tolerance below this take their sums in float64: the target
+// lies under the rounding of float64 sums, so the step counts and the last digits follow
+// that rounding, and stay float64's own.
+constexpr double kFloat64Eps = 1e-13;
 constexpr int kMaxGrid = 4096;   // cap on persistent grid size (partials per problem)
 #ifndef EXCMG_CLUSTER_MAX_NODES
 #define EXCMG_CLUSTER_MAX_NODES 20000
@@ -68,6 +68,14 @@ struct Coef {
   double c0, fx, fy, fz, exy, exz, eyz;
 };
 Coef make_coef(const Grid3& g);
+// a = 1/hx^2, b, c as integers h 2^32 + l = a 2^k, the largest in [2^59, 2^60]: the
+// weights of the fixed-point sums (fixed_point.cuh).
+struct FxWeights {
+  int h[3], l[3];
+  int k;
+  long long m0;  // fx_weigh's start: its rounding terms
+};
+FxWeights make_fx_weights(const Grid3& g);
 
 // A finest-grid node array seen at the nodes of a coarser level (injection).
 struct View {
@@ -100,12 +108,11 @@ struct Tiling {
   __host__ __device__ long long count() const { return (long long)ntx * nty * ntz; }
 };
 Tiling make_tiling(const Grid3& g, int tz);
-// The residual kernel's tiling: kTY * rows rows per tile, the same x-width, slab depth tz
-// (choose_res_tz: the residual's own model of its launch).
-Tiling make_res_tiling(const Grid3& g, int tz, int rows);
-int choose_res_tz(const Grid3& g, int grid_blocks, int requested, int rows);
-// The model's rows per thread of the residual kernel for grid g (1 or kResRowsWide).
-int res_rows_model(const Grid3& g);
+// The fixed-point stencil kernels' tiling (residual, float64 CG): slabs of kTX x kFxSlabY
+// columns and tz planes of interior nodes.
+Tiling make_fx_tiling(const Grid3& g, int tz);
+// The slab depth for one launch over the n grids.
+int choose_fx_tz(const Grid3* grids, int n);
 int choose_tz(const Grid3& g, int grid_blocks, int requested);
 
 // Tensor maps of one float32 CG problem (cp.async.bulk.tensor): r and the two p buffers,
@@ -121,7 +128,9 @@ template <typename T>
 struct CGDesc {
   Grid3 g;
   Coef A;
-  Tiling t;
+  FxWeights W;            // float64: the fixed-point weights
+  int float64;            // 1: the sums in float64 (kFloat64Eps)
+  Tiling t;               // float64: fixed-point slabs (make_fx_tiling); float32: make_tiling
   Tiling tt;              // float32 tensor-copy engine: its own tiles (make_tma_tiling)
   long long tile_begin;   // first global tile index of this problem
   int slot;               // index of this problem's CGState
@@ -153,6 +162,8 @@ struct CGDesc {
 struct ResDesc {
   Grid3 g;
   Coef A;
+  FxWeights W;
+  int float64;          // 1: the sums in float64 (kFloat64Eps)
   Tiling t;
   long long tile_begin;
   int slot;             // index of this problem's CGState
@@ -160,12 +171,12 @@ struct ResDesc {
   View f;               // f at this level's nodes (unused when src is set)
   const double* src;    // NULL, or b given directly on interior nodes: r = LHS(u) + src
                         // (the adjoint's A lambda = s with lambda's boundary zero)
-  const double* rhs2;   // NULL, or 2 RHS(f) on interior nodes as an earlier pass kept it
-                        // in rhs_out (MIXED refinement steps after the first)
-  double* rhs_out;      // NULL, or receives 2 RHS(f) on interior nodes (f path only)
+  const double* rhs_in; // NULL, or RHS(f) on interior nodes as an earlier pass kept it in
+                        // rhs_out (MIXED refinement steps after the first)
+  double* rhs_out;      // NULL, or receives RHS(f) on interior nodes (f path only)
   void* r;              // TR* output
   long long osy, osz;   // node strides of r (the padded layout when TR is float; the
-                        // padding columns nx + 1 .. osy - 1 are written as zeros)
+                        // padding columns are not written: launch_zero_far_faces)
   double tol_b2;        // tol2 = max(tol_b2 * bb, tol_r2 * rr)
   double tol_r2;
   int want_b;           // compute bb (else keep the state's bb)
@@ -176,8 +187,6 @@ struct ResDesc {
   int fixed;            // exact iteration count
   double* hist;         // NULL, or receives r.r of the start in hist[0] (device)
   int hist_len;
-  int rows;             // y-rows per thread of the tiling t (1 or kResRowsWide); the same
-                        // for every problem of one launch
 };
 
 // Launch helpers (defined in cg_kernels.cu).  `descs` point to DEVICE copies.
@@ -189,12 +198,12 @@ cudaError_t launch_cg_step(int nprob, const CGDesc<T>* descs, long long total_ti
                            cudaStream_t s, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr,
                            cudaEvent_t e2 = nullptr);
 cudaError_t launch_residual(bool out_float, int nprob, const ResDesc* descs,
-                            long long total_tiles, int grid, CGState* st, double* partials,
-                            unsigned* counters, cudaStream_t s, int rows);
+                            long long total_tiles, CGState* st, double* partials,
+                            unsigned* counters, cudaStream_t s);
 // Copies n CG states into a device-mapped page-locked host buffer (dst: its device
 // address), by one block: the states reach the host without a copy-engine transfer.
 cudaError_t launch_export_states(const CGState* src, CGState* dst, int n, cudaStream_t s);
-// Zeros p_a, p_b and q of one float32 problem on its far boundary faces (x = nx and the
+// Zeros p_a, p_b, q and r of one float32 problem on its far boundary faces (x = nx and the
 // padding columns, y = ny, z = nz), which the tensor-copy engine reads but never writes.
 cudaError_t launch_zero_far_faces(const CGDesc<float>& d, cudaStream_t s);
 cudaError_t launch_add_correction(int nprob, const CGDesc<float>* inner, long long total_tiles,
@@ -204,8 +213,6 @@ cudaError_t launch_add_correction(int nprob, const CGDesc<float>* inner, long lo
 cudaError_t launch_scale_rhs(int nprob, const CGDesc<float>* inner, long long total_tiles,
                              int grid, CGState* st, cudaStream_t s);
 int persistent_grid(long long total_tiles);
-// Blocks of a residual launch: all co-resident blocks of k_residual, at most one per tile.
-int residual_grid(long long total_tiles, int rows);
 
 // All CG steps of every problem of `descs` in one cooperative launch.  Problem p owns
 // the blocks [blk_begin, blk_begin + blk_count) and iterates independently of the

@@ -1,0 +1,113 @@
+// Block fixed point: the 19-point sums of float64 data on the integer units.
+//
+// GB300 issues float64 arithmetic -- and every conversion to or from float64 -- at 2 lanes
+// per clock and SM (measured), 32-bit integer adds at 119 and shifts, logic and multiplies
+// at 64.  The stencils of the scheme are short linear forms, so a tile of float64 values
+// is brought to one power-of-two scale (the largest exponent of the tile and its halo),
+// held as 64-bit integers, and its second differences are formed there exactly; only
+// their three products with 1/hx^2, 1/hy^2, 1/hz^2 round (to about 2^-62 of the largest
+// possible sum, against float64's 2^-53 of every partial sum).
+//
+// With c a node's value, S_x, S_y, S_z its neighbour sums and E_xy ... its edge sums, and
+// d_x the second difference along x, eq. (compact)'s left-hand side is
+//   2 LHS(u) = a X + b Y + c Z,   X = d_x (12 + d_y + d_z) u
+//            = 8 S_x + E_xy + E_xz - 16 u - 2 S_y - 2 S_z   (Y, Z likewise),
+// with a = 1/hx^2, b = 1/hy^2, c = 1/hz^2: the printed weights, grouped by a, b and c.
+#pragma once
+
+#include <stdint.h>
+
+#include "excmg_internal.cuh"
+
+namespace excmg {
+
+// Bits of a fixed-point u: |u| < 2^kFxBits, so |X| <= 48 2^56 < 2^61.6.
+constexpr int kFxBits = 56;
+// Bits of a fixed-point f: |6 f + six faces| <= 12 2^57 < 2^60.6.
+constexpr int kFxBitsF = 57;
+// Tiles whose largest biased exponent lies outside [kFxMinExp, kFxMaxExp] (zeros apart)
+// take the float64 form: infinities and NaN (2047), and values whose scale or result
+// could leave float64's normal range.
+constexpr int kFxMinExp = 200, kFxMaxExp = 1800;
+
+#ifdef __CUDACC__
+
+// The magnitude bits of x's high word: ordered as |x| is, to 2^-20.
+__device__ __forceinline__ unsigned fx_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// x as an integer of scale 2^(BITS - (E - 1022)), E >= every biased exponent of the tile:
+// |result| <= 2^BITS.  Bits below the scale are dropped (none for x within 2^(BITS - 53) of
+// the largest) and negative x are complemented, not negated: x moves by one unit at most,
+// 2^-BITS of the tile's largest value.  Zero and denormal x give 0 or -1 (E >= kFxMinExp).
+template <int BITS>
+__device__ __forceinline__ long long fx_from_double(double x, int E) {
+  static_assert(BITS >= 53 && BITS <= 62, "the significand is shifted left by BITS - 53");
+  const int hi = __double2hiint(x);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u, d = (unsigned)(E - ((hi >> 20) & 0x7ff));
+  const long long m = (long long)(((unsigned long long)mh << 32 | (unsigned)__double2loint(x)) << (BITS - 53));
+  const int s = hi >> 31;
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(m ^ (long long)s), "r"(d));  // clamps at 64
+  return r;
+}
+
+// 2^n for |n| <= 1022.
+__device__ __forceinline__ double fx_pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
+
+// (float)x, to nearest (ties away from zero), by integer instructions where the result is
+// a normal number: the conversion instruction runs at the float64 rate.
+__device__ __forceinline__ float fx_to_float(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)x;  // zero, denormal or overflowing as a float, Inf, NaN
+  const unsigned m = (((unsigned)hi << 3) | (lo >> 29)) & 0x7fffffu;
+  const unsigned b = ((e - 896u) << 23 | m) + ((lo >> 28) & 1u);  // a carry moves to the next power of two
+  return __uint_as_float(b | ((unsigned)hi & 0x80000000u));
+}
+
+// x 2^q by its exponent field, for x = 0 or |x| and |x 2^q| in the normal range.
+__device__ __forceinline__ double fx_scale(double x, int q) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7fffffff) ? hi + (q << 20) : hi, __double2loint(x));
+}
+
+// -x 2^q, likewise.
+__device__ __forceinline__ double fx_scale_neg(double x, int q) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7fffffff) ? hi + (int)(((unsigned)q << 20) ^ 0x80000000u) : hi, __double2loint(x));
+}
+
+// (X W_0 + Y W_1 + Z W_2) / 2^60 for |X|, |Y|, |Z| < 2^61.6,
+// 0 <= W = h 2^32 + l <= 2^60 (l signed).  The high parts' products are kept in full, the
+// mixed ones above 2^28; the low parts' products (up to 8 units each) enter with their
+// mean, and the result is rounded, not floored: W.m0 holds both.  (A floor, half a unit
+// the same way at every node, is a smooth right-hand side: the solution of the level
+// moved by 1e-14 with it.)  |result| < 2^62.
+// PTX multiply-adds: one instruction per product, where the C form of the mixed-sign ones
+// expands to 36 for the nine.
+__device__ __forceinline__ long long fx_mad_s(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ long long fx_mad_u(unsigned a, unsigned b, long long c) {
+  long long r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ long long fx_weigh(long long X, long long Y, long long Z, const FxWeights& W) {
+  const int xh = (int)(X >> 32), yh = (int)(Y >> 32), zh = (int)(Z >> 32);
+  const long long t = fx_mad_s(zh, W.h[2], fx_mad_s(yh, W.h[1], (long long)xh * W.h[0]));
+  long long m = fx_mad_u((unsigned)X, (unsigned)W.h[0], W.m0);
+  m = fx_mad_u((unsigned)Y, (unsigned)W.h[1], m);
+  m = fx_mad_u((unsigned)Z, (unsigned)W.h[2], m);
+  m = fx_mad_s(xh, W.l[0], m);
+  m = fx_mad_s(yh, W.l[1], m);
+  m = fx_mad_s(zh, W.l[2], m);
+  return (t << 4) + (m >> 28);
+}
+
+#endif  // __CUDACC__
+
+}  // namespace excmg

@@ -113,14 +113,14 @@ extern "C" excmg_status excmg_cg_noalloc(const excmg_grid* grid, const double* f
   double* partials = reinterpret_cast<double*>(base + L.partials);
 
   const Grid3 g = make_grid(grid->Nx, grid->Ny, grid->Nz, grid->Lx, grid->Ly, grid->Lz);
-  const Tiling t = make_tiling(g, choose_tz(g, persistent_grid(1LL << 40), opt->tile_z));
+  const Tiling t = make_fx_tiling(g, choose_fx_tz(&g, 1));
   const int nblk = persistent_grid(t.count());
   ResDesc rd;
   memset(&rd, 0, sizeof(rd));
   rd.g = g;
   rd.A = make_coef(g);
-  rd.rows = 1;
-  rd.t = make_res_tiling(g, choose_res_tz(g, residual_grid(1LL << 40, 1), opt->tile_z, 1), 1);
+  rd.W = make_fx_weights(g);
+  rd.t = t;
   rd.slot = 0;
   rd.u = u;
   rd.f = View{f, 1, g.sy, g.sz};
@@ -129,6 +129,7 @@ extern "C" excmg_status excmg_cg_noalloc(const excmg_grid* grid, const double* f
   rd.want_b = 1;
   rd.forcing = opt->rhs_norm == EXCMG_RHS_NORM_FORCING;
   rd.fixed = opt->fixed_iters ? 1 : 0;
+  rd.float64 = !rd.fixed && opt->eps < kFloat64Eps;
   rd.max_iter = opt->fixed_iters ? opt->fixed_iters[0] : opt->max_iter;
   rd.tol_b2 = opt->eps * opt->eps;
   rd.tol_r2 = 0.0;
@@ -136,7 +137,9 @@ extern "C" excmg_status excmg_cg_noalloc(const excmg_grid* grid, const double* f
   memset(&cd, 0, sizeof(cd));
   cd.g = g;
   cd.A = rd.A;
-  cd.t = t;
+  cd.W = rd.W;
+  cd.float64 = rd.float64;
+  cd.t = rd.t;
   cd.slot = 0;
   cd.x = u;
   cd.r = reinterpret_cast<double*>(base + L.r);
@@ -151,8 +154,7 @@ extern "C" excmg_status excmg_cg_noalloc(const excmg_grid* grid, const double* f
   CKN(cudaMemcpyAsync(base + L.cgd, &cd, sizeof(cd), cudaMemcpyHostToDevice, s));
   const ResDesc* drd = reinterpret_cast<const ResDesc*>(base + L.resd);
   const CGDesc<double>* dcd = reinterpret_cast<const CGDesc<double>*>(base + L.cgd);
-  CKN(launch_residual(false, 1, drd, rd.t.count(), residual_grid(rd.t.count(), 1), st, partials,
-                      counters, s, 1));
+  CKN(launch_residual(false, 1, drd, rd.t.count(), st, partials, counters, s));
   long long launches = 1;
   CGState hs;
   int chunk = opt->chunk > 0 ? opt->chunk : 4;
