@@ -414,67 +414,68 @@ __global__ void __launch_bounds__(kThreads, 4) k_exp_finite_one(ProlongDesc d, l
 
 // EXP_true: u~ = u_h + (1/15) (mean of d = u_h - u_2h over the grid-2h corners of the
 // edge / face / element the node is the centre of; d itself at grid-2h nodes).
-// EXP_true tiles: 64 x 8 x 2 fine nodes per block, whose grid-2h corners are the
-// 33 x 5 x 2 coarse nodes from (x0/2, y0/2, z0/2).
-constexpr int kEtX = 64, kEtY = 8, kEtZ = 2;
-constexpr int kEcX = kEtX / 2 + 1, kEcY = kEtY / 2 + 1, kEcZ = kEtZ / 2 + 1;
+// A block marches 64 x 8 fine columns (32 x 4 coarse ones) along z, kEtK coarse planes: per
+// coarse plane it forms d at its 33 x 5 corners once, in shared memory, and a thread (one
+// fine x, the rows 2 J and 2 J + 1) sums its corner columns I and I + (i odd) -- for even i
+// the same twice, so that every lane does the same -- over rows J and J + 1; the sums of the
+// plane before serve the odd fine plane between.  2.4 float64 instructions per node (a
+// thread per node and plane pair summed the corner rows anew, 4.3).
+constexpr int kEtX = 64, kEtY = 8, kEtK = 8;
+constexpr int kEcX = kEtX / 2 + 1, kEcY = kEtY / 2 + 1;
 
 __global__ void __launch_bounds__(kThreads)
     k_exp_true(Grid3 g, const double* __restrict__ uh, const double* __restrict__ u2h,
                double* __restrict__ ut, int ntx, int nty) {
-  // EXP_true (eqs. t1, chenlin): u~ = u_h + (1/15) x (mean of d over the grid-2h corners
-  // of the node's edge, face or cell), d = u_h - u_2h at grid-2h nodes (a grid-2h node is
-  // its own corner).  The block forms d at the coarse corners of its tile once, in
-  // shared memory.  A node sums d over its corner rows (J, J + oy) x (K, K + oz) -- oy
-  // and oz are the same in every lane of a warp (a warp owns fixed rows and planes of
-  // the tile), so these branches do not diverge and only existing corners cost FP64
-  // instructions (GB300 issues few) -- at the two corner columns I and I + ox; for even
-  // i both columns are I, and the sum of the two counts it twice, so the mean over the
-  // distinct corners is (e_I + e_{I+ox}) / (2 nrows) in every lane.
-  __shared__ double D[kEcZ][kEcY][kEcX];
+  __shared__ double D[2][kEcY][kEcX];
+  static_assert(kThreads == kEtX * (kEtY / 2) && kEcX * kEcY <= kThreads, "a coarse row of fine columns per thread");
   const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, bz = blockIdx.x / (ntx * nty);
-  const int x0 = bx * kEtX, y0 = by * kEtY, z0 = bz * kEtZ;
-  const int I0 = x0 / 2, J0 = y0 / 2, K0 = z0 / 2;
   const int n1x = g.nx / 2, n1y = g.ny / 2, n1z = g.nz / 2;
+  const int I0 = bx * (kEtX / 2), J0 = by * (kEtY / 2), K0 = bz * kEtK, K1 = min(K0 + kEtK, n1z + 1);
   const long long s1y = n1x + 1, s1z = (long long)(n1x + 1) * (n1y + 1);
-  for (int e = threadIdx.x; e < kEcX * kEcY * kEcZ; e += kThreads) {
-    const int a = e % kEcX, b = (e / kEcX) % kEcY, c = e / (kEcX * kEcY);
-    const int I = I0 + a, J = J0 + b, K = K0 + c;
-    double dv = 0.0;
-    if (I <= n1x && J <= n1y && K <= n1z)
-      dv = uh[2LL * I + 2LL * J * g.sy + 2LL * K * g.sz] - u2h[I + J * s1y + K * s1z];
-    D[c][b][a] = dv;
-  }
-  __syncthreads();
-  const int tx = threadIdx.x % kEtX, tq = threadIdx.x / kEtX;  // tq = 0 .. 3
-  const int i = x0 + tx;
-  if (i > g.nx) return;  // no barrier below
-  const int ox = i & 1, ia = (i >> 1) - I0;
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int jl = tq + 4 * (m & 1), kl = m >> 1;
-    const int j = y0 + jl, k = z0 + kl;
-    if (j > g.ny || k > g.nz) continue;
-    const int oy = j & 1, oz = k & 1, ja = (j >> 1) - J0, ka = (k >> 1) - K0;
-    double e0 = D[ka][ja][ia], e1 = D[ka][ja][ia + ox];
-    if (oy) {  // uniform in the warp
-      e0 += D[ka][ja + 1][ia];
-      e1 += D[ka][ja + 1][ia + ox];
+  // this thread's corner (the first 165) and its fine column
+  const int ca = threadIdx.x % kEcX, cb = threadIdx.x / kEcX;
+  const bool corner = cb < kEcY && I0 + ca <= n1x && J0 + cb <= n1y;
+  const double* pc = uh + (2LL * (I0 + ca) + 2LL * (J0 + cb) * g.sy + 2LL * K0 * g.sz);
+  const double* pd = u2h + (I0 + ca + (J0 + cb) * s1y + K0 * s1z);
+  const int tx = threadIdx.x % kEtX, jq = threadIdx.x / kEtX;
+  const int i = 2 * I0 + tx, j = 2 * (J0 + jq), ia = tx >> 1, ib = ia + (tx & 1);
+  const bool row0 = i <= g.nx && j <= g.ny, row1 = i <= g.nx && j + 1 <= g.ny;
+  const long long o = i + j * g.sy + 2LL * K0 * g.sz;
+  const double* u = uh + o;
+  double* t = ut + o;
+  double a1 = 0.0, s1 = 0.0;  // the plane before: row J, rows J and J + 1
+  for (int K = K0; K <= K1; ++K) {
+    if (K > n1z) break;  // the grid's last plane is done
+    const bool last = K == K1;  // the next block's first plane, for the odd plane before it
+    double (*P)[kEcX] = D[K & 1];
+    if (corner) P[cb][ca] = __ldg(pc) - __ldg(pd);
+    pc += 2 * g.sz;
+    pd += s1z;
+    // u of the odd plane before and of this plane
+    double um0 = 0.0, um1 = 0.0, u0 = 0.0, u1 = 0.0;
+    if (K > K0) {
+      if (row0) um0 = __ldg(u - g.sz);
+      if (row1) um1 = __ldg(u - g.sz + g.sy);
     }
-    if (oz) {
-      double f0 = D[ka + 1][ja][ia], f1 = D[ka + 1][ja][ia + ox];
-      if (oy) {
-        f0 += D[ka + 1][ja + 1][ia];
-        f1 += D[ka + 1][ja + 1][ia + ox];
-      }
-      e0 += f0;
-      e1 += f1;
+    if (!last) {
+      if (row0) u0 = __ldg(u);
+      if (row1) u1 = __ldg(u + g.sy);
     }
-    // (1/15) x 1 / (2 x the number of corner rows): compile-time constants
-    const int nrows = (1 + oy) * (1 + oz);
-    const double w = nrows == 1 ? 1.0 / 30.0 : (nrows == 2 ? 1.0 / 60.0 : 1.0 / 120.0);
-    const long long o = i + (long long)j * g.sy + (long long)k * g.sz;
-    ut[o] = fma(e0 + e1, w, uh[o]);
+    __syncthreads();  // (the other buffer's readers are a barrier behind)
+    const double a = P[jq][ia] + P[jq][ib], s = a + (P[jq + 1][ia] + P[jq + 1][ib]);
+    // (1/15) over twice the number of corner rows
+    if (K > K0) {
+      if (row0) t[-g.sz] = fma(a + a1, 1.0 / 60.0, um0);
+      if (row1) t[g.sy - g.sz] = fma(s + s1, 1.0 / 120.0, um1);
+    }
+    if (!last) {
+      if (row0) t[0] = fma(a, 1.0 / 30.0, u0);
+      if (row1) t[g.sy] = fma(s, 1.0 / 60.0, u1);
+    }
+    a1 = a;
+    s1 = s;
+    u += 2 * g.sz;
+    t += 2 * g.sz;
   }
 }
 
@@ -590,7 +591,7 @@ cudaError_t launch_exp_finite_one(const ProlongDesc& d, cudaStream_t s) {
 cudaError_t launch_exp_true(const Grid3& g, const double* uh, const double* u2h, double* ut,
                             cudaStream_t s) {
   const int ntx = (g.nx + 1 + kEtX - 1) / kEtX, nty = (g.ny + 1 + kEtY - 1) / kEtY;
-  const long long ntz = (g.nz + 1 + kEtZ - 1) / kEtZ;
+  const long long ntz = (g.nz / 2 + 1 + kEtK - 1) / kEtK;
   const long long blocks = (long long)ntx * nty * ntz;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   k_exp_true<<<(unsigned)blocks, kThreads, 0, s>>>(g, uh, u2h, ut, ntx, nty);
