@@ -495,6 +495,8 @@ excmg_status cg_loop(const Ctx& c, int n, CGDesc<T>* ddesc, long long tiles, int
     if (resident_box(hd[0].g, D, smem)) {
       D.g = hd[0].g;
       D.A = hd[0].A;
+      D.W = hd[0].W;
+      D.float64 = hd[0].float64;
       D.slot = hd[0].slot;
       D.x = reinterpret_cast<double*>(hd[0].x);
       D.r = reinterpret_cast<double*>(hd[0].r);
@@ -505,7 +507,7 @@ excmg_status cg_loop(const Ctx& c, int n, CGDesc<T>* ddesc, long long tiles, int
       D.s1 = reinterpret_cast<double*>(hd[0].s1);
       D.hist = hd[0].hist;
       D.hist_len = hd[0].hist_len;
-      double2* pairs = reinterpret_cast<double2*>(c.partials());  // 2 G pairs
+      void* pairs = c.partials();  // 2 G block sums
       CK(cudaMemsetAsync(c.bar(), 0, 2 * sizeof(unsigned), c.s));  // counter, time-out flag
       if (c.launches) *c.launches += 1;
       if (c.prof) {

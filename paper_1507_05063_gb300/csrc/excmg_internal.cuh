@@ -267,6 +267,8 @@ constexpr long long kBatchSoloNodes = EXCMG_BATCH_SOLO_NODES;
 struct ResidentDesc {
   Grid3 g;
   Coef A;
+  FxWeights W;            // the fixed-point weights
+  int float64;            // 1: the sums in float64 (kFloat64Eps)
   int slot;               // CGState of the problem
   int bx, by, bz;         // interior nodes per box
   int nbx, nby, nbz;      // boxes per direction (grid = their product)
@@ -283,8 +285,8 @@ struct ResidentDesc {
 // Chooses the boxes for grid g; false if the grid does not fit or the device has no
 // cooperative launch.  smem: dynamic shared memory per block.
 bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem);
-// pairs: 2 G double2 (G = nbx nby nbz); counter, err: zeroed.
-cudaError_t launch_cg_resident(const ResidentDesc& D, size_t smem, CGState* st, double2* pairs,
+// parts: 2 G block sums of 32 bytes (G = nbx nby nbz <= 320); counter, err: zeroed.
+cudaError_t launch_cg_resident(const ResidentDesc& D, size_t smem, CGState* st, void* parts,
                                unsigned* counter, int* err, cudaStream_t s);
 
 // DSOLVE by the discrete sine transform (dsolve_kernels.cu): one block per descriptor

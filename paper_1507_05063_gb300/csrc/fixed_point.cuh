@@ -84,6 +84,9 @@ __device__ __forceinline__ double fx_scale_neg(double x, int q) {
 // mean, and the result is rounded, not floored: W.m0 holds both.  (A floor, half a unit
 // the same way at every node, is a smooth right-hand side: the solution of the level
 // moved by 1e-14 with it.)  |result| < 2^62.
+// The power of two of the sums L (2 LHS = L 2^q) at scale E.
+__device__ __forceinline__ int fx_sum_exp(int k, int E) { return 60 - k - (kFxBits - (E - 1022)); }
+
 // PTX multiply-adds: one instruction per product, where the C form of the mixed-sign ones
 // expands to 36 for the nine.
 __device__ __forceinline__ long long fx_mad_s(int a, int b, long long c) {

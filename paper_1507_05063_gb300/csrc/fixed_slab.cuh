@@ -137,9 +137,6 @@ __device__ __forceinline__ int block_exp(const uint4* s_mag) {
   return m == 0 ? 0 : E >= kFxMinExp && E <= kFxMaxExp ? E : -1;
 }
 
-// The power of two of the sums L (2 LHS = L 2^q) at scale E.
-__device__ __forceinline__ int fx_sum_exp(int k, int E) { return 60 - k - (kFxBits - (E - 1022)); }
-
 // The scale of a group from its exponent and the previous group's.
 __device__ __forceinline__ int fx_group_scale(int E, int Eprev) { return max(max(E, Eprev), kFxMinExp); }
 

@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "excmg_internal.cuh"
+#include "fixed_point.cuh"
 
 namespace excmg {
 namespace {
@@ -33,7 +34,7 @@ namespace {
 constexpr int kRsThreads = 256;
 constexpr unsigned long long kRsSpinLimit = 1ull << 25;
 constexpr int kRsHB = 6;  // halo nodes per thread whose loads are issued ahead
-constexpr int kRsPB = 8;  // block partials per lane in flight
+constexpr int kRsPB = 10;  // block sums per lane: up to 320 blocks
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
@@ -46,14 +47,12 @@ __device__ __forceinline__ double rs_xor_sum(double v, int from) {
   return v;
 }
 
-// Block sums of (a, b) over the first nw warps (the warps that own nodes; the others
-// hold zeros), valid in every lane of warp 0.  Those threads park their values in shared
-// memory; warp 0 adds them with a and b packed into the two half-warps (lanes 0-15 the
-// a-values, lanes 16-31 the b-values: 2 nw values per lane as a pairwise tree, then a
-// butterfly over 16 lanes), so each level of the dependence chain is one float64 warp
-// instruction for both sums.  On GB300 every float64 warp instruction costs the narrow
-// FP64 pipe the same whether it carries one sum or two.  nw is the same in every block.
-__device__ double2 rs_block_sum2(double a, double b, double* s_park, int nw) {
+// Float64 block sums of (a, b) over the first nw warps (the warps that own nodes; the others
+// hold zeros), valid in every lane of warp 0: for blocks whose sums are not for fixed point.
+// Those threads park their values in shared memory; warp 0 adds them with a and b packed into
+// the two half-warps, so each level of the dependence chain is one float64 warp instruction
+// for both sums.
+__device__ __noinline__ double2 rs_block_sum2(double a, double b, double* s_park, int nw) {
   if (threadIdx.x < 32 * nw) {
     s_park[threadIdx.x] = a;
     s_park[kRsThreads + threadIdx.x] = b;
@@ -78,16 +77,68 @@ __device__ double2 rs_block_sum2(double a, double b, double* s_park, int nw) {
   return t;
 }
 
-// Reduction number `seq` (1, 2, ...): thread 0 stores this block's partials as pair b of
+// ---- sums of r.r and w.r as integers ----
+// A float64 warp instruction occupies the narrow FP64 pipe for 64 clocks and a level of a
+// float64 tree takes at least that; a step of a small level is a chain of such levels.  The
+// threads' partial sums are therefore brought to one power of two and added as integers: in
+// a warp by three 32-bit reductions of 19-bit pieces, in a block and over the grid as 64-bit
+// sums.  Every block adds the same integers, so the sums are the same in every block.
+
+// One block's sums: gamma = g 2^eg, delta = d 2^ed; eg = kRsRaw: g and d are the bits of
+// float64 sums (infinities, NaN, extreme exponents, float64 solves).
+struct alignas(16) RsPart {
+  long long g, d;
+  int eg, ed;
+  long long pad;
+};
+constexpr int kRsRaw = 1 << 20;
+constexpr int kRsBits = 57;  // of a thread's partial sum: 32 of them fit 62 bits
+
+// x as an integer of scale 2^(kRsBits - (E - 1022)), rounded; |x| < 2^(E - 1022).
+__device__ __forceinline__ long long rs_fixed(double x, int E) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  // one bit below the unit, for rounding
+  unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(x)) << (kRsBits - 53 + 1);
+  const int d = min(E - e, 63);
+  m = ((m >> d) + 1) >> 1;
+  return hi < 0 ? -(long long)m : (long long)m;
+}
+
+// The warp's sum of v, |v| <= 2^57, in every lane.
+__device__ __forceinline__ long long rs_warp_sum(long long v) {
+  const int c0 = __reduce_add_sync(0xffffffffu, (int)(v & 0x7ffff));
+  const int c1 = __reduce_add_sync(0xffffffffu, (int)((v >> 19) & 0x7ffff));
+  const int c2 = __reduce_add_sync(0xffffffffu, (int)(v >> 38));
+  return ((long long)c2 << 38) + ((long long)c1 << 19) + c0;
+}
+
+// v 2^-n, rounded.
+__device__ __forceinline__ long long rs_round(long long v, int n) {
+  n = min(n, 62);
+  return (v + ((1LL << n) >> 1)) >> n;
+}
+
+// v 2^e as float64.
+__device__ __forceinline__ double rs_double(long long v, int e) {
+  const double x = (double)v;
+  const int h = e / 2;
+  return x * fx_pow2(h) * fx_pow2(e - h);
+}
+
+// Reduction number `seq` (1, 2, ...): thread 0 stores this block's sums as part b of
 // the set seq & 1 (two sets: a block can be one reduction ahead of another's reads, never
 // two), arrives on the counter with release semantics -- which also publishes every
 // global store the block's threads made before the block barrier that precedes this
 // call -- and waits (bounded) until all G blocks have arrived.  Returns, in every
 // thread, false if the wait ran out or another block reported a time-out.
-__device__ bool rs_arrive_wait(double2 part, double2* pairs, unsigned* counter, int G, unsigned seq,
+__device__ bool rs_arrive_wait(const RsPart& part, RsPart* parts, unsigned* counter, int G, unsigned seq,
                                int* err, int* s_ok) {
   if (threadIdx.x == 0) {
-    __stcg(&pairs[(size_t)(seq & 1) * G + blockIdx.x], part);
+    int4* to = reinterpret_cast<int4*>(&parts[(size_t)(seq & 1) * G + blockIdx.x]);
+    __stcg(to, reinterpret_cast<const int4*>(&part)[0]);
+    __stcg(to + 1, reinterpret_cast<const int4*>(&part)[1]);
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
     const unsigned target = seq * (unsigned)G;
     int ok = 1;
@@ -106,32 +157,52 @@ __device__ bool rs_arrive_wait(double2 part, double2* pairs, unsigned* counter, 
   return *s_ok != 0;
 }
 
-// Warp 0, after the wait: the sums of the G pairs of set seq & 1, in a fixed order,
-// identical in every lane and every block.  As in rs_block_sum2 the two sums share the
-// warp: lanes 0-15 take the first members of pairs h, h + 16, ... (h = lane mod 16),
-// lanes 16-31 the second members (kRsPB loads in flight, a tree within the lane), then a
-// butterfly over 16 lanes.
-__device__ double2 rs_read_pairs(const double2* pairs, int G, unsigned seq) {
-  const double* set = reinterpret_cast<const double*>(pairs + (size_t)(seq & 1) * G);
-  const int lane = threadIdx.x & 31, h = lane & 15, m = lane >> 4;
-  double acc = 0.0;
-  for (int i0 = 0; i0 < G; i0 += 16 * kRsPB) {
-    const int nv = min(kRsPB, (G - i0 + 15) / 16);  // values per lane in this chunk
-    double v[kRsPB];
+// Warp 0, after the wait: the sums of the G parts of set seq & 1, identical in every lane and
+// every block: the parts brought to the largest exponent (nine bits above it for up to 512
+// parts) and added as integers, or, where a part is float64, all as float64 in a fixed order.
+__device__ double2 rs_read_parts(const RsPart* parts, int G, unsigned seq) {
+  const int4* set = reinterpret_cast<const int4*>(parts + (size_t)(seq & 1) * G);
+  const int lane = threadIdx.x & 31;
+  RsPart v[kRsPB];
+  int mg = -kRsRaw, md = -kRsRaw;
+  bool raw = false;
+#pragma unroll
+  for (int u = 0; u < kRsPB; ++u) {
+    const int i = lane + 32 * u;
+    v[u].g = v[u].d = 0;
+    v[u].eg = v[u].ed = -kRsRaw;
+    if (i < G) {
+      reinterpret_cast<int4*>(&v[u])[0] = __ldcg(set + 2 * i);
+      reinterpret_cast<int4*>(&v[u])[1] = __ldcg(set + 2 * i + 1);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kRsPB; ++u) {
+    raw = raw || v[u].eg == kRsRaw;
+    mg = max(mg, v[u].eg);
+    md = max(md, v[u].ed);
+  }
+  if (__any_sync(0xffffffffu, raw)) {
+    double g = 0.0, d = 0.0;
 #pragma unroll
     for (int u = 0; u < kRsPB; ++u) {
-      const int i = i0 + h + 16 * u;
-      v[u] = i < G ? __ldcg(set + 2 * i + m) : 0.0;
+      if (lane + 32 * u >= G) break;
+      const bool f = v[u].eg == kRsRaw;
+      g += f ? __longlong_as_double(v[u].g) : rs_double(v[u].g, v[u].eg);
+      d += f ? __longlong_as_double(v[u].d) : rs_double(v[u].d, v[u].ed);
     }
-#pragma unroll
-    for (int w = 1; w < kRsPB; w *= 2)
-#pragma unroll
-      for (int u = 0; u + w < kRsPB; u += 2 * w)
-        if (u + w < nv) v[u] += v[u + w];
-    acc += v[0];
+    return make_double2(rs_xor_sum(g, 16), rs_xor_sum(d, 16));
   }
-  const double r = rs_xor_sum(acc, 8);
-  return make_double2(__shfl_sync(0xffffffffu, r, 0), __shfl_sync(0xffffffffu, r, 16));
+  mg = __reduce_max_sync(0xffffffffu, mg);
+  md = __reduce_max_sync(0xffffffffu, md);
+  long long g = 0, d = 0;
+#pragma unroll
+  for (int u = 0; u < kRsPB; ++u) {
+    g += rs_round(v[u].g, mg - v[u].eg + 9);
+    d += rs_round(v[u].d, md - v[u].ed + 9);
+  }
+  // |sum over a lane's parts| < 2^(62 - 9 + 4)
+  return make_double2(rs_double(rs_warp_sum(g), mg + 9), rs_double(rs_warp_sum(d), md + 9));
 }
 
 // 19-point A-stencil at offset 0 of P with strides (1, ey, ez).  `shallow`: the seven
@@ -152,10 +223,25 @@ __device__ __forceinline__ double rs_stencil(const double* P, int ey, int ez, co
   return fma(A.c0, P[0], fma(A.fx, SX, fma(A.fy, SY, fma(A.fz, SZ, fma(A.exy, EXY, fma(A.exz, EXZ, A.eyz * EYZ))))));
 }
 
-__global__ void __launch_bounds__(kRsThreads)
-    k_cg_resident(const ResidentDesc D, CGState* st, double2* pairs, unsigned* counter, int* err) {
+// 2 LHS at offset 0 of the integers P with strides (1, ey, ez) (fixed_point.cuh).
+__device__ __forceinline__ long long rs_stencil_fx(const long long* P, int ey, int ez, const FxWeights& W) {
+  const long long SX = P[-1] + P[1], SY = P[-ey] + P[ey], SZ = P[-ez] + P[ez];
+  const long long EXY = (P[-1 - ey] + P[1 - ey]) + (P[-1 + ey] + P[1 + ey]);
+  const long long EXZ = (P[-1 - ez] + P[1 - ez]) + (P[-1 + ez] + P[1 + ez]);
+  const long long EYZ = (P[-ey - ez] + P[ey - ez]) + (P[-ey + ez] + P[ey + ez]);
+  const long long Q = ((SX + SY) + (SZ + (P[0] << 3))) << 1;
+  return fx_weigh((EXY + EXZ - Q) + 10 * SX, (EXY + EYZ - Q) + 10 * SY, (EXZ + EYZ - Q) + 10 * SZ, W);
+}
+
+// ONE: boxes of at most one node per thread, whose vectors stay in the threads' registers;
+// else they are in shared memory.
+template <bool ONE>
+__global__ void __launch_bounds__(kRsThreads, 2)
+    k_cg_resident(const ResidentDesc D, CGState* st, RsPart* parts, unsigned* counter, int* err) {
   extern __shared__ __align__(16) double s_vec[];
   __shared__ double s_park[2 * kRsThreads];
+  __shared__ uint4 s_mag[kRsThreads / 128];
+  __shared__ long long s_sum[2][kRsThreads / 32];
   __shared__ int s_ok;
   __shared__ double s_alpha, s_beta;
   __shared__ int s_stop;
@@ -167,18 +253,21 @@ __global__ void __launch_bounds__(kRsThreads)
   const int EX = BX + 2, EY = BY + 2, EZ = BZ + 2;
   const int B = BX * BY * BZ, ext = EX * EY * EZ;
   const int nw_own = min(kRsThreads, B + 31) / 32;  // warps that own nodes
-  const bool shallow = B <= kRsThreads;               // at most one node per thread
   const int b = blockIdx.x;
   const int ibx = b % D.nbx, iby = (b / D.nbx) % D.nby, ibz = b / (D.nbx * D.nby);
   // global node of box-local (0, 0, 0); the halo starts one node before
   const int i0 = 1 + ibx * BX, j0 = 1 + iby * BY, k0 = 1 + ibz * BZ;
-  double* R = s_vec;  // ext: (lx+1) + EX (ly+1) + EX EY (lz+1)
-  double* X = R + ext;
+  // r of the box and its halo as integers of the block's scale (or float64 bits):
+  // (lx+1) + EX (ly+1) + EX EY (lz+1); then r, x, p, s, w of the box
+  long long* RI = reinterpret_cast<long long*>(s_vec);
+  double* R = s_vec + ext;
+  double* X = R + B;
   double* P = X + B;
   double* Sv = P + B;
   double* W = Sv + B;
   const Coef A = D.A;
-  // own node q of the box: its index in R and in the level's node array; valid = the
+  const FxWeights FW = D.W;
+  // own node q of the box: its index in RI and in the level's node array; valid = the
   // node exists (boxes at the far faces of the grid may be partial)
   struct Own {
     int e;
@@ -191,13 +280,24 @@ __global__ void __launch_bounds__(kRsThreads)
     Own w;
     w.e = (lx + 1) + EX * ((ly + 1) + EY * (lz + 1));
     w.o = gi + gj * g.sy + (long long)gk * g.sz;
-    w.valid = gi < g.nx && gj < g.ny && gk < g.nz;
+    w.valid = q < B && gi < g.nx && gj < g.ny && gk < g.nz;
     return w;
   };
-  // boxes of at most one node per thread: this thread's node, computed once (the index
-  // arithmetic divides by the box extents) instead of in every step
-  const Own mine = own_node(threadIdx.x < B ? threadIdx.x : 0);
-  auto node_of = [&](int q) -> Own { return shallow ? mine : own_node(q); };
+  // ONE: this thread's node, computed once (the index arithmetic divides by the box extents)
+  // instead of in every step, and its vectors
+  const Own mine = own_node(threadIdx.x);
+  double xr = 0.0, xx = 0.0, xp = 0.0, xs = 0.0, xw = 0.0;
+  // every own node of this thread: f(node, r, x, p, s, w)
+  auto each = [&](auto f) {
+    if (ONE) {
+      if (mine.valid) f(mine, xr, xx, xp, xs, xw);
+    } else {
+      for (int q = threadIdx.x; q < B; q += kRsThreads) {
+        const Own n = own_node(q);
+        if (n.valid) f(n, R[q], X[q], P[q], Sv[q], W[q]);
+      }
+    }
+  };
   // shell position h (0 .. ext - B - 1): the 2 z-faces, then the 2 y-faces, then the 2
   // x-faces of the extended box
   const int zf = EX * EY, yf = EX * BZ, xf = BY * BZ;
@@ -230,49 +330,9 @@ __global__ void __launch_bounds__(kRsThreads)
   auto interior = [&](int gi, int gj, int gk) {
     return gi > 0 && gi < g.nx && gj > 0 && gj < g.ny && gk > 0 && gk < g.nz;
   };
-  // ---- start: r_0 on the box and its halo, x; p = s = 0; w_0 = A r_0; publish w_0, s = 0
-  for (int e = threadIdx.x; e < ext; e += kRsThreads) R[e] = 0.0;
-  __syncthreads();
-  for (int q = threadIdx.x; q < B; q += kRsThreads) {
-    const Own w = own_node(q);
-    R[w.e] = w.valid ? D.r[w.o] : 0.0;
-    X[q] = w.valid ? D.x[w.o] : 0.0;
-    P[q] = 0.0;
-    Sv[q] = 0.0;
-  }
-  for (int h = threadIdx.x; h < nshell; h += kRsThreads) {
-    int e, gi, gj, gk;
-    shell_node(h, e, gi, gj, gk);
-    R[e] = interior(gi, gj, gk) ? D.r[gi + gj * g.sy + (long long)gk * g.sz] : 0.0;
-  }
-  __syncthreads();
-  double acc_d = 0.0;
-  for (int q = threadIdx.x; q < B; q += kRsThreads) {
-    const Own n = own_node(q);
-    double w = 0.0;
-    if (n.valid) {
-      w = rs_stencil(R + n.e, EX, EX * EY, A, shallow);
-      acc_d = fma(w, R[n.e], acc_d);
-      D.w0[n.o] = w;
-      D.s0[n.o] = 0.0;
-    }
-    W[q] = w;
-  }
-  // CG scalars: warp 0 keeps identical copies in all its lanes (and in every block)
-  double gam = S->rr, alpha = 0.0, beta = 0.0, delta = 0.0;
-  const double tol2 = S->tol2;
-  int iter = S->iter;
-  const int max_iter = S->max_iter, fixed = S->fixed;
-  int status = EXCMG_OK;
-  const int lane = threadIdx.x & 31;
-  // the published r, w, s of up to kRsHB halo nodes per thread, loaded right after each
-  // reduction's wait, so that the load latency overlaps the reading of the partials and
-  // the scalar arithmetic (zero on the boundary)
-  double hr[kRsHB], hw[kRsHB], hs[kRsHB];
-  int he[kRsHB];
-  // this thread's shell nodes (index in R, offset in the level's arrays or -1 outside the
+  // this thread's shell nodes (index in RI, offset in the level's arrays or -1 outside the
   // interior), computed once: after each wait the loads issue at once
-  int ho[kRsHB];
+  int he[kRsHB], ho[kRsHB];
 #pragma unroll
   for (int u = 0; u < kRsHB; ++u) {
     const int h = threadIdx.x + u * kRsThreads;
@@ -284,6 +344,78 @@ __global__ void __launch_bounds__(kRsThreads)
       if (interior(gi, gj, gk)) ho[u] = gi + gj * g.sy + gk * g.sz;
     }
   }
+  // The box of integers from the new r: own (each thread its r), halo hn (and, of shells of
+  // more than kRsHB per thread, the float64 bits already in RI); mag: this thread's largest
+  // magnitude word.  Returns the scale E, or -1 for a box of float64 bits.  Two barriers.
+  auto fill = [&](unsigned mag, const double (&hn)[kRsHB]) -> int {
+    mag = __reduce_max_sync(0xffffffffu, mag);
+    if ((threadIdx.x & 31) == 0) reinterpret_cast<unsigned*>(s_mag)[threadIdx.x >> 5] = mag;
+    __syncthreads();
+    const uint4 m0 = s_mag[0], m1 = s_mag[1];
+    mag = max(max(max(m0.x, m0.y), max(m0.z, m0.w)), max(max(m1.x, m1.y), max(m1.z, m1.w)));
+    // r.r and w.r stay in the normal range too
+    int E = (int)(mag >> 20);
+    const int q = fx_sum_exp(FW.k, E);
+    if (E < 600 || E > 1400 || q < -400 || q > 300 || D.float64) E = -1;
+    auto put = [&](double v) { return E < 0 ? __double_as_longlong(v) : fx_from_double<kFxBits>(v, E); };
+    each([&](const Own& n, double& r, double&, double&, double&, double&) { RI[n.e] = put(r); });
+#pragma unroll
+    for (int u = 0; u < kRsHB; ++u)
+      if (he[u] >= 0) RI[he[u]] = put(hn[u]);
+    for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
+      int e, gi, gj, gk;
+      shell_node(h, e, gi, gj, gk);
+      RI[e] = put(__longlong_as_double(RI[e]));
+    }
+    __syncthreads();
+    return E;
+  };
+  // w = A r of the box (published to Wn), and the block's sums of r.r and w.r in thread 0
+  auto apply = [&](int E, double* Wn) -> RsPart {
+    double acc_g = 0.0, acc_d = 0.0;
+    const int qL = fx_sum_exp(FW.k, E) - 1;
+    each([&](const Own& n, double& r, double&, double&, double&, double& w) {
+      if (E >= 0)
+        w = fx_scale_neg((double)rs_stencil_fx(RI + n.e, EX, EX * EY, FW), qL);
+      else
+        w = rs_stencil(reinterpret_cast<const double*>(RI) + n.e, EX, EX * EY, A, ONE);
+      acc_g = fma(r, r, acc_g);
+      acc_d = fma(w, r, acc_d);
+      __stcg(Wn + n.o, w);
+    });
+    RsPart part;
+    part.pad = 0;
+    if (E < 0) {
+      const double2 t = rs_block_sum2(acc_g, acc_d, s_park, nw_own);
+      part.g = __double_as_longlong(t.x);
+      part.d = __double_as_longlong(t.y);
+      part.eg = part.ed = kRsRaw;
+      return part;
+    }
+    // bounds of a thread's sums: up to 16 nodes, |r| < 2^(E - 1022), |w| < 2^(qL + 63)
+    const int eg = 1022 + 2 * (E - 1022) + 4, ed = 1022 + (E - 1022) + (qL + 63) + 4;
+    const long long sg = rs_warp_sum(rs_fixed(acc_g, eg)), sd = rs_warp_sum(rs_fixed(acc_d, ed));
+    if ((threadIdx.x & 31) == 0) {
+      s_sum[0][threadIdx.x >> 5] = rs_round(sg, 3);
+      s_sum[1][threadIdx.x >> 5] = rs_round(sd, 3);
+    }
+    __syncthreads();
+    part.g = part.d = 0;
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int w = 0; w < kRsThreads / 32; ++w) {
+        part.g += s_sum[0][w];
+        part.d += s_sum[1][w];
+      }
+    }
+    part.eg = eg - 1022 - kRsBits + 3;
+    part.ed = ed - 1022 - kRsBits + 3;
+    return part;
+  };
+  // the published r, w, s of up to kRsHB halo nodes per thread, loaded right after each
+  // reduction's wait, so that the load latency overlaps the reading of the partials and
+  // the scalar arithmetic (zero on the boundary)
+  double hr[kRsHB], hw[kRsHB], hs[kRsHB];
   auto load_halo = [&](int par) {
     const double* Rg = par ? D.r1 : D.r;
     const double* Wg = par ? D.w1 : D.w0;
@@ -298,10 +430,40 @@ __global__ void __launch_bounds__(kRsThreads)
       }
     }
   };
+  // ---- start: r_0 on the box and its halo, x; p = s = 0; w_0 = A r_0; publish w_0, s = 0
+  for (int e = threadIdx.x; e < ext; e += kRsThreads) RI[e] = 0;
+  __syncthreads();
+  unsigned mag = 0;
+  each([&](const Own& n, double& r, double& x, double& p, double& s, double& w) {
+    r = D.r[n.o];
+    x = D.x[n.o];
+    p = s = w = 0.0;
+    D.s0[n.o] = 0.0;
+    mag = max(mag, fx_mag(r));
+  });
+#pragma unroll
+  for (int u = 0; u < kRsHB; ++u) {
+    hr[u] = ho[u] >= 0 ? D.r[ho[u]] : 0.0;
+    mag = max(mag, fx_mag(hr[u]));
+  }
+  for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
+    int e, gi, gj, gk;
+    shell_node(h, e, gi, gj, gk);
+    const double v = interior(gi, gj, gk) ? D.r[gi + gj * g.sy + (long long)gk * g.sz] : 0.0;
+    RI[e] = __double_as_longlong(v);
+    mag = max(mag, fx_mag(v));
+  }
+  RsPart part = apply(fill(mag, hr), D.w0);
+  // CG scalars: warp 0 keeps identical copies in all its lanes (and in every block)
+  double gam = S->rr, alpha = 0.0, beta = 0.0, delta = 0.0;
+  const double tol2 = S->tol2;
+  int iter = S->iter;
+  const int max_iter = S->max_iter, fixed = S->fixed;
+  int status = EXCMG_OK;
+  const int lane = threadIdx.x & 31;
   unsigned seq = 1;
   {
-    const double2 part = rs_block_sum2(0.0, acc_d, s_park, nw_own);
-    const bool ok = rs_arrive_wait(part, pairs, counter, G, seq, err, &s_ok);
+    const bool ok = rs_arrive_wait(part, parts, counter, G, seq, err, &s_ok);
     if (ok) load_halo(0);
     if (threadIdx.x < 32) {
       int stop = 0;
@@ -309,7 +471,7 @@ __global__ void __launch_bounds__(kRsThreads)
         status = EXCMG_ERR_TIMEOUT;
         stop = 1;
       } else {
-        delta = rs_read_pairs(pairs, G, seq).y;
+        delta = rs_read_parts(parts, G, seq).y;
         if (delta == 0.0 && gam == 0.0) {
           stop = 1;  // exact solution (fixed-count mode)
         } else if (!(delta > 0.0) || !isfinite(delta)) {
@@ -338,27 +500,26 @@ __global__ void __launch_bounds__(kRsThreads)
     double* Wn = par ? D.w0 : D.w1;
     double* Sn = par ? D.s0 : D.s1;
     // 1. own nodes: p, s, x, r; publish r and s
-    for (int q = threadIdx.x; q < B; q += kRsThreads) {
-      const Own n = node_of(q);
-      if (!n.valid) continue;
-      const int e = n.e;
-      const long long o = n.o;
-      const double r = R[e];
-      const double pv = fma(bt, P[q], r);
-      const double sv = fma(bt, Sv[q], W[q]);
-      P[q] = pv;
-      Sv[q] = sv;
-      X[q] = fma(a, pv, X[q]);
+    mag = 0;
+    each([&](const Own& n, double& r, double& x, double& p, double& s, double& w) {
+      const double pv = fma(bt, p, r), sv = fma(bt, s, w);
+      p = pv;
+      s = sv;
+      x = fma(a, pv, x);
       const double rn = fma(-a, sv, r);
-      R[e] = rn;
-      __stcg(Rn + o, rn);
-      __stcg(Sn + o, sv);
-    }
+      r = rn;
+      mag = max(mag, fx_mag(rn));
+      __stcg(Rn + n.o, rn);
+      __stcg(Sn + n.o, sv);
+    });
     // 2. the halo's new r, with the owner's fused operations; shells larger than kRsHB
     // per thread finish with plain loads
+    double hn[kRsHB];
 #pragma unroll
-    for (int u = 0; u < kRsHB; ++u)
-      if (he[u] >= 0) R[he[u]] = fma(-a, fma(bt, hs[u], hw[u]), hr[u]);
+    for (int u = 0; u < kRsHB; ++u) {
+      hn[u] = ho[u] >= 0 ? fma(-a, fma(bt, hs[u], hw[u]), hr[u]) : 0.0;
+      mag = max(mag, fx_mag(hn[u]));
+    }
     for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
       int e, gi, gj, gk;
       shell_node(h, e, gi, gj, gk);
@@ -367,28 +528,14 @@ __global__ void __launch_bounds__(kRsThreads)
         const long long o = gi + gj * g.sy + (long long)gk * g.sz;
         rn = fma(-a, fma(bt, __ldcg(Sg + o), __ldcg(Wg + o)), __ldcg(Rg + o));
       }
-      R[e] = rn;
+      RI[e] = __double_as_longlong(rn);
+      mag = max(mag, fx_mag(rn));
     }
-    __syncthreads();
     // 3. w = A r, gamma, delta; publish w
-    double acc_g = 0.0;
-    acc_d = 0.0;
-    for (int q = threadIdx.x; q < B; q += kRsThreads) {
-      const Own n = node_of(q);
-      double w = 0.0;
-      if (n.valid) {
-        const double r = R[n.e];
-        w = rs_stencil(R + n.e, EX, EX * EY, A, shallow);
-        acc_g = fma(r, r, acc_g);
-        acc_d = fma(w, r, acc_d);
-        __stcg(Wn + n.o, w);
-      }
-      W[q] = w;
-    }
+    part = apply(fill(mag, hn), Wn);
     // 4. the grid reduction (it also orders every block's publications before the next
     // step's halo loads); the next halo's loads; scalars
-    const double2 part = rs_block_sum2(acc_g, acc_d, s_park, nw_own);
-    const bool ok = rs_arrive_wait(part, pairs, counter, G, seq, err, &s_ok);
+    const bool ok = rs_arrive_wait(part, parts, counter, G, seq, err, &s_ok);
     par ^= 1;
     if (ok) load_halo(par);
     if (threadIdx.x < 32) {
@@ -397,7 +544,7 @@ __global__ void __launch_bounds__(kRsThreads)
         status = EXCMG_ERR_TIMEOUT;
         stop = 1;
       } else {
-        const double2 red = rs_read_pairs(pairs, G, seq);
+        const double2 red = rs_read_parts(parts, G, seq);
         const double gn = red.x, dn = red.y;
         iter += 1;
         if (b == 0 && lane == 0 && D.hist && iter < D.hist_len) D.hist[iter] = gn;
@@ -436,12 +583,10 @@ __global__ void __launch_bounds__(kRsThreads)
     __syncthreads();
   }
   // x and the last r of the box
-  for (int q = threadIdx.x; q < B; q += kRsThreads) {
-    const Own n = own_node(q);
-    if (!n.valid) continue;
-    D.x[n.o] = X[q];
-    D.r[n.o] = R[n.e];
-  }
+  each([&](const Own& n, double& r, double& x, double&, double&, double&) {
+    D.x[n.o] = x;
+    D.r[n.o] = r;
+  });
   if (b == 0 && threadIdx.x == 0) {
     S->rr = gam;
     S->pq = delta;
@@ -461,12 +606,12 @@ size_t g_rs_max_smem = 0;
 }  // namespace
 
 size_t resident_smem(int bx, int by, int bz) {
-  const size_t ext = (size_t)(bx + 2) * (by + 2) * (bz + 2);
-  return sizeof(double) * (ext + 4 * (size_t)bx * by * bz);
+  const size_t ext = (size_t)(bx + 2) * (by + 2) * (bz + 2), nodes = (size_t)bx * by * bz;
+  return sizeof(double) * (ext + (nodes > kRsThreads ? 5 * nodes : 0));
 }
 
 #ifndef EXCMG_RESIDENT_MAX_SMEM
-#define EXCMG_RESIDENT_MAX_SMEM (96 * 1024)
+#define EXCMG_RESIDENT_MAX_SMEM (107 * 1024)  // two blocks of an SM, with 5 KB each of their own
 #endif
 
 bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem) {
@@ -478,9 +623,9 @@ bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem) {
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     g_rs_max_smem = std::min<size_t>(EXCMG_RESIDENT_MAX_SMEM, (size_t)std::max(0, optin - 2048));
     if (!coop || g_rs_sms <= 0 ||
-        cudaFuncSetAttribute(k_cg_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_cg_resident<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)g_rs_max_smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_rs_blocks_per_sm, k_cg_resident, kRsThreads,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_rs_blocks_per_sm, k_cg_resident<false>, kRsThreads,
                                                       g_rs_max_smem) != cudaSuccess) {
       cudaGetLastError();
       g_rs_blocks_per_sm = 0;
@@ -490,7 +635,8 @@ bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem) {
   if (g_rs_blocks_per_sm <= 0) return false;
   const int ni = g.nx - 1, nj = g.ny - 1, nk = g.nz - 1;
   if (ni < 1 || nj < 1 || nk < 1) return false;
-  const long long max_blocks = std::min<long long>((long long)g_rs_sms * g_rs_blocks_per_sm, kMaxGrid);
+  // (two sets of 32-byte block sums, kRsPB per lane of a warp)
+  const long long max_blocks = std::min<long long>((long long)g_rs_sms * g_rs_blocks_per_sm, 32 * kRsPB);
   // per-step model in SM clocks: the busiest SM's float64 work (~12.5 clocks per node,
   // 2 DFMA per clock, plus ~400 per block for its reduction), the halo loads of a box
   // (3 per shell node), and the grid reduction's share per block (arrival, partials)
@@ -525,12 +671,13 @@ bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem) {
   return found;
 }
 
-cudaError_t launch_cg_resident(const ResidentDesc& D, size_t smem, CGState* st, double2* pairs,
+cudaError_t launch_cg_resident(const ResidentDesc& D, size_t smem, CGState* st, void* parts,
                                unsigned* counter, int* err, cudaStream_t s) {
   const int grid = D.nbx * D.nby * D.nbz;
   ResidentDesc d = D;
-  void* args[] = {(void*)&d, (void*)&st, (void*)&pairs, (void*)&counter, (void*)&err};
-  return cudaLaunchCooperativeKernel((const void*)k_cg_resident, dim3(grid), dim3(kRsThreads), args,
+  void* args[] = {(void*)&d, (void*)&st, (void*)&parts, (void*)&counter, (void*)&err};
+  const bool one = D.bx * D.by * D.bz <= kRsThreads;
+  return cudaLaunchCooperativeKernel(one ? (const void*)k_cg_resident<true> : (const void*)k_cg_resident<false>, dim3(grid), dim3(kRsThreads), args,
                                      smem, s);
 }
 
