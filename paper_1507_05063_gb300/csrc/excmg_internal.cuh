@@ -285,7 +285,7 @@ struct ResidentDesc {
 // Chooses the boxes for grid g; false if the grid does not fit or the device has no
 // cooperative launch.  smem: dynamic shared memory per block.
 bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem);
-// parts: 2 G block sums of 32 bytes (G = nbx nby nbz <= 320); counter, err: zeroed.
+// parts: 2 G block sums of 32 bytes (G = nbx nby nbz <= 512); counter, err: zeroed.
 cudaError_t launch_cg_resident(const ResidentDesc& D, size_t smem, CGState* st, void* parts,
                                unsigned* counter, int* err, cudaStream_t s);
 

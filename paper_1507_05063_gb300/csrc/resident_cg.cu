@@ -18,9 +18,17 @@
 // and w of its box into node arrays of the level (two copies by step parity), and the
 // next step recomputes the new r on its halo from its neighbours' published r, w, s with
 // the same fused operations as the owner (bit-identical).  So one step needs one grid-wide
-// synchronisation, the reduction's: per-block partials, one arrival counter (release /
-// acquire, bounded wait: EXCMG_ERR_TIMEOUT), then every block adds the G partials in
-// index order, so all blocks hold bit-identical scalars and take the same decisions.
+// synchronisation, the reduction's: per-block sums, one arrival counter (release /
+// acquire, bounded wait: EXCMG_ERR_TIMEOUT), then every block adds the G blocks' sums, so
+// all blocks hold bit-identical scalars and take the same decisions.
+//
+// What bounds a step: the chain of its parts on the smallest levels, the FP64 pipe on the
+// largest.  A float64 warp instruction takes the pipe 64 clocks whatever its lanes do, so
+// the 19-point sums (fixed_point.cuh) and the reductions run on integers, and float64 is
+// left with the vector updates, the two products and the scalars: 8.5 instructions per node
+// and step instead of 25.  Measured per step, before and after: 16^3 cells 6.1 us, 3.8;
+// 32^3 7.3, 4.5; 64^3 21.9, 10.2; 128 x 128 x 32 36.4, 17.4.  The blocks' sums are read by
+// all warps (one or two per thread): read by one warp, ten per lane, they cost 1.5 us more.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,7 +42,6 @@ namespace {
 constexpr int kRsThreads = 256;
 constexpr unsigned long long kRsSpinLimit = 1ull << 25;
 constexpr int kRsHB = 6;  // halo nodes per thread whose loads are issued ahead
-constexpr int kRsPB = 10;  // block sums per lane: up to 320 blocks
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
@@ -120,12 +127,8 @@ __device__ __forceinline__ long long rs_round(long long v, int n) {
   return (v + ((1LL << n) >> 1)) >> n;
 }
 
-// v 2^e as float64.
-__device__ __forceinline__ double rs_double(long long v, int e) {
-  const double x = (double)v;
-  const int h = e / 2;
-  return x * fx_pow2(h) * fx_pow2(e - h);
-}
+// v 2^e as float64, |v| < 2^63 and |e| <= 900 (what the blocks' scales allow).
+__device__ __forceinline__ double rs_double(long long v, int e) { return fx_scale((double)v, e); }
 
 // Reduction number `seq` (1, 2, ...): thread 0 stores this block's sums as part b of
 // the set seq & 1 (two sets: a block can be one reduction ahead of another's reads, never
@@ -157,52 +160,71 @@ __device__ bool rs_arrive_wait(const RsPart& part, RsPart* parts, unsigned* coun
   return *s_ok != 0;
 }
 
-// Warp 0, after the wait: the sums of the G parts of set seq & 1, identical in every lane and
-// every block: the parts brought to the largest exponent (nine bits above it for up to 512
-// parts) and added as integers, or, where a part is float64, all as float64 in a fixed order.
-__device__ double2 rs_read_parts(const RsPart* parts, int G, unsigned seq) {
-  const int4* set = reinterpret_cast<const int4*>(parts + (size_t)(seq & 1) * G);
-  const int lane = threadIdx.x & 31;
-  RsPart v[kRsPB];
-  int mg = -kRsRaw, md = -kRsRaw;
-  bool raw = false;
+// The sum of a part per lane (eg = -kRsRaw: none), identical in every lane: the parts brought
+// to the largest exponent and added as integers (`bits`: log2 of the terms of a lane plus 5),
+// or, where one is float64, all as float64 in a fixed order.  v: two parts per lane.
+__device__ __forceinline__ RsPart rs_warp_parts(const RsPart (&v)[2], int bits) {
+  RsPart t;
+  t.pad = 0;
+  const bool raw = v[0].eg == kRsRaw || v[1].eg == kRsRaw;
+  if (__any_sync(0xffffffffu, raw)) {
+    double g = 0.0, d = 0.0;
 #pragma unroll
-  for (int u = 0; u < kRsPB; ++u) {
-    const int i = lane + 32 * u;
-    v[u].g = v[u].d = 0;
-    v[u].eg = v[u].ed = -kRsRaw;
+    for (int u = 0; u < 2; ++u) {
+      if (v[u].eg == -kRsRaw) continue;
+      const bool f = v[u].eg == kRsRaw;
+      g += f ? __longlong_as_double(v[u].g) : rs_double(v[u].g, v[u].eg);
+      d += f ? __longlong_as_double(v[u].d) : rs_double(v[u].d, v[u].ed);
+    }
+    t.g = __double_as_longlong(rs_xor_sum(g, 16));
+    t.d = __double_as_longlong(rs_xor_sum(d, 16));
+    t.eg = t.ed = kRsRaw;
+    return t;
+  }
+  const int mg = __reduce_max_sync(0xffffffffu, max(v[0].eg, v[1].eg));
+  const int md = __reduce_max_sync(0xffffffffu, max(v[0].ed, v[1].ed));
+  t.g = rs_warp_sum(rs_round(v[0].g, mg - v[0].eg + bits) + rs_round(v[1].g, mg - v[1].eg + bits));
+  t.d = rs_warp_sum(rs_round(v[0].d, md - v[0].ed + bits) + rs_round(v[1].d, md - v[1].ed + bits));
+  t.eg = mg == -kRsRaw ? mg : mg + bits;
+  t.ed = md == -kRsRaw ? md : md + bits;
+  return t;
+}
+
+__device__ __forceinline__ RsPart rs_no_part() {
+  RsPart t;
+  t.g = t.d = t.pad = 0;
+  t.eg = t.ed = -kRsRaw;
+  return t;
+}
+
+// After the wait, every warp: the sum of its share of the G parts of set seq & 1 into
+// s_warp (then a block barrier).
+__device__ __forceinline__ void rs_read_parts(const RsPart* parts, int G, unsigned seq, RsPart* s_warp) {
+  const int4* set = reinterpret_cast<const int4*>(parts + (size_t)(seq & 1) * G);
+  RsPart v[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int i = threadIdx.x + u * kRsThreads;
+    v[u] = rs_no_part();
     if (i < G) {
       reinterpret_cast<int4*>(&v[u])[0] = __ldcg(set + 2 * i);
       reinterpret_cast<int4*>(&v[u])[1] = __ldcg(set + 2 * i + 1);
     }
   }
-#pragma unroll
-  for (int u = 0; u < kRsPB; ++u) {
-    raw = raw || v[u].eg == kRsRaw;
-    mg = max(mg, v[u].eg);
-    md = max(md, v[u].ed);
-  }
-  if (__any_sync(0xffffffffu, raw)) {
-    double g = 0.0, d = 0.0;
-#pragma unroll
-    for (int u = 0; u < kRsPB; ++u) {
-      if (lane + 32 * u >= G) break;
-      const bool f = v[u].eg == kRsRaw;
-      g += f ? __longlong_as_double(v[u].g) : rs_double(v[u].g, v[u].eg);
-      d += f ? __longlong_as_double(v[u].d) : rs_double(v[u].d, v[u].ed);
-    }
-    return make_double2(rs_xor_sum(g, 16), rs_xor_sum(d, 16));
-  }
-  mg = __reduce_max_sync(0xffffffffu, mg);
-  md = __reduce_max_sync(0xffffffffu, md);
-  long long g = 0, d = 0;
-#pragma unroll
-  for (int u = 0; u < kRsPB; ++u) {
-    g += rs_round(v[u].g, mg - v[u].eg + 9);
-    d += rs_round(v[u].d, md - v[u].ed + 9);
-  }
-  // |sum over a lane's parts| < 2^(62 - 9 + 4)
-  return make_double2(rs_double(rs_warp_sum(g), mg + 9), rs_double(rs_warp_sum(d), md + 9));
+  const RsPart t = rs_warp_parts(v, 6);
+  if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = t;
+}
+
+// Warp 0, after that barrier: the sums, identical in every lane and every block.
+__device__ __forceinline__ double2 rs_sums(const RsPart* s_warp) {
+  const int lane = threadIdx.x & 31;
+  RsPart v[2] = {rs_no_part(), rs_no_part()};
+  if (lane < kRsThreads / 32) v[0] = s_warp[lane];
+  const RsPart t = rs_warp_parts(v, 5);
+  if (t.eg == kRsRaw) return make_double2(__longlong_as_double(t.g), __longlong_as_double(t.d));
+  // both conversions in one warp instruction
+  const double x = rs_double(lane == 0 ? t.g : t.d, lane == 0 ? t.eg : t.ed);
+  return make_double2(__shfl_sync(0xffffffffu, x, 0), __shfl_sync(0xffffffffu, x, 1));
 }
 
 // 19-point A-stencil at offset 0 of P with strides (1, ey, ez).  `shallow`: the seven
@@ -242,6 +264,7 @@ __global__ void __launch_bounds__(kRsThreads, 2)
   __shared__ double s_park[2 * kRsThreads];
   __shared__ uint4 s_mag[kRsThreads / 128];
   __shared__ long long s_sum[2][kRsThreads / 32];
+  __shared__ RsPart s_warp[kRsThreads / 32];
   __shared__ int s_ok;
   __shared__ double s_alpha, s_beta;
   __shared__ int s_stop;
@@ -274,8 +297,9 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     bool valid;
     long long o;
   };
+  const int sx = 31 - __clz(BX), sxy = sx + 31 - __clz(BY);  // box extents are powers of two
   auto own_node = [&](int q) -> Own {
-    const int lx = q % BX, ly = (q / BX) % BY, lz = q / (BX * BY);
+    const int lx = q & (BX - 1), ly = (q >> sx) & (BY - 1), lz = q >> sxy;
     const int gi = i0 + lx, gj = j0 + ly, gk = k0 + lz;
     Own w;
     w.e = (lx + 1) + EX * ((ly + 1) + EY * (lz + 1));
@@ -332,6 +356,8 @@ __global__ void __launch_bounds__(kRsThreads, 2)
   };
   // this thread's shell nodes (index in RI, offset in the level's arrays or -1 outside the
   // interior), computed once: after each wait the loads issue at once
+  // (the slots past `slots` hold none)
+  const int slots = min(kRsHB, (nshell + kRsThreads - 1) / kRsThreads);
   int he[kRsHB], ho[kRsHB];
 #pragma unroll
   for (int u = 0; u < kRsHB; ++u) {
@@ -360,8 +386,10 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     auto put = [&](double v) { return E < 0 ? __double_as_longlong(v) : fx_from_double<kFxBits>(v, E); };
     each([&](const Own& n, double& r, double&, double&, double&, double&) { RI[n.e] = put(r); });
 #pragma unroll
-    for (int u = 0; u < kRsHB; ++u)
+    for (int u = 0; u < kRsHB; ++u) {
+      if (u >= slots) break;
       if (he[u] >= 0) RI[he[u]] = put(hn[u]);
+    }
     for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
       int e, gi, gj, gk;
       shell_node(h, e, gi, gj, gk);
@@ -464,14 +492,18 @@ __global__ void __launch_bounds__(kRsThreads, 2)
   unsigned seq = 1;
   {
     const bool ok = rs_arrive_wait(part, parts, counter, G, seq, err, &s_ok);
-    if (ok) load_halo(0);
+    if (ok) {
+      load_halo(0);
+      rs_read_parts(parts, G, seq, s_warp);
+    }
+    __syncthreads();
     if (threadIdx.x < 32) {
       int stop = 0;
       if (!ok) {
         status = EXCMG_ERR_TIMEOUT;
         stop = 1;
       } else {
-        delta = rs_read_parts(parts, G, seq).y;
+        delta = rs_sums(s_warp).y;
         if (delta == 0.0 && gam == 0.0) {
           stop = 1;  // exact solution (fixed-count mode)
         } else if (!(delta > 0.0) || !isfinite(delta)) {
@@ -517,7 +549,8 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     double hn[kRsHB];
 #pragma unroll
     for (int u = 0; u < kRsHB; ++u) {
-      hn[u] = ho[u] >= 0 ? fma(-a, fma(bt, hs[u], hw[u]), hr[u]) : 0.0;
+      if (u >= slots) break;  // (a float64 instruction takes its 64 clocks with every lane predicated off too)
+      hn[u] = fma(-a, fma(bt, hs[u], hw[u]), hr[u]);  // 0 where there is no node: hr, hw, hs are
       mag = max(mag, fx_mag(hn[u]));
     }
     for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
@@ -537,14 +570,18 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     // step's halo loads); the next halo's loads; scalars
     const bool ok = rs_arrive_wait(part, parts, counter, G, seq, err, &s_ok);
     par ^= 1;
-    if (ok) load_halo(par);
+    if (ok) {
+      rs_read_parts(parts, G, seq, s_warp);
+      load_halo(par);
+    }
+    __syncthreads();
     if (threadIdx.x < 32) {
       int stop = 0;
       if (!ok) {
         status = EXCMG_ERR_TIMEOUT;
         stop = 1;
       } else {
-        const double2 red = rs_read_parts(parts, G, seq);
+        const double2 red = rs_sums(s_warp);
         const double gn = red.x, dn = red.y;
         iter += 1;
         if (b == 0 && lane == 0 && D.hist && iter < D.hist_len) D.hist[iter] = gn;
@@ -635,8 +672,8 @@ bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem) {
   if (g_rs_blocks_per_sm <= 0) return false;
   const int ni = g.nx - 1, nj = g.ny - 1, nk = g.nz - 1;
   if (ni < 1 || nj < 1 || nk < 1) return false;
-  // (two sets of 32-byte block sums, kRsPB per lane of a warp)
-  const long long max_blocks = std::min<long long>((long long)g_rs_sms * g_rs_blocks_per_sm, 32 * kRsPB);
+  // (a block reads at most two sums per thread)
+  const long long max_blocks = std::min<long long>((long long)g_rs_sms * g_rs_blocks_per_sm, 2 * kRsThreads);
   // per-step model in SM clocks: the busiest SM's float64 work (~12.5 clocks per node,
   // 2 DFMA per clock, plus ~400 per block for its reduction), the halo loads of a box
   // (3 per shell node), and the grid reduction's share per block (arrival, partials)
