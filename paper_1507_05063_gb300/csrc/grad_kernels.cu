@@ -21,25 +21,35 @@ namespace excmg {
 namespace {
 
 constexpr int kTab = 64;
+// threads of a strided-line block: two warps, so that a grid's lines spread evenly over the
+// SMs (blocks of 256 left 258 on 152 SMs at 512 x 256 x 256: a second round 70% empty)
+constexpr int kLineThreads = 64;
 constexpr int kAhead = 8;  // line steps whose loads are in flight together (strided lines)
 
 // The factors of the forward sweep written as dp_t = (u_{i+1} - u_{i-1}) A_t + B_t dp_{t-1}
 // (A_t = (1/(2h)) / m_t, B_t = -(1/6) / m_t; the first step's dp_{t-1} is D_0, the
 // last one's carries + D_N: the boundary derivatives moved to the right-hand side), and
-// c'_t of the back substitution.
-__device__ void thomas_table(double* cp, double* A, double* B, int n, double i2h) {
-  // a = c = 1/6, b = 4/6
-  const double a = 1.0 / 6.0, c = 1.0 / 6.0, b = 4.0 / 6.0;
+// c'_t of the back substitution; entries past the line's unknowns are not used.  Formed on
+// the host and passed with the launch: in the kernel one thread's 64 dependent float64
+// divisions took as long as a block's lines (the x-line kernel 7.3 float64 instructions per
+// node instead of 4).
+struct ThomasTable {
+  double cp[kTab], A[kTab], B[kTab];
+};
+
+ThomasTable thomas_table(double h) {
+  const double a = 1.0 / 6.0, c = 1.0 / 6.0, b = 4.0 / 6.0, i2h = 0.5 / h;
+  ThomasTable T;
   double prev = 0.0;
-  const int m = n < kTab ? n : kTab;
-  for (int t = 0; t < m; ++t) {
-    const double piv = (t == 0) ? b : b - a * prev;
+  for (int t = 0; t < kTab; ++t) {
+    const double piv = t == 0 ? b : fma(-a, prev, b);
     const double im = 1.0 / piv;
-    A[t] = i2h * im;
-    B[t] = -a * im;
-    cp[t] = c / piv;
-    prev = cp[t];
+    T.A[t] = i2h * im;
+    T.B[t] = -a * im;
+    T.cp[t] = c / piv;
+    prev = T.cp[t];
   }
+  return T;
 }
 
 __device__ __forceinline__ double d_left(double u0, double u1, double u2, double u3, double u4, double ih) {
@@ -55,12 +65,17 @@ __device__ __forceinline__ double d_right(double uN, double u1, double u2, doubl
 // the dependent FP64 operations of one overlap the other's (each step of the forward
 // sweep is a product and an FMA on the previous step's value); neighbouring threads
 // still take neighbouring a, so every step stays a coalesced row access.
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kLineThreads)
     k_grad_strided(const double* __restrict__ u, double* __restrict__ out, int N, double h,
-                   long long step, int na, int nb, long long sa, long long sb) {
+                   long long step, int na, int nb, long long sa, long long sb,
+             const __grid_constant__ ThomasTable T) {
   __shared__ double cp[kTab], A[kTab], B[kTab];
-  const double ih = 1.0 / h, i2h = 0.5 / h;
-  if (threadIdx.x == 0) thomas_table(cp, A, B, N - 1, i2h);
+  const double ih = 1.0 / h;
+  for (int t = threadIdx.x; t < kTab; t += kLineThreads) {
+    cp[t] = T.cp[t];
+    A[t] = T.A[t];
+    B[t] = T.B[t];
+  }
   __syncthreads();
   const long long nl = (long long)na * nb, half = (nl + 1) / 2;
   for (long long L = blockIdx.x * (long long)blockDim.x + threadIdx.x; L < half;
@@ -90,10 +105,6 @@ __global__ void __launch_bounds__(kThreads)
     double um1 = U1[0], uc1 = U1[step], dp1 = a1;
     auto fstep = [&](int i, double up0, double up1) {
       const int t = i - 1 < kTab ? i - 1 : kTab - 1;
-      if (i == N - 1) {
-        dp0 += n0;
-        dp1 += n1;
-      }
       dp0 = fma(B[t], dp0, (up0 - um0) * A[t]);
       dp1 = fma(B[t], dp1, (up1 - um1) * A[t]);
       D0p[(long long)i * step] = dp0;
@@ -104,7 +115,7 @@ __global__ void __launch_bounds__(kThreads)
       uc1 = up1;
     };
     int i = 1;
-    for (; i + kAhead - 1 <= N - 1; i += kAhead) {
+    for (; i + kAhead - 1 <= N - 2; i += kAhead) {
       double q0[kAhead], q1[kAhead];
 #pragma unroll
       for (int k = 0; k < kAhead; ++k) {
@@ -115,10 +126,15 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
       for (int k = 0; k < kAhead; ++k) fstep(i + k, q0[k], q1[k]);
     }
-    for (; i <= N - 1; ++i) {
+    for (; i <= N - 2; ++i) {
       const long long o = (long long)(i + 1) * step;
       fstep(i, U0[o], U1[o]);
     }
+    // the last step carries the far boundary derivative (outside the loop: a predicated
+    // float64 add takes its turn on the pipe in every step)
+    dp0 += n0;
+    dp1 += n1;
+    fstep(N - 1, U0[N * step], U1[N * step]);
     // back substitution, likewise kAhead nodes' loads at a time
     double x0 = dp0, x1 = dp1;
     auto bstep = [&](int i, double d0, double d1) {
@@ -192,11 +208,16 @@ __device__ __forceinline__ void unstage_rows(double (*tile)[35], double* dst, lo
 // x-nodes staged through shared memory.
 __global__ void __launch_bounds__(32)
     k_grad_x(const double* __restrict__ u, double* __restrict__ out, int N, double h,
-             long long nlines) {
+             long long nlines,
+             const __grid_constant__ ThomasTable T) {
   __shared__ double cp[kTab], A[kTab], B[kTab];
   __shared__ double tile[32][35];  // [line][x0-1 .. x0+32]
-  const double ih = 1.0 / h, i2h = 0.5 / h;
-  if (threadIdx.x == 0) thomas_table(cp, A, B, N - 1, i2h);
+  const double ih = 1.0 / h;
+  for (int t = threadIdx.x; t < kTab; t += 32) {
+    cp[t] = T.cp[t];
+    A[t] = T.A[t];
+    B[t] = T.B[t];
+  }
   __syncwarp();
   const int lane = threadIdx.x;
   const long long stride = N + 1;
@@ -219,12 +240,16 @@ __global__ void __launch_bounds__(32)
       stage_rows(tile, u, L0, nlines, stride, x0 - 1, cnt + 2, lane);
       __syncwarp();
       if (mine) {
-        for (int c = 0; c < cnt; ++c) {
-          const int i = x0 + c;
-          const int t = i - 1 < kTab ? i - 1 : kTab - 1;
-          if (i == N - 1) dp += DN;
+        auto step = [&](int c) {
+          const int t = x0 + c - 1 < kTab ? x0 + c - 1 : kTab - 1;
           dp = fma(B[t], dp, (tile[lane][c + 2] - tile[lane][c]) * A[t]);
           tile[lane][c] = dp;
+        };
+        const bool end = x0 + cnt == N;  // the last step carries the far boundary derivative
+        for (int c = 0; c < cnt - end; ++c) step(c);
+        if (end) {
+          dp += DN;
+          step(cnt - 1);
         }
       }
       __syncwarp();
@@ -240,15 +265,12 @@ __global__ void __launch_bounds__(32)
       stage_rows(tile, out, L0, nlines, stride, xs, cnt, lane);
       __syncwarp();
       if (mine) {
-        for (int c = cnt - 1; c >= 0; --c) {
+        int c = cnt - 1;
+        if (last) xv = tile[lane][c--];  // x_{N-1} = dp_{N-1}
+        for (; c >= 0; --c) {
           const int i = xs + c;
-          if (last) {
-            xv = tile[lane][c];  // x_{N-1} = dp_{N-1}
-            last = false;
-          } else {
-            const int t = i - 1 < kTab ? i - 1 : kTab - 1;
-            xv = tile[lane][c] - cp[t] * xv;
-          }
+          const int t = i - 1 < kTab ? i - 1 : kTab - 1;
+          xv = tile[lane][c] - cp[t] * xv;
           tile[lane][c] = xv;
         }
       }
@@ -261,7 +283,7 @@ __global__ void __launch_bounds__(32)
 
 int grid_for(long long items, int per_block) {
   long long b = (items + per_block - 1) / per_block;
-  if (b > 152 * 32) b = 152 * 32;
+  if (b > 152 * 64) b = 152 * 64;
   return b < 1 ? 1 : (int)b;
 }
 
@@ -270,13 +292,13 @@ int grid_for(long long items, int per_block) {
 cudaError_t launch_grad(const Grid3& g, const double* u, double* ux, double* uy, double* uz,
                         cudaStream_t s) {
   const long long nlx = (long long)(g.ny + 1) * (g.nz + 1);
-  k_grad_x<<<grid_for(nlx, 32), 32, 0, s>>>(u, ux, g.nx, g.hx, nlx);
+  k_grad_x<<<grid_for(nlx, 32), 32, 0, s>>>(u, ux, g.nx, g.hx, nlx, thomas_table(g.hx));
   // y-lines: a = i (fastest), b = k; two lines per thread
-  k_grad_strided<<<grid_for(((long long)(g.nx + 1) * (g.nz + 1) + 1) / 2, kThreads), kThreads, 0, s>>>(
-      u, uy, g.ny, g.hy, g.sy, g.nx + 1, g.nz + 1, 1, g.sz);
+  k_grad_strided<<<grid_for(((long long)(g.nx + 1) * (g.nz + 1) + 1) / 2, kLineThreads), kLineThreads, 0, s>>>(
+      u, uy, g.ny, g.hy, g.sy, g.nx + 1, g.nz + 1, 1, g.sz, thomas_table(g.hy));
   // z-lines: a = i + sy*j flattened (fastest), b unused
-  k_grad_strided<<<grid_for((g.sz + 1) / 2, kThreads), kThreads, 0, s>>>(u, uz, g.nz, g.hz, g.sz,
-                                                                        (int)g.sz, 1, 1, 0);
+  k_grad_strided<<<grid_for((g.sz + 1) / 2, kLineThreads), kLineThreads, 0, s>>>(u, uz, g.nz, g.hz, g.sz,
+                                                                        (int)g.sz, 1, 1, 0, thomas_table(g.hz));
   return cudaGetLastError();
 }
 
