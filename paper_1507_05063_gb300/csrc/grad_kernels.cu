@@ -14,6 +14,8 @@
 // chunks of the lines through shared memory so that global accesses stay coalesced.
 #include <math.h>
 
+#include <algorithm>
+
 #include "excmg_internal.cuh"
 
 namespace excmg {
@@ -24,7 +26,10 @@ constexpr int kTab = 64;
 // threads of a strided-line block: two warps, so that a grid's lines spread evenly over the
 // SMs (blocks of 256 left 258 on 152 SMs at 512 x 256 x 256: a second round 70% empty)
 constexpr int kLineThreads = 64;
-constexpr int kAhead = 8;  // line steps whose loads are in flight together (strided lines)
+constexpr int kAhead = 4;  // line steps whose loads are in flight together (strided lines)
+// resident blocks per SM (80 registers): 512 x 256 x 256 takes 1015 us with 11 blocks and 4
+// steps ahead; 9 blocks and 4 ahead 1027, 11 and 6 1035, 11 and 8 1034, 9 and 8 1071
+constexpr int kLineBlocks = 11;
 
 // The factors of the forward sweep written as dp_t = (u_{i+1} - u_{i-1}) A_t + B_t dp_{t-1}
 // (A_t = (1/(2h)) / m_t, B_t = -(1/6) / m_t; the first step's dp_{t-1} is D_0, the
@@ -65,21 +70,12 @@ __device__ __forceinline__ double d_right(double uN, double u1, double u2, doubl
 // the dependent FP64 operations of one overlap the other's (each step of the forward
 // sweep is a product and an FMA on the previous step's value); neighbouring threads
 // still take neighbouring a, so every step stays a coalesced row access.
-__global__ void __launch_bounds__(kLineThreads)
-    k_grad_strided(const double* __restrict__ u, double* __restrict__ out, int N, double h,
-                   long long step, int na, int nb, long long sa, long long sb,
-             const __grid_constant__ ThomasTable T) {
-  __shared__ double cp[kTab], A[kTab], B[kTab];
+__device__ __forceinline__ void strided_lines(const double* __restrict__ u, double* __restrict__ out, int N, double h,
+                                              long long step, int na, int nb, long long sa, long long sb,
+                                              const double* cp, const double* A, const double* B, int block, int blocks) {
   const double ih = 1.0 / h;
-  for (int t = threadIdx.x; t < kTab; t += kLineThreads) {
-    cp[t] = T.cp[t];
-    A[t] = T.A[t];
-    B[t] = T.B[t];
-  }
-  __syncthreads();
   const long long nl = (long long)na * nb, half = (nl + 1) / 2;
-  for (long long L = blockIdx.x * (long long)blockDim.x + threadIdx.x; L < half;
-       L += (long long)gridDim.x * blockDim.x) {
+  for (long long L = (long long)block * kLineThreads + threadIdx.x; L < half; L += (long long)blocks * kLineThreads) {
     const bool two = L + half < nl;
     const long long L1 = two ? L + half : L;  // the second line (a copy of the first if none)
     const double* __restrict__ U0 = u + (L % na) * sa + (L / na) * sb;
@@ -205,23 +201,14 @@ __device__ __forceinline__ void unstage_rows(double (*tile)[35], double* dst, lo
 }
 
 // x-lines: one warp handles 32 consecutive lines (line = j + (ny+1) k), chunks of 32
-// x-nodes staged through shared memory.
-__global__ void __launch_bounds__(32)
-    k_grad_x(const double* __restrict__ u, double* __restrict__ out, int N, double h,
-             long long nlines,
-             const __grid_constant__ ThomasTable T) {
-  __shared__ double cp[kTab], A[kTab], B[kTab];
-  __shared__ double tile[32][35];  // [line][x0-1 .. x0+32]
+// x-nodes staged through shared memory (tile: the warp's own).
+__device__ __forceinline__ void x_lines(const double* __restrict__ u, double* __restrict__ out, int N, double h,
+                                        long long nlines, const double* cp, const double* A, const double* B,
+                                        double (*tile)[35], int warp, int warps) {
   const double ih = 1.0 / h;
-  for (int t = threadIdx.x; t < kTab; t += 32) {
-    cp[t] = T.cp[t];
-    A[t] = T.A[t];
-    B[t] = T.B[t];
-  }
-  __syncwarp();
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31;
   const long long stride = N + 1;
-  for (long long L0 = (long long)blockIdx.x * 32; L0 < nlines; L0 += (long long)gridDim.x * 32) {
+  for (long long L0 = (long long)warp * 32; L0 < nlines; L0 += (long long)warps * 32) {
     const long long L = L0 + lane;
     const bool mine = L < nlines;
     double D0 = 0.0, DN = 0.0;
@@ -281,24 +268,71 @@ __global__ void __launch_bounds__(32)
   }
 }
 
-int grid_for(long long items, int per_block) {
-  long long b = (items + per_block - 1) / per_block;
-  if (b > 152 * 64) b = 152 * 64;
-  return b < 1 ? 1 : (int)b;
+// The three directions in one launch: a block takes lines of one direction, and the
+// directions alternate from block to block, so that each one's waits (loads, and the x-lines'
+// staging) are covered by the others' float64 work.  Bound by the float64 pipe (2 lanes per
+// clock and SM on this chip; 12.9 operations per node and the three directions, the pipe 72%
+// busy at 512 x 256 x 256).  That grid: 1015 us; as three launches 1036 us; with the factors
+// made by each block and 256-thread blocks as well 1470 us.
+struct GradDir {
+  ThomasTable T;
+  int blocks;
+};
+
+__global__ void __launch_bounds__(kLineThreads, kLineBlocks)
+    k_grad(const Grid3 g, const double* __restrict__ u, double* __restrict__ ux, double* __restrict__ uy,
+           double* __restrict__ uz, const __grid_constant__ GradDir X, const __grid_constant__ GradDir Y,
+           const __grid_constant__ GradDir Z) {
+  __shared__ double cp[kTab], A[kTab], B[kTab];
+  __shared__ double tile[kLineThreads / 32][32][35];  // [warp][line][x0-1 .. x0+32]
+  // direction and block within it: in turn while all three have blocks, then the rest
+  const int m = min(X.blocks, min(Y.blocks, Z.blocks));
+  int dir = blockIdx.x % 3, b = blockIdx.x / 3;
+  if (b >= m) {
+    b = blockIdx.x - 2 * m;  // m + the place among the rest
+    dir = 0;
+    if (b >= X.blocks) {
+      b -= X.blocks - m;
+      dir = 1;
+      if (b >= Y.blocks) {
+        b -= Y.blocks - m;
+        dir = 2;
+      }
+    }
+  }
+  const ThomasTable& T = dir == 0 ? X.T : dir == 1 ? Y.T : Z.T;
+  for (int t = threadIdx.x; t < kTab; t += kLineThreads) {
+    cp[t] = T.cp[t];
+    A[t] = T.A[t];
+    B[t] = T.B[t];
+  }
+  __syncthreads();
+  constexpr int kW = kLineThreads / 32;
+  if (dir == 0)
+    x_lines(u, ux, g.nx, g.hx, (long long)(g.ny + 1) * (g.nz + 1), cp, A, B, tile[threadIdx.x >> 5],
+            b * kW + (threadIdx.x >> 5), X.blocks * kW);
+  else if (dir == 1)  // a = i (fastest), b = k
+    strided_lines(u, uy, g.ny, g.hy, g.sy, g.nx + 1, g.nz + 1, 1, g.sz, cp, A, B, b, Y.blocks);
+  else  // a = i, b = j
+    strided_lines(u, uz, g.nz, g.hz, g.sz, g.nx + 1, g.ny + 1, 1, g.sy, cp, A, B, b, Z.blocks);
+}
+
+GradDir grad_dir(double h, long long items, int per_block) {
+  GradDir d;
+  d.T = thomas_table(h);
+  d.blocks = (int)std::max(1LL, std::min((items + per_block - 1) / per_block, 152LL * 64));
+  return d;
 }
 
 }  // namespace
 
 cudaError_t launch_grad(const Grid3& g, const double* u, double* ux, double* uy, double* uz,
                         cudaStream_t s) {
-  const long long nlx = (long long)(g.ny + 1) * (g.nz + 1);
-  k_grad_x<<<grid_for(nlx, 32), 32, 0, s>>>(u, ux, g.nx, g.hx, nlx, thomas_table(g.hx));
-  // y-lines: a = i (fastest), b = k; two lines per thread
-  k_grad_strided<<<grid_for(((long long)(g.nx + 1) * (g.nz + 1) + 1) / 2, kLineThreads), kLineThreads, 0, s>>>(
-      u, uy, g.ny, g.hy, g.sy, g.nx + 1, g.nz + 1, 1, g.sz, thomas_table(g.hy));
-  // z-lines: a = i + sy*j flattened (fastest), b unused
-  k_grad_strided<<<grid_for((g.sz + 1) / 2, kLineThreads), kLineThreads, 0, s>>>(u, uz, g.nz, g.hz, g.sz,
-                                                                        (int)g.sz, 1, 1, 0, thomas_table(g.hz));
+  const long long wx = g.nx + 1, wy = g.ny + 1, wz = g.nz + 1;
+  const GradDir X = grad_dir(g.hx, wy * wz, kLineThreads);
+  const GradDir Y = grad_dir(g.hy, (wx * wz + 1) / 2, kLineThreads);  // two lines per thread
+  const GradDir Z = grad_dir(g.hz, (wx * wy + 1) / 2, kLineThreads);
+  k_grad<<<X.blocks + Y.blocks + Z.blocks, kLineThreads, 0, s>>>(g, u, ux, uy, uz, X, Y, Z);
   return cudaGetLastError();
 }
 

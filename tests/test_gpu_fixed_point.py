@@ -182,3 +182,16 @@ def test_exp_true_tiles(X, N):
     got = X.exp_true(dev(uh), dev(u2), (1.0, 1.0, 1.0)).cpu().numpy()
     want = O.extrapolate_true(uh, u2)
     assert np.max(np.abs(got - want)) <= 30 * max(np.max(np.abs(uh)), np.max(np.abs(u2))) * 2.0 ** -53
+
+
+@pytest.mark.parametrize("N", [(4, 4, 4), (4, 5, 67), (33, 4, 6), (6, 131, 5), (31, 32, 33), (65, 34, 66)])
+def test_gradient_line_edges(X, N):
+    """All three directions from one launch: lengths about the groups of line steps (4), the
+    staged chunks of x-lines (32) and the factors' table (64), and unequal numbers of lines.
+    The compact system's inverse is below 3 and its right-hand sides below 3 U / h, so some
+    tens of rounded operations stay within 200 U / h 2^-53."""
+    L = (1.0, 0.7, 1.9)
+    u, _ = fields(N, 7)
+    h = O.meshsizes(L, N)
+    for got, want, hd in zip(X.grad(dev(u), L), O.gradient(u, h), h):
+        assert np.max(np.abs(got.cpu().numpy() - want)) <= 200 * np.max(np.abs(u)) / hd * 2.0 ** -53
