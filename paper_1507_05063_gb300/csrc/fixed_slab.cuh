@@ -2,9 +2,9 @@
 //
 // A slab is 32 x 8 columns of interior nodes, its first (1 + 32 a, 1 + 8 b), over tz planes
 // from 1 + tz c: a direction of 2^k cells (2^k - 1 interior nodes) has no ragged slab but
-// the last.  A block of 256 threads, one per column, marches it along z in groups of four
-// planes: a thread loads its 4 nodes of a group and at most 2 of the group's x- and y-halo,
-// the group is brought to one scale, stored as 64-bit integers in shared memory (11 KB) and
+// the last.  A block of 256 threads, one per column, marches it along z in groups of six
+// planes: a thread loads its 6 nodes of a group and at most 2 of the group's x- and y-halo,
+// the group is brought to one scale, stored as 64-bit integers in shared memory (16 KB) and
 // summed; the partial sums of the last planes stay in registers from group to group, so
 // nothing is loaded or converted twice along z but the slab's two halo planes.  Three blocks
 // of an SM (80 registers) cover each other's loads and barriers.  Measured slower: two rows
@@ -22,7 +22,11 @@ namespace excmg {
 namespace {
 
 constexpr int kFxX = kTX, kFxY = kThreads / 32;
-constexpr int kFxG = 4;  // planes per group
+// Planes per group: 84 rim nodes a plane go to 256 threads, so groups of 3 and 6 planes fill
+// the loads' rounds and others do not, and a deeper group has fewer barriers.  Residual at
+// 320 x 255 x 257 with 3 / 4 / 5 / 6 / 7 / 8 planes: 475 / 455 / 422 / 421 / 452 / 424 us; CG at
+// 385 x 201 x 121, 40 steps: 4.39 / 4.39 / 4.24 / 4.15 / 4.30 / 4.88 ms.
+constexpr int kFxG = 6;
 constexpr int kBoxX = kFxX + 2, kBoxY = kFxY + 2;
 constexpr int kPlane = kBoxX * kBoxY;
 constexpr int kOwn = kFxG;                                         // own nodes per thread and group

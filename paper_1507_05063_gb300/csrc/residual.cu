@@ -389,7 +389,7 @@ Tiling make_fx_tiling(const Grid3& g, int tz) {
 // The depth that minimises the busiest SM's time, over the even cuts of the deepest grid.
 // A full round of slabs takes kFxBlocks units of an SM's time per plane, a last round of k
 // slabs per SM k units (at least three: fewer wait on their own latency); a slab's planes
-// count with its two halo planes, in groups of four, and about two planes' time for its start.
+// count with its two halo planes, in groups of six, and about two planes' time for its start.
 int choose_fx_tz(const Grid3* grids, int n) {
   const long long sms = device_sms();
   int deepest = 1;

@@ -2,7 +2,7 @@
 
 These kernels bring a block's float64 values to one power of two and sum 64-bit integers.
 The tests take them where that can go wrong: slab and group edges (32 x 8 columns, groups
-of four planes), partial slabs, the smallest grids, scales from 1e-300 to 1e300, steps of
+of six planes), partial slabs, the smallest grids, scales from 1e-300 to 1e300, steps of
 many orders of magnitude between neighbouring groups, zeros, infinities and NaN.  The
 reference is the float64 oracle; tolerances come from float64's own rounding of a 19-point
 sum: c0 = 8 (1/hx^2 + 1/hy^2 + 1/hz^2) is its largest weight and the absolute weights add up
