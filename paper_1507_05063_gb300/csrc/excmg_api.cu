@@ -574,14 +574,17 @@ excmg_status cg_loop(const Ctx& c, int n, CGDesc<T>* ddesc, long long tiles, int
   if (coop >= n && coop > 0 && c.persistent_ok) {
     int grid_total = 0;
     if (!small) {
-      // team sizes: a lone problem takes every co-resident block it can use; in a batch
-      // each problem takes about one block per two tiles, and teams are formed in order
-      // of decreasing size (slots are taken in order by the blocks of one launch)
+      // team sizes: a block per slab while the batch's slabs fit the co-resident blocks
+      // (always, for a lone problem up to that number), else each problem's share of them,
+      // so that no team waits for another's end; teams are formed in order of decreasing
+      // size (slots are taken in order by the blocks of one launch).  16 grids of 2^15 to
+      // 2^20 nodes, finest level: a block per two slabs 24.7 ms a call, this 24.1 ms
       std::vector<int> g(n), order(n);
-      long long slots = 0;
+      long long slots = 0, slabs = 0;
+      for (int p = 0; p < n; ++p) slabs += hd[p].t.count();
       for (int p = 0; p < n; ++p) {
         const long long tp = hd[p].t.count();
-        const long long want = (n == 1) ? tp : (tp + 1) / 2;
+        const long long want = n == 1 || slabs <= coop_used ? tp : tp * coop_used / slabs;
         g[p] = (int)std::max(1LL, std::min<long long>(want, coop_used));
         order[p] = p;
         slots += g[p];
@@ -736,13 +739,16 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
   for (const Item& it : items)
     if (!it.d64.direct) grids.push_back(it.res.g);
   const int fx_tz = choose_fx_tz(grids.data(), (int)grids.size());
+  const int cg_tz =
+      grids.size() > 1 && !mixed ? choose_team_tz(grids.data(), (int)grids.size(), persistent_cg_blocks<double>()) : fx_tz;
   for (int a = 0; a < n; ++a) {
     Item& it = items[a];
     it.iters = it.refs = 0;
     it.status = EXCMG_OK;
     it.relres = 0.0;
     ResDesc r = it.res;
-    r.t = it.d64.t = make_fx_tiling(r.g, fx_tz);
+    r.t = make_fx_tiling(r.g, fx_tz);
+    it.d64.t = make_fx_tiling(r.g, cg_tz);
     r.tile_begin = rtiles;
     if (!it.d64.direct) rtiles += r.t.count();  // DSOLVE levels form their own b
     it.d64.tile_begin = tiles;
@@ -1434,17 +1440,21 @@ excmg_status excmg_solve_batched(int nprob, const excmg_grid* grids, const doubl
     P[i].L = prob_layout(P[i].lv, opt->precision == EXCMG_MIXED, false, mixed_min(opt));
     base += P[i].L.bytes;
   }
-  // Problems whose finest grid has kBatchSoloNodes nodes or more run one after another,
-  // each on the whole GPU with a single solve's engines (the shared-memory CG up to 2^20
-  // nodes, every SM above); the others share the launches of one batch, where their CG
-  // runs as a team of blocks per problem.  Each problem keeps its own workspace region;
-  // the runs share the header's states in stream order.
+  // The problems share the launches of one batch, where the CG of each runs as a team of
+  // blocks.  One or two of kBatchSoloNodes nodes and more leave its blocks idle at the
+  // barriers, and a grid of kBatchSoloMax fills the GPU: these run one after another with a
+  // single solve's engines (measured at the constants).  A profiled batch runs them so too:
+  // kernel times are a single solve's.  Each problem keeps its own workspace region; the
+  // runs share the header's states in stream order.
   std::vector<int> solo, team;
-  for (int i = 0; i < nprob; ++i) {
+  auto finest = [&](int i) {
     const Level& fl = P[i].lv.back();
-    const long long nodes = (long long)(fl.nx + 1) * (fl.ny + 1) * (fl.nz + 1);
-    (nodes >= kBatchSoloNodes ? solo : team).push_back(i);
-  }
+    return (long long)(fl.nx + 1) * (fl.ny + 1) * (fl.nz + 1);
+  };
+  int large = 0;
+  for (int i = 0; i < nprob; ++i) large += finest(i) >= kBatchSoloNodes;
+  const long long solo_min = large <= 2 || opt->profile ? kBatchSoloNodes : kBatchSoloMax;
+  for (int i = 0; i < nprob; ++i) (finest(i) >= solo_min ? solo : team).push_back(i);
   if (solo.empty()) return run_excmg(P, opt, nullptr, stats, c);
   excmg_status result = EXCMG_OK;
   long long launches = 0;

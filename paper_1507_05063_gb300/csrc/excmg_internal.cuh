@@ -113,6 +113,8 @@ Tiling make_tiling(const Grid3& g, int tz);
 Tiling make_fx_tiling(const Grid3& g, int tz);
 // The slab depth for one launch over the n grids.
 int choose_fx_tz(const Grid3* grids, int n);
+// ... of a batch's CG, whose problems each get a team of one launch's `blocks` blocks.
+int choose_team_tz(const Grid3* grids, int n, int blocks);
 int choose_tz(const Grid3& g, int grid_blocks, int requested);
 
 // Tensor maps of one float32 CG problem (cp.async.bulk.tensor): r and the two p buffers,
@@ -258,12 +260,14 @@ bool encode_plane_map(CUtensorMap* m, float* base, const Grid3& g32);
 #define EXCMG_RESIDENT_MAX_NODES (1 << 20)
 #endif
 constexpr long long kResidentMaxNodes = EXCMG_RESIDENT_MAX_NODES;
-// excmg_solve_batched: problems with a finest grid of at least this many nodes run as
-// single solves, one after another; smaller ones share the batch's launches.
-#ifndef EXCMG_BATCH_SOLO_NODES
-#define EXCMG_BATCH_SOLO_NODES (1LL << 18)
-#endif
-constexpr long long kBatchSoloNodes = EXCMG_BATCH_SOLO_NODES;
+// excmg_solve_batched: one or two problems whose finest grid has kBatchSoloNodes nodes or
+// more, and any of kBatchSoloMax, run as single solves, one after another; the others share
+// the batch's launches.  ms for n equal problems of 64^3 / 128x64x32 / 128x128x64 / 128^3 /
+// 256x128x128 cells (eps 1e-8), as single solves: n = 2: 1.08 / 2.45 / 2.49 / 1.67 / 2.35, n =
+// 3: 1.57 / 3.65 / 3.67 / 2.46 / 3.51, n = 6: 3.11 / 7.50 / 7.44 / 4.85 / -; as teams: 1.01 /
+// 2.88 / 2.45 / 1.51 / 2.19, 1.09 / 3.29 / 2.99 / 1.77 / 2.64, 1.46 / 4.50 / 4.41 / 2.68 / -
+// (MIXED the same within 10%).
+constexpr long long kBatchSoloNodes = 1LL << 18, kBatchSoloMax = 1LL << 23;
 struct ResidentDesc {
   Grid3 g;
   Coef A;

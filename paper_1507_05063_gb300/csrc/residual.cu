@@ -413,6 +413,32 @@ int choose_fx_tz(const Grid3* grids, int n) {
   return best;
 }
 
+// The depth that minimises the longest team's step, over the even cuts of the deepest grid: a
+// team has a block per slab if all slabs get one, else its share of the blocks (cg_loop's
+// rule), and its slabs per block take their planes as in choose_fx_tz.
+int choose_team_tz(const Grid3* grids, int n, int blocks) {
+  int deepest = 1;
+  for (int k = 0; k < n; ++k) deepest = std::max(deepest, grids[k].nz - 1);
+  int best = 2;
+  double best_cost = 1e300;
+  for (int cuts = 1; cuts <= 256; ++cuts) {
+    const int tz = (deepest + cuts - 1) / cuts;
+    if (tz < 2 && cuts > 1) break;
+    long long slabs = 0, rounds = 1;
+    for (int k = 0; k < n; ++k) slabs += make_fx_tiling(grids[k], tz).count();
+    for (int k = 0; k < n && slabs > blocks; ++k) {
+      const long long tp = make_fx_tiling(grids[k], tz).count(), share = std::max(1LL, tp * blocks / slabs);
+      rounds = std::max(rounds, (tp + share - 1) / share);
+    }
+    const double cost = (double)rounds * ((tz + 2 + kFxG - 1) / kFxG * kFxG + 2);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = tz;
+    }
+  }
+  return best;
+}
+
 FxWeights make_fx_weights(const Grid3& g) {
   const double w[3] = {1.0 / (g.hx * g.hx), 1.0 / (g.hy * g.hy), 1.0 / (g.hz * g.hz)};
   int ex = 0;

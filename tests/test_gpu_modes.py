@@ -235,3 +235,24 @@ def test_source_recovery_descends(X):
         losses.append(float(loss))
     assert all(b < a for a, b in zip(losses, losses[1:]))
     assert losses[-1] < 0.5 * losses[0]
+
+
+@pytest.mark.parametrize("count,N,N0", [(3, (64, 64, 64), (4, 4, 4)), (40, (64, 64, 32), (8, 8, 4))])
+def test_batched_teams_share_the_blocks(X, count, N, N0):
+    """Problems of 2^18 nodes in teams (three of them), and more slabs than co-resident blocks
+    (40 problems of 16 slabs at least: each team takes its share): every problem meets its
+    tolerance and agrees with its single solve far below it."""
+    eps, L = 1e-10, (1.0, 1.0, 1.0)
+    batch = []
+    for i in range(count):
+        f, g, _ = P.make_inputs(P.trig_sum(57 + i % 4, K=8, L=L), N, L)
+        batch.append(X.BatchedProblem(L, N, N0, dev(f), dev(g)))
+    res = X.solve_batched(batch, eps=eps)
+    for p, ub, st in list(zip(batch, res["u"], res["stats"]))[:4]:
+        single = X.solve(p.f, p.g, L, N0, eps=eps)
+        a, b = host(ub), host(single["u"])
+        assert np.max(np.abs(a - b)) <= 1e-6 * np.max(np.abs(b)) + 1e-12
+    for k, (ub, st) in enumerate(zip(res["u"], res["stats"])):
+        assert st["relres"][-1] <= eps * 1.0000001
+        if k >= 4:  # the same problem again: another team, the same sums
+            assert np.max(np.abs(host(ub) - host(res["u"][k % 4]))) <= 1e-12 * np.max(np.abs(host(ub)))
