@@ -293,10 +293,10 @@ bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem);
 cudaError_t launch_cg_resident(const ResidentDesc& D, size_t smem, CGState* st, void* parts,
                                unsigned* counter, int* err, cudaStream_t s);
 
-// DSOLVE by the discrete sine transform (dsolve_kernels.cu): one block per descriptor
+// DSOLVE by the discrete sine transform (dsolve_kernels.cu): one cluster per descriptor
 // with `direct` set (others return at once); x's interior = A^{-1} r, r = the residual
-// of the result, the CG state done with 0 steps.  dsolve_fits: the grid's interior fits
-// one block's shared memory; dsolve_smem: the bytes it needs.
+// of the result, the CG state done with 0 steps.  dsolve_fits: three arrays of the grid's
+// interior fit one block's shared memory; dsolve_smem: the bytes that a block needs.
 bool dsolve_fits(const Grid3& g);
 size_t dsolve_smem(const Grid3& g);
 cudaError_t launch_dsolve(int nprob, const CGDesc<double>* descs, size_t smem, CGState* st,

@@ -136,6 +136,21 @@ def test_streaming_cg_sums(X, N, steps, scale):
     assert np.max(np.abs(u.cpu().numpy() - want)) <= 1e-12 * np.max(np.abs(want))
 
 
+@pytest.mark.parametrize("N,scale,steps", [((16, 17, 18), 1.0, 6), ((31, 33, 35), 1e-60, 6), ((40, 9, 70), 1e60, 6),
+                                           ((100, 80, 60), 1.0, 6), ((120, 65, 80), 1.0, 3)])
+def test_resident_cg_sums(X, N, scale, steps):
+    """The shared-memory CG (up to 2^20 nodes) after fixed steps: boxes cut by the grid's far
+    faces, one node per thread and several; tolerance as above."""
+    L = (1.0, 0.9, 1.1)
+    f, start = fields(N, 8)
+    f, start = f * scale, start * scale
+    want, _, _ = O.cg(start, f, O.meshsizes(L, N), 0.0, fixed_iters=steps)
+    u = dev(start)
+    st = X.cg(dev(f), u, L, eps=0.0, fixed_iters=[steps], profile=1)
+    assert "cg_resident_f64" in st["profile"]
+    assert np.max(np.abs(u.cpu().numpy() - want)) <= 1e-12 * np.max(np.abs(want))
+
+
 @pytest.mark.parametrize("N", [(8, 8, 8), (24, 8, 16), (32, 16, 8), (40, 24, 16), (72, 16, 40)])
 @pytest.mark.parametrize("scale", [1.0, 1e-250, 1e250])
 def test_exp_finite_bricks(X, N, scale):

@@ -422,3 +422,18 @@ def test_workspace_reuse_gives_same_answer(X):
     b = X.solve(fd, gd, (1, 1, 1), (4, 4, 4), eps=1e-10, ws=ws)
     c = X.solve(fd, gd, (1, 1, 1), (4, 4, 4), eps=1e-10, ws=ws)
     assert torch.equal(a["u"], b["u"]) and torch.equal(b["u"], c["u"])
+
+
+@pytest.mark.parametrize("N0", [(2, 2, 2), (2, 2, 10), (10, 2, 2), (2, 12, 4), (6, 2, 4), (6, 8, 4)])
+def test_dsolve_shares(X, N0):
+    """DSOLVE's blocks share a problem's planes and columns: fewer of either than blocks, and
+    numbers of them that the blocks do not divide.  Against the dense solve; the residual is
+    that of a direct solve (a few hundred roundings of the operator's size)."""
+    L = (1.0, 0.8, 1.3)
+    N = tuple(4 * n for n in N0)
+    f, g, _ = P.make_inputs(P.PROBLEMS["ex3"], N, L)
+    res = X.solve(dev(f), dev(g), L, N0, eps=1e-10)
+    st = res["stats"]
+    assert st["iters"][:2] == [0, 0] and max(st["relres"][:2]) <= 1e-13
+    ref = O.excmg(f, g, L, N, N0, eps=1e-10, dsolve="dense", fixed_iters=st["iters"])
+    assert rel_linf(host(res["u"]), ref["u"][-1]) <= TOL_SOLVE
