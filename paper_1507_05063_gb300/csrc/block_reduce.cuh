@@ -14,23 +14,26 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sum over the block; the result is valid in thread 0.  Every thread must call.
-// float64 instructions are scarce on this GPU (2 per clock per SM, 64-clock latency), so
-// only warp 0 adds: every thread parks its value in shared memory, then each lane of
-// warp 0 sums blockDim/32 of them in a fixed order and the warp reduces by shuffles.
-// The order is fixed, so the result is deterministic.
-__device__ double block_sum(double v) {
-  __shared__ double s_v[kThreads];
-  const int lane = threadIdx.x & 31;
+// Sums over the block of NV values per thread; sum v is valid in warp v's first thread.  Every
+// thread must call.  float64 instructions are scarce on this GPU (2 per clock per SM,
+// 64-clock latency), so one warp adds per value, the values side by side: every thread parks
+// its values in shared memory, then each lane of warp v sums blockDim/32 of value v in a fixed
+// order and the warp reduces by shuffles.  The order is fixed, so the result is deterministic.
+template <int NV>
+__device__ __forceinline__ double block_sums(const double (&v)[NV]) {
+  static_assert(NV <= kThreads / 32, "a warp per value");
+  __shared__ double s_v[NV][kThreads];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __syncthreads();
-  s_v[threadIdx.x] = v;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) s_v[k][threadIdx.x] = v[k];
   __syncthreads();
   double t = 0.0;
-  if (threadIdx.x < 32) {
+  if (warp < NV) {
     // kThreads / 32 values per lane as a pairwise tree (a short dependence chain)
     double w[kThreads / 32];
 #pragma unroll
-    for (int u = 0; u < kThreads / 32; ++u) w[u] = s_v[lane + 32 * u];
+    for (int u = 0; u < kThreads / 32; ++u) w[u] = s_v[warp][lane + 32 * u];
 #pragma unroll
     for (int d = 1; d < kThreads / 32; d *= 2)
 #pragma unroll
@@ -40,11 +43,17 @@ __device__ double block_sum(double v) {
   return t;
 }
 
-// Warp-0 sum of src[0 .. n) from global memory (through L2) in a fixed order: each lane
+// Sum over the block; the result is valid in thread 0.  Every thread must call.
+__device__ double block_sum(double v) {
+  const double vs[1] = {v};
+  return block_sums(vs);
+}
+
+// One warp's sum of src[0 .. n) from global memory (through L2) in a fixed order: each lane
 // takes the values lane, lane + 32, ... in chunks of kSumChunk loads in flight, sums a
 // chunk as a pairwise tree, then the lanes reduce by shuffles.  Valid in lane 0.
 constexpr int kSumChunk = 8;
-__device__ __forceinline__ double warp0_sum_global(const double* src, int n) {
+__device__ __forceinline__ double warp_sum_global(const double* src, int n) {
   const int lane = threadIdx.x & 31;
   double acc = 0.0;
   for (int i0 = 0; i0 < n; i0 += 32 * kSumChunk) {
@@ -76,6 +85,7 @@ template <int NV, typename Fin>
 __device__ void publish_and_finish(int nprob, const int* s_active, const double* s_part,
                                    double* partials, unsigned* counters, const Fin& fin) {
   __shared__ int s_last[kMaxProb];
+  __shared__ double s_sums[NV];
   const int G = gridDim.x;
   for (int p = threadIdx.x; p < nprob; p += blockDim.x) {
     s_last[p] = 0;
@@ -92,12 +102,14 @@ __device__ void publish_and_finish(int nprob, const int* s_active, const double*
   for (int p = 0; p < nprob; ++p) {
     if (!s_last[p]) continue;  // shared value: uniform across the block
     __threadfence();
-    double sums[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-      sums[v] = threadIdx.x < 32 ? warp0_sum_global(partials + ((long long)p * NV + v) * G, G) : 0.0;
+    const int v = threadIdx.x >> 5;  // a warp per value
+    if (v < NV) {
+      const double t = warp_sum_global(partials + ((long long)p * NV + v) * G, G);
+      if ((threadIdx.x & 31) == 0) s_sums[v] = t;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-      fin(p, sums);
+      fin(p, s_sums);
       counters[p] = 0u;
     }
     __syncthreads();

@@ -909,7 +909,7 @@ __device__ bool grid_barrier(unsigned* bar, unsigned target, int* err, unsigned 
 // Sum of n partials in a fixed order, identical in every block (warp 0 only: the adds
 // are float64).  Result in thread 0.
 __device__ double sum_partials_all(const double* part, int n) {
-  return threadIdx.x < 32 ? warp0_sum_global(part, n) : 0.0;
+  return threadIdx.x < 32 ? warp_sum_global(part, n) : 0.0;
 }
 
 #ifndef EXCMG_PERSIST_MIN_BLOCKS

@@ -46,10 +46,11 @@ struct FxSlab {
 
 __device__ __forceinline__ FxSlab fx_slab(const Grid3& g, const Tiling& tl, long long lt) {
   FxSlab c;
-  c.x0 = 1 + (int)(lt % tl.ntx) * kFxX;
-  const long long r = lt / tl.ntx;
-  c.y0 = 1 + (int)(r % tl.nty) * kFxY;
-  c.z0 = 1 + (int)(r / tl.nty) * tl.tz;
+  // (a grid that fits the memory has fewer than 2^32 slabs of 512 nodes and more)
+  const unsigned r = (unsigned)lt / (unsigned)tl.ntx, z = r / (unsigned)tl.nty;
+  c.x0 = 1 + (int)((unsigned)lt - r * (unsigned)tl.ntx) * kFxX;
+  c.y0 = 1 + (int)(r - z * (unsigned)tl.nty) * kFxY;
+  c.z0 = 1 + (int)z * tl.tz;
   c.z1 = min(c.z0 + tl.tz, g.nz);
   return c;
 }

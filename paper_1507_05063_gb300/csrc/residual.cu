@@ -86,14 +86,9 @@ __device__ __forceinline__ double res_rhs(const ResDesc& d, int i, int j, int k,
 // added to its three partials in shared memory.  Called at problem switches only; kept
 // out of line so that it adds no registers to the plane loop.
 __device__ __noinline__ void residual_flush(double acc_r, double acc_b, double acc_f, double* part) {
-  const double s1 = block_sum(acc_r);
-  const double s2 = block_sum(acc_f + acc_b);
-  const double s3 = block_sum(acc_f);
-  if (threadIdx.x == 0) {
-    part[0] += s1;
-    part[1] += s2;
-    part[2] += s3;
-  }
+  const double v[3] = {acc_r, acc_f + acc_b, acc_f};
+  const double s = block_sums(v);
+  if ((threadIdx.x & 31) == 0 && threadIdx.x < 96) part[threadIdx.x >> 5] += s;
 }
 
 // lift (lift + 2 RHS) of the interior nodes x0 .. x1 - 1 (y, z likewise) of a slab that are
@@ -297,25 +292,19 @@ __device__ __forceinline__ void residual_slab_any(const ResDesc& d, const FxSlab
   }
 }
 
-// r = 0 on the grid's boundary nodes, by block bl of G.
+// r = 0 on the grid's boundary nodes, by block bl of G: a row per warp (no divisions: they
+// took a third of a small grid's prologue).
 template <typename TR>
 __device__ __noinline__ void zero_r_faces(const ResDesc& d, int bl, int G) {
   const Grid3& g = d.g;
   const long long osy = sizeof(TR) == 4 ? d.osy : g.sy, osz = sizeof(TR) == 4 ? d.osz : g.sz;
   TR* r = reinterpret_cast<TR*>(d.r);
-  const int tid = bl * kThreads + threadIdx.x, nth = G * kThreads;
-  const int wx = g.nx + 1, wy = g.ny + 1, wz = g.nz + 1;
-  for (long long t = tid; t < (long long)wx * wy; t += nth) {
-    const long long o = t % wx + t / wx * osy;
-    r[o] = r[o + g.nz * osz] = (TR)0.0;
-  }
-  for (long long t = tid; t < (long long)wx * wz; t += nth) {
-    const long long o = t % wx + t / wx * osz;
-    r[o] = r[o + g.ny * osy] = (TR)0.0;
-  }
-  for (long long t = tid; t < (long long)wy * wz; t += nth) {
-    const long long o = t % wy * osy + t / wy * osz;
-    r[o] = r[o + g.nx] = (TR)0.0;
+  const int lane = threadIdx.x & 31, warp = bl * (kThreads / 32) + (threadIdx.x >> 5), nw = G * (kThreads / 32);
+  for (int j = warp; j <= g.ny; j += nw)
+    for (int i = lane; i <= g.nx; i += 32) r[i + j * osy] = r[i + j * osy + g.nz * osz] = (TR)0.0;
+  for (int k = warp; k <= g.nz; k += nw) {
+    for (int i = lane; i <= g.nx; i += 32) r[i + k * osz] = r[i + k * osz + g.ny * osy] = (TR)0.0;
+    for (int j = lane; j <= g.ny; j += 32) r[j * osy + k * osz] = r[j * osy + k * osz + g.nx] = (TR)0.0;
   }
 }
 
