@@ -187,7 +187,8 @@ def test_exp_finite_nonfinite(X):
     assert np.array_equal(got[9:], clean[9:]) and np.array_equal(got[:, :, 33:], clean[:, :, 33:])
 
 
-@pytest.mark.parametrize("N", [(2, 2, 2), (4, 2, 6), (62, 6, 14), (64, 8, 16), (66, 10, 18), (126, 30, 34)])
+@pytest.mark.parametrize("N", [(2, 2, 2), (4, 2, 6), (62, 6, 14), (64, 8, 16), (66, 10, 18), (126, 30, 34),
+                               (128, 10, 20)])
 def test_exp_true_tiles(X, N):
     """EXP_true across its 64 x 8 columns and chunks of eight coarse planes: a sum of eight
     differences of at most 2 U, and the addition: ten roundings of 3 U."""
