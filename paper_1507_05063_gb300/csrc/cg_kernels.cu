@@ -207,6 +207,10 @@ __device__ __forceinline__ T spmv_tile(const CGDesc<T>& d, long long lt, bool fi
   return tacc;
 }
 
+// v 2^(a + b) where that may leave the normal range (a call, so that its products take the
+// float64 pipe only then).
+__device__ __noinline__ double scale_pq(double v, int a, int b) { return v * fx_pow2(a) * fx_pow2(b); }
+
 // One slab of a float64 problem: p_new = r + beta p_old (p = r when first) and q = A p_new on
 // its interior nodes; adds this thread's share of p.q to acc.  p is formed on load (1.3
 // float64 FMA per node, halo included) and stored as integers for the sums; p.q is taken
@@ -214,8 +218,7 @@ __device__ __forceinline__ T spmv_tile(const CGDesc<T>& d, long long lt, bool fi
 // F64: the sums in float64.  Returns false, in every thread, when a group is not for fixed
 // point (the caller then takes the slab again with F64).  All threads of the block must call.
 // Measured, a whole CG step: 385 x 201 x 121 cells 0.517 ms with the sums in float64 (19
-// float64 instructions per node and step), 0.220 ms here (8; the FP64 pipe 63% busy);
-// 128^3 0.14 ms, 0.061 ms here.
+// float64 instructions per node and step), 0.195 ms here (7.5); 128^3 0.150 ms, 0.055 ms here.
 template <bool F64>
 __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, bool first, double beta,
                                        const double* __restrict__ pold, double* __restrict__ pnew, FxSmem& S,
@@ -308,7 +311,11 @@ __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, 
         });
     }
     // the scales of p and q
-    acc += F64 ? accg : accg * fx_pow2(scale - 1022 - kFxBits) * fx_pow2(qL);
+    if (!F64) {
+      const int q = scale - 1022 - kFxBits + qL;  // |accg| < 2^122, a sum of integers
+      accg = q > -1000 && q < 800 ? fx_scale(accg, q) : scale_pq(accg, scale - 1022 - kFxBits, qL);
+    }
+    acc += accg;
   }
   acc_out += acc;
   return true;
