@@ -68,26 +68,27 @@ DESCRIPTION = {
 # (streams the method must move; halo re-reads excluded).  DP ops count FMA, MUL and
 # ADD as one each: they take one issue slot of the FP64 pipe.
 ALGO = {
-    "spmv_f64": {"bytes": 32.0, "dp_ops": 16.0},     # r, p_old in; p, q out
+    # DP ops count float64 instructions, conversions included: the 19-point sums of the float64
+    # kernels run on integers (block fixed point)
+    # r, p_old in; p, q out; 1.3 (p, halo included), 2 (q's and p's conversions), 1.2 (p.q)
+    "spmv_f64": {"bytes": 32.0, "dp_ops": 4.5},
     "update_f64": {"bytes": 48.0, "dp_ops": 3.0},    # x, p, r, q in; x, r out
     "spmv_f32": {"bytes": 16.0, "dp_ops": 0.0},
     "update_f32": {"bytes": 24.0, "dp_ops": 0.0},
-    # u, f in; r out.  DP ops: per plane 12 (19-point C/T terms), per node 2 (combine),
-    # 6 (twice the RHS), 1 (r), 1 (r.r), 1 (b.b; the lift terms only near the boundary)
-    "residual": {"bytes": 24.0, "dp_ops": 23.0},
-    # per fine node: ~4.4 FMA for the three quartic passes (odd positions only), ~1 for
-    # the extrapolated lattice (separable corner sums + one FMA per grid-2h node)
-    "exp_finite": {"bytes": 8.0 * (1 + 1 / 8 + 1 / 64), "dp_ops": 5.4},
+    # u, f in; r out; DP ops: the conversions of the two sums, r, r.r, RHS.RHS
+    "residual": {"bytes": 24.0, "dp_ops": 5.0},
+    # per fine node: the result's conversion
+    "exp_finite": {"bytes": 8.0 * (1 + 1 / 8 + 1 / 64), "dp_ops": 1.0},
     "init": {"bytes": 8.0, "dp_ops": 0.0},
     # MIXED refinement: u += e / s (u in and out, e in and zeroed): 8 + 4 + 8 + 4
     "correct": {"bytes": 24.0, "dp_ops": 1.0},
-    "exp_true": {"bytes": 8.0 * (2 + 1 / 8), "dp_ops": 4.0},
+    "exp_true": {"bytes": 8.0 * (2 + 1 / 8), "dp_ops": 2.4},
     # persistent CG: per node and CG step (the two fused bodies above)
-    "cg_f64": {"bytes": 80.0, "dp_ops": 19.0},
+    "cg_f64": {"bytes": 80.0, "dp_ops": 7.5},
     "cg_f32": {"bytes": 40.0, "dp_ops": 0.0},
     "cg_cluster_f64": {"bytes": 0.0, "dp_ops": 25.0},
     "cg_cluster_f32": {"bytes": 0.0, "dp_ops": 0.0},
-    "cg_resident_f64": {"bytes": 24.0, "dp_ops": 25.0},
+    "cg_resident_f64": {"bytes": 24.0, "dp_ops": 8.5},
     "dsolve": {"bytes": 24.0, "dp_ops": 72.0},
     "prolong_cmp": {"bytes": 8.0 * (1 + 1 / 8 + 1 / 64), "dp_ops": 3.0},
     # compact gradient: u in, three components out; the one-sided formulas, the
@@ -103,10 +104,10 @@ KERNEL_SYMBOL = {"spmv_f64": "k_dir_spmv_dot<double>", "update_f64": "k_update_d
                  "cg_f32": "k_cg_persistent<float> (tensor-copy staged)",
                  "cg_cluster_f64": "k_cg_cluster<double>", "cg_cluster_f32": "k_cg_cluster<float>",
                  "cg_resident_f64": "k_cg_resident", "dsolve": "k_dsolve",
-                 "prolong_cmp": "k_prolong_cmp", "grad": "k_grad_x + k_grad_strided"}
+                 "prolong_cmp": "k_prolong_cmp", "grad": "k_grad"}
 KERNEL_SOURCE = {"spmv_f64": "cg_kernels.cu", "update_f64": "cg_kernels.cu",
                  "spmv_f32": "cg_kernels.cu", "update_f32": "cg_kernels.cu",
-                 "residual": "cg_kernels.cu", "exp_finite": "transfer_kernels.cu",
+                 "residual": "residual.cu", "exp_finite": "transfer_kernels.cu",
                  "init": "transfer_kernels.cu", "correct": "cg_kernels.cu",
                  "exp_true": "transfer_kernels.cu", "cg_f64": "cg_kernels.cu",
                  "cg_f32": "cg_kernels.cu", "cg_cluster_f64": "cluster_cg.cu",

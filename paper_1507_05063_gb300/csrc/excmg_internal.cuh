@@ -22,7 +22,8 @@ constexpr int kTY = 8;           // y-rows of a stencil tile
 // Nodes of a fixed-point stencil slab along y (fixed_slab.cuh; kTX along x).
 constexpr int kFxSlabY = 8;
 // Blocks per SM of the fixed-point stencil kernels (80 registers): the residual of
-// 320 x 255 x 257 cells takes 375 us with three, 620 with four (64 registers, spills).
+// 320 x 255 x 257 cells takes 375 us with three, 620 with four (64 registers, spills;
+// groups of four planes).
 constexpr int kFxBlocks = 3;
 // Float64 solves with a stopping tolerance below this take their sums in float64: the target
 // lies under the rounding of float64 sums, so the step counts and the last digits follow

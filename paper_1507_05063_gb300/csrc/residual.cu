@@ -5,7 +5,7 @@
 // about 23 float64 instructions per node, 11.5 clocks of an SM at 2 lanes per clock, ten
 // times the 24 bytes a node moves.  Here five remain (the two conversions of the sums, the
 // difference, r.r and RHS.RHS).  Measured, one call on 320 x 255 x 257 cells: 1.11 ms in
-// float64, 0.46 ms here (the kernel 375 us; float64 pipe 55% busy, issue slots 46%), and the
+// float64, 0.42 ms here (the kernel 360 us; float64 pipe 61% busy, issue slots 46%), and the
 // error of r against 128-bit arithmetic 1.3 to 30 times smaller (random and smooth u).
 #include <math.h>
 
