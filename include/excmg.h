@@ -283,9 +283,9 @@ excmg_status excmg_grad(const excmg_grid* grid, const double* u, double* ux, dou
  * excmg_solve_batched -- `nprob` independent problems (each its own grid, f, g) solved by
  * Algorithm 1 together: each CG step of every active problem runs in ONE launch of the
  * stencil kernels over the union of all problems' tiles; problems are aligned on their
- * finest level.  Where only one or two finest grids have 2^18 nodes or more, and for grids of
- * 2^23 and more, those problems run first, one after another, as single solves (too few to
- * fill a shared launch, or enough each by itself); the others share the batch's launches.
+ * finest level.  Problems of 2^18 nodes and more share launches in groups of similar size, up
+ * to 2^23 nodes a group; one or two that are left, and grids of 2^23 nodes, run first, one
+ * after another, as single solves.  Smaller problems share one batch of launches.
  * With opt->profile every problem of 2^18 nodes and more runs as a single solve.  The results
  * are those of single solves up to rounding.  grids[nprob]: host array; f, g, u: host arrays of device pointers.
  * opt: shared options (fixed_iters must be NULL).  stats: NULL or host array[nprob].

@@ -1445,17 +1445,39 @@ excmg_status excmg_solve_batched(int nprob, const excmg_grid* grids, const doubl
   // barriers, and a grid of kBatchSoloMax fills the GPU: these run one after another with a
   // single solve's engines (measured at the constants).  A profiled batch runs them so too:
   // kernel times are a single solve's.  Each problem keeps its own workspace region; the
-  // runs share the header's states in stream order.
-  std::vector<int> solo, team;
+  // runs share the header's states in stream order.  The larger problems form teams
+  // in groups of similar size and at most kBatchGroupNodes nodes: a team keeps its blocks to
+  // its end, and in one launch over 64 problems of very different step counts the last ones
+  // ran on a few blocks each.
+  std::vector<int> solo, large, small;
   auto finest = [&](int i) {
     const Level& fl = P[i].lv.back();
     return (long long)(fl.nx + 1) * (fl.ny + 1) * (fl.nz + 1);
   };
-  int large = 0;
-  for (int i = 0; i < nprob; ++i) large += finest(i) >= kBatchSoloNodes;
-  const long long solo_min = large <= 2 || opt->profile ? kBatchSoloNodes : kBatchSoloMax;
-  for (int i = 0; i < nprob; ++i) (finest(i) >= solo_min ? solo : team).push_back(i);
-  if (solo.empty()) return run_excmg(P, opt, nullptr, stats, c);
+  for (int i = 0; i < nprob; ++i)
+    (finest(i) < kBatchSoloNodes ? small : finest(i) < kBatchSoloMax && !opt->profile ? large : solo).push_back(i);
+  std::stable_sort(large.begin(), large.end(), [&](int a, int b) { return finest(a) > finest(b); });
+  std::vector<std::vector<int>> teams;
+  for (size_t k = 0; k < large.size();) {
+    std::vector<int> group;
+    long long nodes = 0;
+    while (k < large.size() && (group.empty() || nodes + finest(large[k]) <= kBatchGroupNodes)) {
+      nodes += finest(large[k]);
+      group.push_back(large[k++]);
+    }
+    if (group.size() <= 2)
+      solo.insert(solo.end(), group.begin(), group.end());
+    else
+      teams.push_back(group);
+  }
+  // the small ones go with a single group, else form a launch of their own
+  if (teams.size() == 1) {
+    teams[0].insert(teams[0].end(), small.begin(), small.end());
+    std::sort(teams[0].begin(), teams[0].end());
+  } else if (!small.empty()) {
+    teams.push_back(small);
+  }
+  if (solo.empty() && teams.size() == 1) return run_excmg(P, opt, nullptr, stats, c);
   excmg_status result = EXCMG_OK;
   long long launches = 0;
   auto run_part = [&](const std::vector<int>& idx) -> excmg_status {
@@ -1477,7 +1499,7 @@ excmg_status excmg_solve_batched(int nprob, const excmg_grid* grids, const doubl
     if (e != EXCMG_OK && e != EXCMG_ERR_NOT_CONVERGED) return e;
     if (e != EXCMG_OK) result = e;
   }
-  if (!team.empty()) {
+  for (const std::vector<int>& team : teams) {
     const excmg_status e = run_part(team);
     if (e != EXCMG_OK && e != EXCMG_ERR_NOT_CONVERGED) return e;
     if (e != EXCMG_OK) result = e;

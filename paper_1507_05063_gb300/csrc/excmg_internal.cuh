@@ -269,6 +269,10 @@ constexpr long long kResidentMaxNodes = EXCMG_RESIDENT_MAX_NODES;
 // 2.88 / 2.45 / 1.51 / 2.19, 1.09 / 3.29 / 2.99 / 1.77 / 2.64, 1.46 / 4.50 / 4.41 / 2.68 / -
 // (MIXED the same within 10%).
 constexpr long long kBatchSoloNodes = 1LL << 18, kBatchSoloMax = 1LL << 23;
+// Teams of one launch: at most this many nodes.  64 problems of 2^15 to 2^24 nodes and very
+// different step counts: 608 ms in one launch, 416 in groups of 2^24 nodes, 378 of 2^23 (377 one
+// by one); 16 of 2^15 to 2^20: 22.9 / 22.9 / 22.5 (30.3).
+constexpr long long kBatchGroupNodes = 1LL << 23;
 struct ResidentDesc {
   Grid3 g;
   Coef A;
