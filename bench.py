@@ -31,7 +31,6 @@ for _v in ("OMP_NUM_THREADS", "OPENBLAS_NUM_THREADS", "MKL_NUM_THREADS"):
     os.environ[_v] = "1"
 
 import argparse  # noqa: E402
-import hashlib  # noqa: E402
 import json  # noqa: E402
 import multiprocessing  # noqa: E402
 import subprocess  # noqa: E402
@@ -126,26 +125,6 @@ def load_peaks():
         return float(d["hbm_gbs"]), "measured"
     except Exception:
         return 6800.0, "fallback"
-
-
-def source_hash(fname):
-    with open(os.path.join(ROOT, "paper_1507_05063_gb300", "csrc", fname), "rb") as fh:
-        return hashlib.sha256(fh.read()).hexdigest()[:16]
-
-
-def recorded_traffic(kind, workload):
-    """Per-node DRAM bytes of a kernel on this workload from a committed ncu summary, if
-    the kernel source is unchanged since (profiles/ncu_traffic.txt: kind workload
-    bytes_per_node source_sha)."""
-    path = os.path.join(ROOT, "profiles", "ncu_traffic.txt")
-    if not os.path.exists(path):
-        return None
-    for line in open(path):
-        parts = line.split()
-        if len(parts) >= 4 and not line.startswith("#") and parts[0] == kind and parts[1] == workload:
-            if parts[3] == source_hash(KERNEL_SOURCE[kind]):
-                return float(parts[2])
-    return None
 
 
 class Clocks:
@@ -458,9 +437,8 @@ def kernel_table(prof, hbm_peak):
     return kernels
 
 
-def roofline_of(kind, k, prof, hbm_peak, peak_kind, workload):
+def roofline_of(kind, k, prof, hbm_peak, peak_kind):
     nodes_per_launch = prof[kind]["nodes"] / prof[kind]["launches"]
-    traffic = recorded_traffic(kind, workload)
     if k["bound"] == "alu":
         roof = {"bound": "alu", "achieved": k["Gdpop_s"], "peak": DP_PEAK_GOPS, "unit": "G DP-op/s",
                 "frac": k["Gdpop_s"] / DP_PEAK_GOPS,
@@ -469,7 +447,7 @@ def roofline_of(kind, k, prof, hbm_peak, peak_kind, workload):
         roof = {"bound": "hbm", "achieved": k["GB_s"], "peak": hbm_peak, "unit": "GB/s",
                 "frac": k["GB_s"] / hbm_peak, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"}
     roof.update({"kernel": KERNEL_SYMBOL[kind], "share_of_step": k["share"],
-                 "traffic": traffic * nodes_per_launch if traffic is not None else None,
+                 "source": KERNEL_SOURCE[kind],
                  "algorithmic_bytes_per_launch": ALGO[kind]["bytes"] * nodes_per_launch,
                  "dp_ops_per_launch": ALGO[kind]["dp_ops"] * nodes_per_launch,
                  "avg_launch_us": k["avg_launch_us"],
@@ -1030,8 +1008,8 @@ def main():
 
     kernels = kernel_table(prof, hbm_peak)
     dom = max(kernels, key=lambda k: kernels[k]["ms"])
-    roof = roofline_of(dom, kernels[dom], prof, hbm_peak, peak_kind, wl)
-    roof_cg = roofline_of("cg_f32", kernels["cg_f32"], prof, hbm_peak, peak_kind, wl) if "cg_f32" in kernels else None
+    roof = roofline_of(dom, kernels[dom], prof, hbm_peak, peak_kind)
+    roof_cg = roofline_of("cg_f32", kernels["cg_f32"], prof, hbm_peak, peak_kind) if "cg_f32" in kernels else None
 
     line = {"metric": METRIC, "value": value, "unit": "unknowns/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
