@@ -69,12 +69,11 @@ struct Coef {
   double c0, fx, fy, fz, exy, exz, eyz;
 };
 Coef make_coef(const Grid3& g);
-// a = 1/hx^2, b, c as integers h 2^32 + l = a 2^k, the largest in [2^59, 2^60]: the
-// weights of the fixed-point sums (fixed_point.cuh).
+// a = 1/hx^2, b, c as integers h 2^31 + l = a 2^k, the largest in [2^59, 2^60], -2^30 <= l <
+// 2^30: the weights of the fixed-point sums (fixed_point.cuh).
 struct FxWeights {
-  int h[3], l[3];
+  int h[3], l[3], l2[3];  // l2 = 2 l
   int k;
-  long long m0;  // fx_weigh's start: its rounding terms
 };
 FxWeights make_fx_weights(const Grid3& g);
 

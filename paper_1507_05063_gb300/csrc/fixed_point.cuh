@@ -4,8 +4,8 @@
 // per clock and SM (measured), 32-bit integer adds at 119 and shifts, logic and multiplies
 // at 64.  The stencils of the scheme are short linear forms, so a tile of float64 values
 // is brought to one power-of-two scale (the largest exponent of the tile and its halo),
-// held as 64-bit integers, and its second differences are formed there exactly; only
-// their three products with 1/hx^2, 1/hy^2, 1/hz^2 round (to about 2^-62 of the largest
+// held as 64-bit integers, and its second differences and their products with 1/hx^2,
+// 1/hy^2, 1/hz^2 are formed there exactly; the sum rounds once (to about 2^-62 of the largest
 // possible sum, against float64's 2^-53 of every partial sum).
 //
 // With c a node's value, S_x, S_y, S_z its neighbour sums and E_xy ... its edge sums, and
@@ -35,20 +35,21 @@ constexpr int kFxMinExp = 200, kFxMaxExp = 1800;
 // The magnitude bits of x's high word: ordered as |x| is, to 2^-20.
 __device__ __forceinline__ unsigned fx_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
-// x as an integer of scale 2^(BITS - (E - 1022)), E >= every biased exponent of the tile:
-// |result| <= 2^BITS.  Bits below the scale are dropped (none for x within 2^(BITS - 53) of
-// the largest) and negative x are complemented, not negated: x moves by one unit at most,
-// 2^-BITS of the tile's largest value.  Zero and denormal x give 0 or -1 (E >= kFxMinExp).
+// x as an integer of scale 2^(BITS - (E - 1022)), E >= every biased exponent of the tile,
+// to nearest: |result| <= 2^BITS, exact for x within 2^(BITS - 53) of the largest, else off
+// by 2^-(BITS + 1) of the tile's largest value at most.  The magnitude is rounded and the sign
+// put back: -x gives the negative (zeros of either sign, and denormal x, give 0: E >=
+// kFxMinExp).
 template <int BITS>
 __device__ __forceinline__ long long fx_from_double(double x, int E) {
-  static_assert(BITS >= 53 && BITS <= 62, "the significand is shifted left by BITS - 53");
+  static_assert(BITS >= 53 && BITS <= 62, "the significand is shifted left by BITS - 52");
   const int hi = __double2hiint(x);
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u, d = (unsigned)(E - ((hi >> 20) & 0x7ff));
-  const long long m = (long long)(((unsigned long long)mh << 32 | (unsigned)__double2loint(x)) << (BITS - 53));
-  const int s = hi >> 31;
-  long long r;
-  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(m ^ (long long)s), "r"(d));  // clamps at 64
-  return r;
+  // one bit below the unit, for rounding
+  const unsigned long long m = ((unsigned long long)mh << 32 | (unsigned)__double2loint(x)) << (BITS - 52);
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(d));  // clamps at 64
+  return ((long long)(r ^ (unsigned long long)(long long)(hi >> 31)) + 1) >> 1;  // r + 1 or -r, halved
 }
 
 // 2^n for |n| <= 1022.
@@ -78,37 +79,37 @@ __device__ __forceinline__ double fx_scale_neg(double x, int q) {
   return __hiloint2double((hi & 0x7fffffff) ? hi + (int)(((unsigned)q << 20) ^ 0x80000000u) : hi, __double2loint(x));
 }
 
-// (X W_0 + Y W_1 + Z W_2) / 2^60 for |X|, |Y|, |Z| < 2^61.6,
-// 0 <= W = h 2^32 + l <= 2^60 (l signed).  The high parts' products are kept in full, the
-// mixed ones above 2^28; the low parts' products (up to 8 units each) enter with their
-// mean, and the result is rounded, not floored: W.m0 holds both.  (A floor, half a unit
-// the same way at every node, is a smooth right-hand side: the solution of the level
-// moved by 1e-14 with it.)  |result| < 2^62.
 // The power of two of the sums L (2 LHS = L 2^q) at scale E.
 __device__ __forceinline__ int fx_sum_exp(int k, int E) { return 60 - k - (kFxBits - (E - 1022)); }
 
-// PTX multiply-adds: one instruction per product, where the C form of the mixed-sign ones
-// expands to 36 for the nine.
+// PTX multiply-adds: one instruction per product.
 __device__ __forceinline__ long long fx_mad_s(int a, int b, long long c) {
   long long r;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
 }
-__device__ __forceinline__ long long fx_mad_u(unsigned a, unsigned b, long long c) {
-  long long r;
-  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
+
+// (X W_0 + Y W_1 + Z W_2) / 2^60 for |X|, |Y|, |Z| < 2^61.6 and 0 <= W = h 2^31 + l <= 2^60 (l
+// signed, l2 = 2 l); |result| <= 96 2^56 < 2^62.6.  With X = x_h 2^32 + x_l (x_l signed) the sum
+// is t 2^63 + m 2^31 + n, every product one 32 x 32 multiply-add: t = sum x_h h, m = sum x_l h +
+// x_h l2 (< 2^62.9), n = sum x_l l (< 2^62.6).  The whole sum is formed and rounded once, to
+// odd: exact, or the odd one of its two neighbours, so that -X, -Y, -Z give the negative and
+// no rounding has a preferred side.  (A floor, half a unit the same way at every node, is a
+// smooth right-hand side: the solution of the level moved by 1e-14 with it; dropped low
+// products break the symmetry in sign.)
 __device__ __forceinline__ long long fx_weigh(long long X, long long Y, long long Z, const FxWeights& W) {
-  const int xh = (int)(X >> 32), yh = (int)(Y >> 32), zh = (int)(Z >> 32);
+  const int xl = (int)X, yl = (int)Y, zl = (int)Z;
+  const int xh = (int)(X >> 32) - (xl >> 31), yh = (int)(Y >> 32) - (yl >> 31), zh = (int)(Z >> 32) - (zl >> 31);
+  const long long n = fx_mad_s(zl, W.l[2], fx_mad_s(yl, W.l[1], (long long)xl * W.l[0]));
+  long long m = fx_mad_s(xl, W.h[0], n >> 31);
+  m = fx_mad_s(yl, W.h[1], m);
+  m = fx_mad_s(zl, W.h[2], m);
+  m = fx_mad_s(xh, W.l2[0], m);
+  m = fx_mad_s(yh, W.l2[1], m);
+  m = fx_mad_s(zh, W.l2[2], m);
   const long long t = fx_mad_s(zh, W.h[2], fx_mad_s(yh, W.h[1], (long long)xh * W.h[0]));
-  long long m = fx_mad_u((unsigned)X, (unsigned)W.h[0], W.m0);
-  m = fx_mad_u((unsigned)Y, (unsigned)W.h[1], m);
-  m = fx_mad_u((unsigned)Z, (unsigned)W.h[2], m);
-  m = fx_mad_s(xh, W.l[0], m);
-  m = fx_mad_s(yh, W.l[1], m);
-  m = fx_mad_s(zh, W.l[2], m);
-  return (t << 4) + (m >> 28);
+  const unsigned rest = ((unsigned)m & 0x1fffffffu) | ((unsigned)n & 0x7fffffffu);
+  return ((t << 3) + (m >> 29)) | min(rest, 1u);
 }
 
 #endif  // __CUDACC__

@@ -145,11 +145,12 @@ __device__ __forceinline__ int block_exp(const uint4* s_mag) {
 // The scale of a group from its exponent and the previous group's.
 __device__ __forceinline__ int fx_group_scale(int E, int Eprev) { return max(max(E, Eprev), kFxMinExp); }
 
-// x 2^d: to the left exactly (the caller knows it fits), to the right rounded.
+// x 2^d: to the left exactly (the caller knows it fits), to the right to nearest, ties to even.
 __device__ __forceinline__ long long fx_shift(long long x, int d) {
   if (d >= 0) return x << min(d, 63);
   const int s = min(-d, 62);
-  return (x + ((1LL << s) >> 1)) >> s;
+  const long long y = x + ((1LL << s) >> 1);
+  return (y >> s) & ~(long long)((y & ((1LL << s) - 1)) == 0);
 }
 
 // The march of a thread's column.  With S_x, S_y, E a plane's in-plane neighbour and edge

@@ -434,20 +434,16 @@ FxWeights make_fx_weights(const Grid3& g) {
   frexp(std::max(w[0], std::max(w[1], w[2])), &ex);
   FxWeights W;
   if (!(w[0] + w[1] + w[2] < 1e300 && w[0] + w[1] + w[2] > 1e-300)) {
-    W = FxWeights{{0, 0, 0}, {0, 0, 0}, 1 << 20, 0};  // no tile's range holds: the float64 form
+    W = FxWeights{{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, 1 << 20};  // no tile's range holds: the float64 form
     return W;
   }
   W.k = 60 - ex;  // the largest weight becomes 2^59 .. 2^60
-  long long l = 0;
   for (int d = 0; d < 3; ++d) {
     const long long v = llrint(ldexp(w[d], W.k));
-    W.l[d] = (int)(unsigned)(v & 0xffffffffLL);
-    W.h[d] = (int)((v - (long long)W.l[d]) >> 32);
-    l += W.l[d];
+    W.l[d] = (int)((v + (1LL << 30)) & 0x7fffffffLL) - (1 << 30);
+    W.l2[d] = 2 * W.l[d];
+    W.h[d] = (int)((v - W.l[d]) >> 31);
   }
-  // half of the 2^28 that fx_weigh drops, and the mean of the low parts' products, l 2^31 each
-  // (of weight 1, m's is 2^32)
-  W.m0 = (1LL << 27) + l / 2;
   return W;
 }
 

@@ -215,8 +215,8 @@ struct BrickFx {
 };
 
 // The four odd (interpolated) values of a cell from its five grid-2h values: sum of w_m
-// 128 l_m(t), over 128, rounded.  w = hi 2^32 + lo with lo signed, so that every product is
-// one 32 x 32 multiply-add; |sum| / 128 < 2^62.
+// 128 l_m(t), over 128, to nearest, ties to even (so that -w gives the negative).  w = hi 2^32
+// + lo with lo signed, so that every product is one 32 x 32 multiply-add; |sum| / 128 < 2^62.
 __device__ __forceinline__ void quartic_fx(const long long (&w)[5], long long (&out)[4]) {
   constexpr int c[4][5] = {{35, 140, -70, 28, -5}, {-5, 60, 90, -20, 3}, {3, -20, 90, 60, -5}, {-5, 28, -70, 140, 35}};
   int hi[5], lo[5];
@@ -233,7 +233,7 @@ __device__ __forceinline__ void quartic_fx(const long long (&w)[5], long long (&
       H = fx_mad_s(hi[m], c[t][m], H);
       L = fx_mad_s(lo[m], c[t][m], L);
     }
-    out[t] = (H << 25) + (L >> 7);
+    out[t] = ((H << 25) + (L >> 7)) & ~(long long)(((int)L & 127) == 0);
   }
 }
 
@@ -305,7 +305,7 @@ __device__ bool exp_finite_brick_fx(const ProlongDesc& d, long long lb, BrickFx&
     S.d[k0][j0][i0] = has0 ? S.w[2 * k0 * BY1 + 2 * j0][2 * i0] - fx_from_double<kBrickBits>(v0, E) : 0;
   __syncthreads();
   // w = u_2h + (mean of d over the corners of the node's edge, face or element) / 16: the sum
-  // over the eight corners (coinciding ones counted as often) over 128, rounded
+  // over the eight corners (coinciding ones counted as often) over 128, to nearest, ties to even
 #pragma unroll
   for (int u = 0; u < kU; ++u) {
     const int e = tid + u * kThreads, ix = e % BX1, r = e / BX1, jy = r % BY1, kz = r / BY1;
@@ -313,7 +313,7 @@ __device__ bool exp_finite_brick_fx(const ProlongDesc& d, long long lb, BrickFx&
     const int ia = ix >> 1, ib = (ix + 1) >> 1, ja = jy >> 1, jb = (jy + 1) >> 1, ka = kz >> 1, kb = (kz + 1) >> 1;
     const long long s = ((S.d[ka][ja][ia] + S.d[ka][ja][ib]) + (S.d[ka][jb][ia] + S.d[ka][jb][ib])) +
                         ((S.d[kb][ja][ia] + S.d[kb][ja][ib]) + (S.d[kb][jb][ia] + S.d[kb][jb][ib]));
-    S.w[r][ix] += (s + 64) >> 7;
+    S.w[r][ix] += ((s + 64) >> 7) & ~(long long)((((int)s + 64) & 127) == 0);
   }
   __syncthreads();
   long long w[5], odd[4];
