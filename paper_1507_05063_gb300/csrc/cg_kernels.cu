@@ -242,7 +242,7 @@ __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, 
   double acc = 0.0;
   FxMarch M;
   F64March D;
-  int E1 = 0, scale = kFxMinExp;
+  FxRange R;
   for (int k0 = c.z0 - 1; k0 <= c.z1; k0 += kFxG) {
     // planes of the group that hold p: 1 .. nz - 1 of the grid, up to the upper halo plane
     const int lo = 1 - k0, hi = min(c.z1, nz - 1) - k0;
@@ -270,22 +270,22 @@ __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, 
     o += kFxG * sz;
 #pragma unroll
     for (int m = 0; m < kRimT; ++m) ro[m] += kFxG * sz;
+    bool held = true;
     if (F64) {
       __syncthreads();  // the box of the group before is read
       store_box(reinterpret_cast<double*>(S.box), p, C, [](double v) { return v; });
     } else {
-      warp_mag(p, S.mag[0]);
+      warp_mag(p, own, c.z1 - 1 - k0, S.mag[0]);
       __syncthreads();
-      const int E = block_exp(S.mag[0]);
-      if (E < 0) return false;
-      const int sc = fx_group_scale(E, E1);
-      E1 = E;
-      if (sc != scale) M.rescale(scale - sc);
-      scale = sc;
+      const int was = R.scale;
+      if (!R.next(S.mag[0])) return false;
+      held = R.near(S.mag[0]);
+      const int sc = R.scale;
+      if (sc != was) M.rescale(was - sc);
       store_box(S.box, p, C, [&](double v) { return fx_from_double<kFxBits>(v, sc); });
     }
-    const int qL = fx_sum_exp(W.k, scale) - 1;  // A p = -L 2^qL
-    if (!F64 && (qL < -1000 || qL > 800)) return false;
+    const int qL = fx_sum_exp(W.k, R.scale) - 1;  // A p = -L 2^qL
+    if (!F64 && (!held || qL < -1000 || qL > 800)) return false;
     __syncthreads();
     double accg = 0.0;
 #pragma unroll 1
@@ -312,8 +312,8 @@ __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, 
     }
     // the scales of p and q
     if (!F64) {
-      const int q = scale - 1022 - kFxBits + qL;  // |accg| < 2^122, a sum of integers
-      accg = q > -1000 && q < 800 ? fx_scale(accg, q) : scale_pq(accg, scale - 1022 - kFxBits, qL);
+      const int q = R.scale - 1022 - kFxBits + qL;  // |accg| < 2^122, a sum of integers
+      accg = q > -1000 && q < 800 ? fx_scale(accg, q) : scale_pq(accg, R.scale - 1022 - kFxBits, qL);
     }
     acc += accg;
   }

@@ -13,6 +13,8 @@
 //
 // The scale of a group is the largest exponent of its planes and the previous group's (whose
 // last two planes its sums still hold): the sums carried over are shifted when it changes.
+// Where a neighbourhood of the group is far smaller than the scale, its values would be held in
+// fewer bits than their own size asks for: such a slab takes the float64 form (FxRange).
 #pragma once
 
 #include "excmg_internal.cuh"
@@ -35,8 +37,12 @@ constexpr int kRimT = (kRim * kFxG + kThreads - 1) / kThreads;     // ... of a g
 constexpr int kLoads = kOwn + kRimT;
 static_assert(kFxX == 32 && kFxY == kFxSlabY, "one warp per x-run of a slab row");
 
+struct FxMags {
+  uint4 top[kThreads / 128];    // a word per warp: warp_mag
+  unsigned low[kThreads / 32];
+};
 struct FxSmem {
-  uint4 mag[2][kThreads / 128];  // a magnitude word per warp (of two arrays)
+  FxMags mag[2];  // of two arrays
   long long box[kFxG * kPlane];
 };
 
@@ -117,33 +123,62 @@ __device__ __forceinline__ void store_box(T* box, const double (&v)[kLoads], con
     if (C.rim_box[m] >= 0) box[C.rim_box[m]] = put(v[kOwn + m]);
 }
 
-// This warp's largest magnitude word into s_mag (a block barrier, then block_exp).
-__device__ __forceinline__ void warp_mag(const double (&v)[kLoads], uint4* s_mag) {
+// This warp's magnitude words of a group (a block barrier, then FxRange): the largest of its
+// values, and the smallest of its own nodes' neighbourhoods (~0: no own nodes).  A
+// neighbourhood is four planes (0 .. 3 or 2 .. 5 of the group) of a column and the columns
+// beside it; `own`: the thread has a column of interior nodes; last: the slab's last own plane
+// in the group.
+__device__ __forceinline__ void warp_mag(const double (&v)[kLoads], bool own, int last, FxMags& S) {
+  static_assert(kFxG == 6, "two overlapping windows of four planes");
   unsigned m = 0;
 #pragma unroll
-  for (int k = 0; k < kLoads; ++k) m = max(m, fx_mag(v[k]));
-  m = __reduce_max_sync(0xffffffffu, m);
+  for (int k = kOwn; k < kLoads; ++k) m = max(m, fx_mag(v[k]));
+  const unsigned mid = max(fx_mag(v[2]), fx_mag(v[3]));
+  unsigned a = max(mid, max(fx_mag(v[0]), fx_mag(v[1]))), b = max(mid, max(fx_mag(v[4]), fx_mag(v[5])));
+  m = __reduce_max_sync(0xffffffffu, max(m, max(a, b)));
+  a = max(a, max(__shfl_up_sync(0xffffffffu, a, 1), __shfl_down_sync(0xffffffffu, a, 1)));
+  b = max(b, max(__shfl_up_sync(0xffffffffu, b, 1), __shfl_down_sync(0xffffffffu, b, 1)));
+  const unsigned l = __reduce_min_sync(0xffffffffu, min(own && last >= 0 ? a : ~0u, own && last >= 2 ? b : ~0u));
   if (m == 0) {  // all zero, or denormal below 2^-1042: not for fixed point
     unsigned lo = 0;
 #pragma unroll
     for (int k = 0; k < kLoads; ++k) lo |= (unsigned)__double2loint(v[k]);
     m = __any_sync(0xffffffffu, lo != 0);
   }
-  if ((threadIdx.x & 31) == 0) reinterpret_cast<unsigned*>(s_mag)[threadIdx.x >> 5] = m;
+  if ((threadIdx.x & 31) == 0) {
+    reinterpret_cast<unsigned*>(S.top)[threadIdx.x >> 5] = m;
+    S.low[threadIdx.x >> 5] = l;
+  }
 }
 
-// The block's largest biased exponent: 0 for values that are all zero, -1 outside
-// [kFxMinExp, kFxMaxExp].
-__device__ __forceinline__ int block_exp(const uint4* s_mag) {
-  static_assert(kThreads == 256, "eight words of two 16-byte reads");
-  const uint4 a = s_mag[0], b = s_mag[1];
-  const unsigned m = max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
-  const int E = (int)(m >> 20);
-  return m == 0 ? 0 : E >= kFxMinExp && E <= kFxMaxExp ? E : -1;
-}
-
-// The scale of a group from its exponent and the previous group's.
-__device__ __forceinline__ int fx_group_scale(int E, int Eprev) { return max(max(E, Eprev), kFxMinExp); }
+// The scales of a slab's groups: a group's is the largest exponent of its planes and the
+// previous group's.
+struct FxRange {
+  int E = 0, low = 4095, scale = kFxMinExp;
+  // The scale of the next group; false, in every thread, where its exponents are outside
+  // [kFxMinExp, kFxMaxExp].
+  __device__ __forceinline__ bool next(const FxMags& S) {
+    static_assert(kThreads == 256, "eight words of two 16-byte reads");
+    const uint4 a = S.top[0], b = S.top[1];
+    const unsigned m = max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
+    const int was = E;
+    E = (int)(m >> 20);
+    scale = max(max(E, was), kFxMinExp);
+    return m == 0 || (E >= kFxMinExp && E <= kFxMaxExp);
+  }
+  // (After next.)  Whether the group's and the previous group's values are held near their own
+  // size: false, in every thread, if all values of a neighbourhood (of three columns, three rows and four
+  // planes) lie more than kFxRange powers of two below the scale, in a group that is not all
+  // zero.
+  __device__ __forceinline__ bool near(const FxMags& S) {
+    const unsigned l = S.low[threadIdx.x & 7], h = l == ~0u ? 0 : l;
+    // a row's neighbourhoods, or those of a row beside it
+    const unsigned h3 = max(h, max(__shfl_up_sync(0xffffffffu, h, 1, 8), __shfl_down_sync(0xffffffffu, h, 1, 8)));
+    const int was = low;
+    low = (int)(__reduce_min_sync(0xffffffffu, l == ~0u || E == 0 ? ~0u : h3) >> 20);
+    return scale - min(low, was) <= kFxRange;
+  }
+};
 
 // x 2^d: to the left exactly (the caller knows it fits), to the right to nearest, ties to even.
 __device__ __forceinline__ long long fx_shift(long long x, int d) {

@@ -182,52 +182,51 @@ __device__ __noinline__ bool residual_slab(const ResDesc& d, const FxSlab c, Res
   // f of the last plane, and 6 f with its faces but the one above
   using FT = typename std::conditional<F64, double, long long>::type;
   FT f1 = 0, s1 = 0;
-  int E1 = 0, F1 = 0, su = kFxMinExp, sf = kFxMinExp;
+  FxRange U, V;  // of u and f
   double acc_r = 0.0, acc_f = 0.0;
   auto ld = [](const double* a) { return __ldg(a); };
   for (int k0 = c.z0 - 1; k0 <= c.z1; k0 += kFxG) {
     double v[kLoads];
+    bool held = true;
     if (TF) {
       load_group(v, pf, lown, rf, rim, C, fz, 0, c.z1 - k0, ld);
       pf += kFxG * fz;
 #pragma unroll
       for (int m = 0; m < kRimT; ++m) rf[m] += kFxG * fz;
-      if (!F64) warp_mag(v, S.u.mag[1]);
+      if (!F64) warp_mag(v, own, c.z1 - 1 - k0, S.u.mag[1]);
       __syncthreads();  // the boxes of the group before are read
       if (F64) {
         store_box(reinterpret_cast<double*>(S.f), v, C, [](double x) { return x; });
       } else {
-        const int F = block_exp(S.u.mag[1]);
-        if (F < 0) return false;
-        const int scf = fx_group_scale(F, F1);
-        F1 = F;
-        if (scf != sf) {
-          f1 = (FT)fx_shift((long long)f1, sf - scf);
-          s1 = (FT)fx_shift((long long)s1, sf - scf);
+        const int was = V.scale;
+        if (!V.next(S.u.mag[1])) return false;
+        held = V.near(S.u.mag[1]);
+        const int sf = V.scale;
+        if (sf != was) {
+          f1 = (FT)fx_shift((long long)f1, was - sf);
+          s1 = (FT)fx_shift((long long)s1, was - sf);
         }
-        sf = scf;
-        store_box(S.f, v, C, [&](double x) { return fx_from_double<kFxBitsF>(x, scf); });
+        store_box(S.f, v, C, [&](double x) { return fx_from_double<kFxBitsF>(x, sf); });
       }
     }
     load_group(v, pu, lown, ru, rim, C, sz, 0, c.z1 - k0, ld);
     pu += kFxG * sz;
 #pragma unroll
     for (int m = 0; m < kRimT; ++m) ru[m] += kFxG * sz;
-    if (!F64) warp_mag(v, S.u.mag[0]);
+    if (!F64) warp_mag(v, own, c.z1 - 1 - k0, S.u.mag[0]);
     if (!F64 || !TF) __syncthreads();
     if (F64) {
       store_box(reinterpret_cast<double*>(S.u.box), v, C, [](double x) { return x; });
     } else {
-      const int E = block_exp(S.u.mag[0]);
-      if (E < 0) return false;
-      const int scu = fx_group_scale(E, E1);
-      E1 = E;
-      if (scu != su) M.rescale(su - scu);
-      su = scu;
-      store_box(S.u.box, v, C, [&](double x) { return fx_from_double<kFxBits>(x, scu); });
+      const int was = U.scale;
+      if (!U.next(S.u.mag[0])) return false;
+      held = held & U.near(S.u.mag[0]);
+      const int su = U.scale;
+      if (su != was) M.rescale(was - su);
+      store_box(S.u.box, v, C, [&](double x) { return fx_from_double<kFxBits>(x, su); });
     }
-    const int qL = fx_sum_exp(W.k, su) - 1, qF = sf - 1022 - kFxBitsF - 1;  // LHS = L 2^qL, RHS = F 2^qF
-    if (!F64 && (qL < -1000 || qL > 900)) return false;
+    const int qL = fx_sum_exp(W.k, U.scale) - 1, qF = V.scale - 1022 - kFxBitsF - 1;  // LHS = L 2^qL, RHS = F 2^qF
+    if (!F64 && (!held || qL < -1000 || qL > 900)) return false;
     const double scale = fx_pow2(qL);
     __syncthreads();
 #pragma unroll 1

@@ -88,3 +88,123 @@ def test_negative_zeros_are_zeros(X):
     r = X.residual(dev(plus[0]), dev(plus[1]), L)
     s = X.residual(dev(minus[0]), dev(minus[1]), L)
     assert torch.equal(r[0], s[0]) and r[1:] == s[1:]
+
+
+# A grid whose slabs (18 planes and their halo) hold four groups of six planes, and enough
+# nodes for the streaming CG.
+GROUPS_N, GROUPS_L = (70, 260, 70), (1.0, 0.9, 1.1)
+
+
+def near(a, planes):
+    """The largest |a| within one column, one row and `planes` planes of a node."""
+    m = np.abs(a)
+    for axis, reach in ((2, 1), (1, 1), (0, planes)):
+        out = m.copy()
+        for d in range(1, reach + 1):
+            lo, hi = [slice(None)] * 3, [slice(None)] * 3
+            lo[axis], hi[axis] = slice(None, -d), slice(d, None)
+            out[tuple(lo)] = np.maximum(out[tuple(lo)], m[tuple(hi)])
+            out[tuple(hi)] = np.maximum(out[tuple(hi)], m[tuple(lo)])
+        m = out
+    return m
+
+
+def ranged(kind, N, seed):
+    """Node arrays with a large range of values: exponential layers, a narrow Gaussian, steps
+    of many powers of ten along z (aligned with the groups of planes or not), compact support."""
+    rng = np.random.default_rng(seed)
+    i, j, k = np.meshgrid(*[np.arange(n + 1) for n in N], indexing="ij")
+    i, j, k = (a.transpose(2, 1, 0) for a in (i, j, k))
+    base = rng.standard_normal(i.shape)
+    if kind.startswith("layer"):
+        return base * np.exp(-{"x": i, "y": j, "z": k}[kind[5]] * 0.9)
+    if kind == "gauss":
+        return np.exp(-0.02 * ((i - N[0] / 2) ** 2 + (j - N[1] / 3) ** 2 + (k - N[2] / 2) ** 2))
+    if kind == "compact":  # ends within rows, columns and planes
+        return np.where((i - 20) ** 2 + (j - 30) ** 2 + (k - 30) ** 2 < 14 ** 2, base, 0.0)
+    step = {"steps6": 6, "steps4": 4, "steps11": 11}[kind]
+    w = 10.0 ** rng.integers(-25, 26, size=N[2] // step + 1)
+    w[rng.integers(0, len(w))] = 0.0
+    return base * np.repeat(w, step)[:N[2] + 1][:, None, None]
+
+
+KINDS = ["layerx", "layery", "layerz", "gauss", "compact", "steps6", "steps4", "steps11"]
+
+
+@pytest.mark.parametrize("which", ["u", "f"])
+@pytest.mark.parametrize("kind", KINDS)
+def test_residual_is_accurate_where_values_are_small(X, kind, which):
+    """Every node's r within 2^-50 of its neighbourhood's values times the weights -- eight
+    roundings in a row of a float64 sum; the absolute weights add up to less than 3 c0 for u
+    and are 6 for f -- not of the largest value of the grid.  Twice that: the oracle rounds as
+    well."""
+    N, L = GROUPS_N, GROUPS_L
+    rng = np.random.default_rng(7)
+    zero = np.zeros([n + 1 for n in N[::-1]])
+    f, u = zero, zero
+    if which == "u":
+        u = ranged(kind, N, 8)
+    else:
+        f = ranged(kind, N, 9)
+    h = O.meshsizes(L, N)
+    got = X.residual(dev(f), dev(u), L)[0].cpu().numpy()[1:-1, 1:-1, 1:-1]
+    want = O.residual(u, f, h)
+    if want.shape != got.shape:
+        want = want[1:-1, 1:-1, 1:-1]
+    c0 = 8 * sum(1.0 / v ** 2 for v in h)
+    tol = 2 * 2.0 ** -50 * (3 * c0 * near(u, 4) + 6 * near(f, 4))[1:-1, 1:-1, 1:-1]
+    assert np.all(np.abs(got - want) <= tol)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_streaming_cg_is_accurate_where_values_are_small(X, kind):
+    """Two steps of CG on A u = 0 from an iterate with a large range: x_2 = x_0 + a_0 r_0 + a_1 (r_0 - a_0 A r_0 + b_1 r_0), node by node.  Sixteen
+    roundings in a row and the scalars' (some 1e-13 of themselves) on each term."""
+    N, L = GROUPS_N, GROUPS_L
+    u0 = ranged(kind, N, 10)
+    for a in (u0[0], u0[-1], u0[:, 0], u0[:, -1], u0[:, :, 0], u0[:, :, -1]):
+        a[...] = 0.0
+    f = np.zeros_like(u0)
+    h = O.meshsizes(L, N)
+    inner = (slice(1, -1),) * 3
+
+    def full(v):
+        if v.shape == u0.shape:
+            return v
+        w = np.zeros_like(u0)
+        w[inner] = v
+        return w
+
+    r0 = full(O.residual(u0, f, h))
+    q0 = -full(O.residual(r0, f, h))  # A r_0
+    a0 = np.sum(r0 * r0) / np.sum(r0 * q0)
+    r1 = r0 - a0 * q0
+    b1 = np.sum(r1 * r1) / np.sum(r0 * r0)
+    p1 = r1 + b1 * r0
+    a1 = np.sum(r1 * r1) / -np.sum(p1 * full(O.residual(p1, f, h)))
+    want = u0 + a0 * r0 + a1 * p1
+    u = dev(u0)
+    st = X.cg(dev(f), u, L, eps=0.0, fixed_iters=[2], profile=1)
+    assert "cg_f64" in st["profile"]
+    c0 = 8 * sum(1.0 / v ** 2 for v in h)
+    # r_0 is itself off by its neighbourhood's rounding; A r_0 likewise, one node further
+    dr = 3 * c0 * near(u0, 4)
+    size = np.abs(u0) + (a0 + a1 * (1 + b1)) * dr + a0 * a1 * 3 * c0 * near(dr, 4)
+    assert np.all(np.abs(u.cpu().numpy() - want) <= (16 * 2.0 ** -50 + 1e-13) * size)
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e290])
+def test_residual_slab_taken_again(X, value):
+    """A value that is not for fixed point in a slab's third group, after two groups were
+    written: the slab is taken again in float64, and no other node sees it."""
+    N, L = GROUPS_N, GROUPS_L
+    f, u = fields(N, 11, "normal")
+    r0 = X.residual(dev(f), dev(u), L)[0].cpu().numpy()
+    u[32, 40, 20] = value
+    r1, rn, bn = X.residual(dev(f), dev(u), L)
+    r1 = r1.cpu().numpy()
+    bad = np.zeros(u.shape, bool)
+    bad[31:34, 39:42, 19:22] = True
+    c0 = 8 * sum(1.0 / v ** 2 for v in O.meshsizes(L, N))
+    assert np.all(np.abs(r1 - r0)[~bad] <= 2 * 2.0 ** -50 * 3 * c0 * np.max(np.abs(np.where(bad, 0.0, u))))
+    assert not np.isfinite(rn)  # 1e290: the square overflows
