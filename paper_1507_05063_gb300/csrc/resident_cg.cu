@@ -87,22 +87,26 @@ __device__ __noinline__ double2 rs_block_sum2(double a, double b, double* s_park
 // ---- sums of r.r and w.r as integers ----
 // A float64 warp instruction occupies the narrow FP64 pipe for 64 clocks and a level of a
 // float64 tree takes at least that; a step of a small level is a chain of such levels.  The
-// threads' partial sums are therefore brought to one power of two and added as integers: in
-// a warp by three 32-bit reductions of 19-bit pieces, in a block and over the grid as 64-bit
-// sums.  Every block adds the same integers, so the sums are the same in every block.
+// threads' partial sums are therefore brought to one power of two and added as integers: in a
+// warp by three 32-bit reductions of 19-bit pieces, over the warps of a block, over the blocks
+// (a warp's share of them, then the warps).  Every block adds the same integers, so the sums
+// are the same in every block.  The power of two is that of the largest value added, anew at
+// every level: a term is rounded to 2^-53 of the largest one or better, and to 2^-58 where the
+// terms are of one size (a float64 sum rounds to 2^-53 of itself at every addition).
 
-// One block's sums: gamma = g 2^eg, delta = d 2^ed; eg = kRsRaw: g and d are the bits of
-// float64 sums (infinities, NaN, extreme exponents, float64 solves).
-struct alignas(16) RsPart {
-  long long g, d;
-  int eg, ed;
-  long long pad;
+// A sum v 2^e; e = kRsRaw: v holds the bits of a float64 sum (infinities, NaN, extreme
+// exponents, float64 solves); e = -kRsRaw: 0.  A block's part is two of them, r.r and w.r.
+struct alignas(16) RsSum {
+  long long v;
+  int e, pad;
 };
 constexpr int kRsRaw = 1 << 20;
-constexpr int kRsBits = 57;  // of a thread's partial sum: 32 of them fit 62 bits
+constexpr int kRsBits = 57;  // of a term: 32 of them fit 62 bits
 
-// x as an integer of scale 2^(kRsBits - (E - 1022)), rounded; |x| < 2^(E - 1022).
+// x as an integer of scale 2^(kRsBits - (E - 1022)), rounded; |x| < 2^(E - 1022).  0 for E < 64:
+// below 2^-958, where the grid's largest |r|^2 is above 2^-846.
 __device__ __forceinline__ long long rs_fixed(double x, int E) {
+  if (E < 64) return 0;
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
@@ -127,21 +131,66 @@ __device__ __forceinline__ long long rs_round(long long v, int n) {
   return (v + ((1LL << n) >> 1)) >> n;
 }
 
-// v 2^e as float64, |v| < 2^63 and |e| <= 900 (what the blocks' scales allow).
+// v 2^e as float64, v = 0 or the result a normal number (what the blocks' scales allow).
 __device__ __forceinline__ double rs_double(long long v, int e) { return fx_scale((double)v, e); }
 
-// Reduction number `seq` (1, 2, ...): thread 0 stores this block's sums as part b of
-// the set seq & 1 (two sets: a block can be one reduction ahead of another's reads, never
-// two), arrives on the counter with release semantics -- which also publishes every
+__device__ __forceinline__ RsSum rs_none() {
+  RsSum t;
+  t.v = 0;
+  t.e = -kRsRaw;
+  t.pad = 0;
+  return t;
+}
+
+// Warp 0, after a block barrier: the sums of the warps' 2 x 8 sums (|v| <= 2^62), r.r in lanes 0
+// .. 7 and w.r in lanes 8 .. 15: |v| <= 2^62.
+__device__ __forceinline__ RsSum rs_over_warps(const RsSum (*s_warp)[kRsThreads / 32]) {
+  static_assert(kRsThreads / 32 == 8, "eight warps");
+  RsSum t = (&s_warp[0][0])[threadIdx.x & 15];
+  const bool raw = t.e == kRsRaw;
+  if (__any_sync(0xffffffffu, raw)) {
+    double x = raw ? __longlong_as_double(t.v) : t.v ? rs_double(t.v, t.e) : 0.0;
+#pragma unroll
+    for (int o = 1; o < 8; o *= 2) x += __shfl_xor_sync(0xffffffffu, x, o);
+    t.v = __double_as_longlong(x);
+    t.e = kRsRaw;
+    return t;
+  }
+  int m = t.e;
+#pragma unroll
+  for (int o = 1; o < 8; o *= 2) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  t.v = rs_round(t.v, m - t.e + 3);
+#pragma unroll
+  for (int o = 1; o < 8; o *= 2) t.v += __shfl_xor_sync(0xffffffffu, t.v, o);
+  t.e = m + 3;
+  return t;
+}
+
+// v 2^e of 56 bits (2^55 <= |v| <= 2^56, or none): two parts per lane are added.
+__device__ __forceinline__ RsSum rs_norm(RsSum t) {
+  if (t.e == kRsRaw) return t;
+  if (t.v == 0) return rs_none();
+  const int s = __clzll(t.v < 0 ? -t.v : t.v) - 1;
+  t.v = rs_round(t.v << s, 7);
+  t.e += 7 - s;
+  return t;
+}
+
+// Reduction number `seq` (1, 2, ...): lanes 0 and 8 of warp 0 store this block's sums as part b
+// of the set seq & 1 (two sets: a block can be one reduction ahead of another's reads, never
+// two), thread 0 arrives on the counter with release semantics -- which also publishes every
 // global store the block's threads made before the block barrier that precedes this
 // call -- and waits (bounded) until all G blocks have arrived.  Returns, in every
 // thread, false if the wait ran out or another block reported a time-out.
-__device__ bool rs_arrive_wait(const RsPart& part, RsPart* parts, unsigned* counter, int G, unsigned seq,
+__device__ bool rs_arrive_wait(const RsSum& part, RsSum* parts, unsigned* counter, int G, unsigned seq,
                                int* err, int* s_ok) {
+  if (threadIdx.x < 32) {
+    if ((threadIdx.x & 23) == 0)
+      __stcg(reinterpret_cast<int4*>(&parts[2 * ((size_t)(seq & 1) * G + blockIdx.x) + (threadIdx.x >> 3)]),
+             reinterpret_cast<const int4&>(part));
+    __syncwarp();
+  }
   if (threadIdx.x == 0) {
-    int4* to = reinterpret_cast<int4*>(&parts[(size_t)(seq & 1) * G + blockIdx.x]);
-    __stcg(to, reinterpret_cast<const int4*>(&part)[0]);
-    __stcg(to + 1, reinterpret_cast<const int4*>(&part)[1]);
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
     const unsigned target = seq * (unsigned)G;
     int ok = 1;
@@ -160,71 +209,52 @@ __device__ bool rs_arrive_wait(const RsPart& part, RsPart* parts, unsigned* coun
   return *s_ok != 0;
 }
 
-// The sum of a part per lane (eg = -kRsRaw: none), identical in every lane: the parts brought
-// to the largest exponent and added as integers (`bits`: log2 of the terms of a lane plus 5),
-// or, where one is float64, all as float64 in a fixed order.  v: two parts per lane.
-__device__ __forceinline__ RsPart rs_warp_parts(const RsPart (&v)[2], int bits) {
-  RsPart t;
-  t.pad = 0;
-  const bool raw = v[0].eg == kRsRaw || v[1].eg == kRsRaw;
-  if (__any_sync(0xffffffffu, raw)) {
-    double g = 0.0, d = 0.0;
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (v[u].eg == -kRsRaw) continue;
-      const bool f = v[u].eg == kRsRaw;
-      g += f ? __longlong_as_double(v[u].g) : rs_double(v[u].g, v[u].eg);
-      d += f ? __longlong_as_double(v[u].d) : rs_double(v[u].d, v[u].ed);
-    }
-    t.g = __double_as_longlong(rs_xor_sum(g, 16));
-    t.d = __double_as_longlong(rs_xor_sum(d, 16));
-    t.eg = t.ed = kRsRaw;
+// The warp's sum of two terms per lane, |v| <= 2^56, identical in every lane: brought to the
+// largest exponent and added as integers, or, where one is float64, all as float64 in a fixed
+// order.
+__device__ __forceinline__ RsSum rs_warp_terms(const RsSum& a, const RsSum& b) {
+  RsSum t = rs_none();
+  if (__any_sync(0xffffffffu, a.e == kRsRaw || b.e == kRsRaw)) {
+    auto f = [](const RsSum& s) {
+      return s.e == kRsRaw ? __longlong_as_double(s.v) : s.v ? rs_double(s.v, s.e) : 0.0;
+    };
+    t.v = __double_as_longlong(rs_xor_sum(f(a) + f(b), 16));
+    t.e = kRsRaw;
     return t;
   }
-  const int mg = __reduce_max_sync(0xffffffffu, max(v[0].eg, v[1].eg));
-  const int md = __reduce_max_sync(0xffffffffu, max(v[0].ed, v[1].ed));
-  t.g = rs_warp_sum(rs_round(v[0].g, mg - v[0].eg + bits) + rs_round(v[1].g, mg - v[1].eg + bits));
-  t.d = rs_warp_sum(rs_round(v[0].d, md - v[0].ed + bits) + rs_round(v[1].d, md - v[1].ed + bits));
-  t.eg = mg == -kRsRaw ? mg : mg + bits;
-  t.ed = md == -kRsRaw ? md : md + bits;
+  t.e = __reduce_max_sync(0xffffffffu, max(a.e, b.e));
+  t.v = rs_warp_sum(rs_round(a.v, t.e - a.e) + rs_round(b.v, t.e - b.e));
   return t;
 }
 
-__device__ __forceinline__ RsPart rs_no_part() {
-  RsPart t;
-  t.g = t.d = t.pad = 0;
-  t.eg = t.ed = -kRsRaw;
-  return t;
-}
-
-// After the wait, every warp: the sum of its share of the G parts of set seq & 1 into
+// After the wait, every warp: the sums of its share of the G parts of set seq & 1 into
 // s_warp (then a block barrier).
-__device__ __forceinline__ void rs_read_parts(const RsPart* parts, int G, unsigned seq, RsPart* s_warp) {
-  const int4* set = reinterpret_cast<const int4*>(parts + (size_t)(seq & 1) * G);
-  RsPart v[2];
+__device__ __forceinline__ void rs_read_parts(const RsSum* parts, int G, unsigned seq,
+                                              RsSum (*s_warp)[kRsThreads / 32]) {
+  const RsSum* set = parts + 2 * (size_t)(seq & 1) * G;
+  RsSum v[2][2];
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int i = threadIdx.x + u * kRsThreads;
-    v[u] = rs_no_part();
-    if (i < G) {
-      reinterpret_cast<int4*>(&v[u])[0] = __ldcg(set + 2 * i);
-      reinterpret_cast<int4*>(&v[u])[1] = __ldcg(set + 2 * i + 1);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      v[k][u] = rs_none();
+      if (i < G) reinterpret_cast<int4&>(v[k][u]) = __ldcg(reinterpret_cast<const int4*>(set + 2 * i + k));
     }
   }
-  const RsPart t = rs_warp_parts(v, 6);
-  if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = t;
+  const RsSum g = rs_warp_terms(v[0][0], v[0][1]), d = rs_warp_terms(v[1][0], v[1][1]);
+  if ((threadIdx.x & 31) == 0) {
+    s_warp[0][threadIdx.x >> 5] = g;
+    s_warp[1][threadIdx.x >> 5] = d;
+  }
 }
 
 // Warp 0, after that barrier: the sums, identical in every lane and every block.
-__device__ __forceinline__ double2 rs_sums(const RsPart* s_warp) {
-  const int lane = threadIdx.x & 31;
-  RsPart v[2] = {rs_no_part(), rs_no_part()};
-  if (lane < kRsThreads / 32) v[0] = s_warp[lane];
-  const RsPart t = rs_warp_parts(v, 5);
-  if (t.eg == kRsRaw) return make_double2(__longlong_as_double(t.g), __longlong_as_double(t.d));
+__device__ __forceinline__ double2 rs_sums(const RsSum (*s_warp)[kRsThreads / 32]) {
+  const RsSum t = rs_over_warps(s_warp);
   // both conversions in one warp instruction
-  const double x = rs_double(lane == 0 ? t.g : t.d, lane == 0 ? t.eg : t.ed);
-  return make_double2(__shfl_sync(0xffffffffu, x, 0), __shfl_sync(0xffffffffu, x, 1));
+  const double x = t.e == kRsRaw ? __longlong_as_double(t.v) : t.v ? rs_double(t.v, t.e) : 0.0;
+  return make_double2(__shfl_sync(0xffffffffu, x, 0), __shfl_sync(0xffffffffu, x, 8));
 }
 
 // 19-point A-stencil at offset 0 of P with strides (1, ey, ez).  `shallow`: the seven
@@ -259,12 +289,12 @@ __device__ __forceinline__ long long rs_stencil_fx(const long long* P, int ey, i
 // else they are in shared memory.
 template <bool ONE>
 __global__ void __launch_bounds__(kRsThreads, 2)
-    k_cg_resident(const ResidentDesc D, CGState* st, RsPart* parts, unsigned* counter, int* err) {
+    k_cg_resident(const ResidentDesc D, CGState* st, RsSum* parts, unsigned* counter, int* err) {
   extern __shared__ __align__(16) double s_vec[];
   __shared__ double s_park[2 * kRsThreads];
   __shared__ uint4 s_mag[kRsThreads / 128];
-  __shared__ long long s_sum[2][kRsThreads / 32];
-  __shared__ RsPart s_warp[kRsThreads / 32];
+  // r.r and w.r of each warp: of its nodes, then of its share of the blocks
+  __shared__ RsSum s_warp[2][kRsThreads / 32];
   __shared__ int s_ok;
   __shared__ double s_alpha, s_beta;
   __shared__ int s_stop;
@@ -398,8 +428,9 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     __syncthreads();
     return E;
   };
-  // w = A r of the box (published to Wn), and the block's sums of r.r and w.r in thread 0
-  auto apply = [&](int E, double* Wn) -> RsPart {
+  // w = A r of the box (published to Wn), and the block's sums of r.r and w.r in lanes 0 and 8
+  // of warp 0
+  auto apply = [&](int E, double* Wn) -> RsSum {
     double acc_g = 0.0, acc_d = 0.0;
     const int qL = fx_sum_exp(FW.k, E) - 1;
     each([&](const Own& n, double& r, double&, double&, double&, double& w) {
@@ -411,33 +442,27 @@ __global__ void __launch_bounds__(kRsThreads, 2)
       acc_d = fma(w, r, acc_d);
       __stcg(Wn + n.o, w);
     });
-    RsPart part;
-    part.pad = 0;
+    RsSum part = rs_none();
     if (E < 0) {
       const double2 t = rs_block_sum2(acc_g, acc_d, s_park, nw_own);
-      part.g = __double_as_longlong(t.x);
-      part.d = __double_as_longlong(t.y);
-      part.eg = part.ed = kRsRaw;
+      part.v = __double_as_longlong((threadIdx.x & 31) < 8 ? t.x : t.y);
+      part.e = kRsRaw;
       return part;
     }
-    // bounds of a thread's sums: up to 16 nodes, |r| < 2^(E - 1022), |w| < 2^(qL + 63)
-    const int eg = 1022 + 2 * (E - 1022) + 4, ed = 1022 + (E - 1022) + (qL + 63) + 4;
-    const long long sg = rs_warp_sum(rs_fixed(acc_g, eg)), sd = rs_warp_sum(rs_fixed(acc_d, ed));
+    // the warp's sums, at the exponents of its largest terms
+    auto expo = [](double x) { return (__double2hiint(x) >> 20) & 0x7ff; };
+    const int xg = __reduce_max_sync(0xffffffffu, expo(acc_g)), xd = __reduce_max_sync(0xffffffffu, expo(acc_d));
+    const long long sg = rs_warp_sum(rs_fixed(acc_g, xg)), sd = rs_warp_sum(rs_fixed(acc_d, xd));
     if ((threadIdx.x & 31) == 0) {
-      s_sum[0][threadIdx.x >> 5] = rs_round(sg, 3);
-      s_sum[1][threadIdx.x >> 5] = rs_round(sd, 3);
+      part.v = sg;
+      part.e = sg ? xg - 1022 - kRsBits : -kRsRaw;
+      s_warp[0][threadIdx.x >> 5] = part;
+      part.v = sd;
+      part.e = sd ? xd - 1022 - kRsBits : -kRsRaw;
+      s_warp[1][threadIdx.x >> 5] = part;
     }
     __syncthreads();
-    part.g = part.d = 0;
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int w = 0; w < kRsThreads / 32; ++w) {
-        part.g += s_sum[0][w];
-        part.d += s_sum[1][w];
-      }
-    }
-    part.eg = eg - 1022 - kRsBits + 3;
-    part.ed = ed - 1022 - kRsBits + 3;
+    if (threadIdx.x < 32) part = rs_norm(rs_over_warps(s_warp));
     return part;
   };
   // the published r, w, s of up to kRsHB halo nodes per thread, loaded right after each
@@ -481,7 +506,7 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     RI[e] = __double_as_longlong(v);
     mag = max(mag, fx_mag(v));
   }
-  RsPart part = apply(fill(mag, hr), D.w0);
+  RsSum part = apply(fill(mag, hr), D.w0);
   // CG scalars: warp 0 keeps identical copies in all its lanes (and in every block)
   double gam = S->rr, alpha = 0.0, beta = 0.0, delta = 0.0;
   const double tol2 = S->tol2;

@@ -208,3 +208,56 @@ def test_residual_slab_taken_again(X, value):
     c0 = 8 * sum(1.0 / v ** 2 for v in O.meshsizes(L, N))
     assert np.all(np.abs(r1 - r0)[~bad] <= 2 * 2.0 ** -50 * 3 * c0 * np.max(np.abs(np.where(bad, 0.0, u))))
     assert not np.isfinite(rn)  # 1e290: the square overflows
+
+
+def stencil(v, h):
+    """A v on the interior of a node array, in the array's own precision."""
+    a, b, c = (np.longdouble(1) / np.longdouble(t) ** 2 for t in h)
+    nz, ny, nx = v.shape
+
+    def s(i, j, k):
+        return v[1 + k:nz - 1 + k, 1 + j:ny - 1 + j, 1 + i:nx - 1 + i]
+
+    sx, sy, sz = s(-1, 0, 0) + s(1, 0, 0), s(0, -1, 0) + s(0, 1, 0), s(0, 0, -1) + s(0, 0, 1)
+    exy = s(-1, -1, 0) + s(1, -1, 0) + s(-1, 1, 0) + s(1, 1, 0)
+    exz = s(-1, 0, -1) + s(1, 0, -1) + s(-1, 0, 1) + s(1, 0, 1)
+    eyz = s(0, -1, -1) + s(0, 1, -1) + s(0, -1, 1) + s(0, 1, 1)
+    return (8 * (a + b + c) * s(0, 0, 0) - (4 * a - b - c) * sx - (4 * b - a - c) * sy - (4 * c - a - b) * sz
+            - ((a + b) * exy + (a + c) * exz + (b + c) * eyz) / 2)
+
+
+@pytest.mark.parametrize("n", [16, 32, 64])
+@pytest.mark.parametrize("kind", ["normal", "sine", "peak", "corner"])
+def test_resident_cg_scalars(X, kind, n):
+    """r.r and w.r of the shared-memory CG, through the first step from zero: x_1 = a r_0 gives
+    a = r_0.r_0 / r_0.A r_0, and the history r_1.r_1 of r_1 = r_0 - a A r_0.  The sums: 2^-50 of
+    themselves (eight roundings in a row).  The terms: A r_0 is off by 2^-50 of its
+    neighbourhood's values times the weights at most, r_1 by as much times a."""
+    N, L = (n, n, n), (1.0, 1.0, 1.0)
+    i, j, k = np.meshgrid(*[np.arange(n + 1)] * 3, indexing="ij")
+    f = {"normal": lambda: np.random.default_rng(12).standard_normal(i.shape),
+         "sine": lambda: np.sin(np.pi * i / n) * np.sin(np.pi * j / n) * np.sin(np.pi * k / n),
+         "peak": lambda: 1.0 * ((i == n // 2) & (j == n // 3) & (k == n // 2 + 1)),
+         "corner": lambda: np.exp(-0.4 * (i + j + k))}[kind]()
+    zero = torch.zeros((n + 1,) * 3, dtype=torch.float64, device="cuda")
+    r0 = X.residual(dev(f), zero, L)[0].cpu().numpy()
+    u = zero.clone()
+    st = X.cg(dev(f), u, L, eps=0.0, fixed_iters=[1], history=2, profile=1)
+    assert "cg_resident_f64" in st["profile"]
+    u = u.cpu().numpy()
+    at = np.unravel_index(np.argmax(np.abs(r0)), r0.shape)
+    alpha = np.longdouble(u[at]) / np.longdouble(r0[at])
+    inner = (slice(1, -1),) * 3
+    r = r0.astype(np.longdouble)
+    w = stencil(r, [1.0 / n] * 3)
+    c0 = 24.0 * n * n
+    dw = 2.0 ** -50 * 3 * c0 * near(r0, 4)[inner]
+    want = np.sum(r * r) / np.sum(r[inner] * w)
+    tol = 3 * 2.0 ** -50 + np.sum(np.abs(r0[inner]) * dw) / np.sum(r[inner] * w)
+    assert abs(alpha / want - 1) <= tol
+    # the history's entries are sqrt(r_k.r_k / b.b), and r_0 = b here
+    r1 = r[inner] - alpha * w
+    g1 = np.sum(r1 * r1)
+    dr = alpha * dw + 2.0 ** -52 * (np.abs(r0[inner]) + np.abs(r1))
+    got = np.longdouble(st["history"][1]) ** 2 * np.sum(r * r)
+    assert abs(got - g1) <= 8 * 2.0 ** -50 * g1 + 2 * np.sum(np.abs(r1) * dr) + np.sum(dr * dr)
