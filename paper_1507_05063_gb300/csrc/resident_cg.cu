@@ -285,6 +285,21 @@ __device__ __forceinline__ long long rs_stencil_fx(const long long* P, int ey, i
   return fx_weigh((EXY + EXZ - Q) + 10 * SX, (EXY + EYZ - Q) + 10 * SY, (EXZ + EYZ - Q) + 10 * SZ, W);
 }
 
+// Whether a node and its six neighbours, integers of the box's scale, all lie more than kFxRange
+// powers of two below it (|v| < 2^(kFxBits - 1 - kFxRange), in either sign): by the high words,
+// and by the low ones where those leave it open.  (With four neighbours white noise took a
+// block to float64 every few steps.)
+__device__ __forceinline__ bool rs_far_below(const long long* P, int ey, int ez) {
+  constexpr int T = 1 << (kFxBits - 1 - kFxRange - 32);
+  auto hi = [&](int o) { return (int)(P[o] >> 32); };
+  const int top = max(hi(0), max(max(max(hi(-1), hi(1)), max(hi(-ey), hi(ey))), max(hi(-ez), hi(ez))));
+  const int low = min(hi(0), min(min(min(hi(-1), hi(1)), min(hi(-ey), hi(ey))), min(hi(-ez), hi(ez))));
+  if (top >= T || low < -T) return false;
+  if (low > -T) return true;
+  constexpr long long t = -((long long)T << 32);
+  return !(P[0] == t || P[-1] == t || P[1] == t || P[-ey] == t || P[ey] == t || P[-ez] == t || P[ez] == t);
+}
+
 // ONE: boxes of at most one node per thread, whose vectors stay in the threads' registers;
 // else they are in shared memory.
 template <bool ONE>
@@ -346,6 +361,8 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     if (ONE) {
       if (mine.valid) f(mine, xr, xx, xp, xs, xw);
     } else {
+      // (unrolled, the stencil's loop: 11.7 us a step on 64^3, 11.3 as it is)
+#pragma unroll 1
       for (int q = threadIdx.x; q < B; q += kRsThreads) {
         const Own n = own_node(q);
         if (n.valid) f(n, R[q], X[q], P[q], Sv[q], W[q]);
@@ -400,9 +417,31 @@ __global__ void __launch_bounds__(kRsThreads, 2)
       if (interior(gi, gj, gk)) ho[u] = gi + gj * g.sy + gk * g.sz;
     }
   }
-  // The box of integers from the new r: own (each thread its r), halo hn (and, of shells of
-  // more than kRsHB per thread, the float64 bits already in RI); mag: this thread's largest
-  // magnitude word.  Returns the scale E, or -1 for a box of float64 bits.  Two barriers.
+  // The halo's new r of shells of more than kRsHB per thread: value(o) of the interior nodes, as
+  // float64 bits into RI; returns the largest magnitude word.
+  auto shell_rest = [&](auto value) -> unsigned {
+    unsigned m = 0;
+    for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
+      int e, gi, gj, gk;
+      shell_node(h, e, gi, gj, gk);
+      const double v = interior(gi, gj, gk) ? value(gi + gj * g.sy + (long long)gk * g.sz) : 0.0;
+      RI[e] = __double_as_longlong(v);
+      m = max(m, fx_mag(v));
+    }
+    return m;
+  };
+  // put(v) of the new r to the box: own (each thread its r) and halo hn.
+  auto put_box = [&](const double (&hn)[kRsHB], auto put) {
+    each([&](const Own& n, double& r, double&, double&, double&, double&) { RI[n.e] = put(r); });
+#pragma unroll
+    for (int u = 0; u < kRsHB; ++u) {
+      if (u >= slots) break;
+      if (he[u] >= 0) RI[he[u]] = put(hn[u]);
+    }
+  };
+  // The box of integers from the new r: own, halo hn (and, of larger shells, the float64 bits
+  // already in RI); mag: this thread's largest magnitude word.  Returns the scale E, or -1 for
+  // a box of float64 bits.  Two barriers.
   auto fill = [&](unsigned mag, const double (&hn)[kRsHB]) -> int {
     mag = __reduce_max_sync(0xffffffffu, mag);
     if ((threadIdx.x & 31) == 0) reinterpret_cast<unsigned*>(s_mag)[threadIdx.x >> 5] = mag;
@@ -414,12 +453,7 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     const int q = fx_sum_exp(FW.k, E);
     if (E < 600 || E > 1400 || q < -400 || q > 300 || D.float64) E = -1;
     auto put = [&](double v) { return E < 0 ? __double_as_longlong(v) : fx_from_double<kFxBits>(v, E); };
-    each([&](const Own& n, double& r, double&, double&, double&, double&) { RI[n.e] = put(r); });
-#pragma unroll
-    for (int u = 0; u < kRsHB; ++u) {
-      if (u >= slots) break;
-      if (he[u] >= 0) RI[he[u]] = put(hn[u]);
-    }
+    put_box(hn, put);
     for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
       int e, gi, gj, gk;
       shell_node(h, e, gi, gj, gk);
@@ -429,40 +463,51 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     return E;
   };
   // w = A r of the box (published to Wn), and the block's sums of r.r and w.r in lanes 0 and 8
-  // of warp 0
-  auto apply = [&](int E, double* Wn) -> RsSum {
+  // of warp 0.  A box with a node that lies, with its neighbours, far below the box's scale is
+  // taken again in float64, as one without a scale (value: shell_rest's).
+  auto apply = [&](int E, const double (&hn)[kRsHB], auto value, double* Wn) -> RsSum {
+    RsSum part = rs_none();
     double acc_g = 0.0, acc_d = 0.0;
-    const int qL = fx_sum_exp(FW.k, E) - 1;
-    each([&](const Own& n, double& r, double&, double&, double&, double& w) {
-      if (E >= 0)
+    if (E >= 0) {
+      const int qL = fx_sum_exp(FW.k, E) - 1;
+      bool far = false;
+      each([&](const Own& n, double& r, double&, double&, double&, double& w) {
+        far |= rs_far_below(RI + n.e, EX, EX * EY);
         w = fx_scale_neg((double)rs_stencil_fx(RI + n.e, EX, EX * EY, FW), qL);
-      else
-        w = rs_stencil(reinterpret_cast<const double*>(RI) + n.e, EX, EX * EY, A, ONE);
+        acc_g = fma(r, r, acc_g);
+        acc_d = fma(w, r, acc_d);
+        __stcg(Wn + n.o, w);
+      });
+      // the warp's sums, at the exponents of its largest terms
+      auto expo = [](double x) { return (__double2hiint(x) >> 20) & 0x7ff; };
+      const int xg = __reduce_max_sync(0xffffffffu, expo(acc_g)), xd = __reduce_max_sync(0xffffffffu, expo(acc_d));
+      const long long sg = rs_warp_sum(rs_fixed(acc_g, xg)), sd = rs_warp_sum(rs_fixed(acc_d, xd));
+      if ((threadIdx.x & 31) == 0) {
+        part.v = sg;
+        part.e = sg ? xg - 1022 - kRsBits : -kRsRaw;
+        s_warp[0][threadIdx.x >> 5] = part;
+        part.v = sd;
+        part.e = sd ? xd - 1022 - kRsBits : -kRsRaw;
+        s_warp[1][threadIdx.x >> 5] = part;
+      }
+      if (!__syncthreads_or(far)) {
+        if (threadIdx.x < 32) part = rs_norm(rs_over_warps(s_warp));
+        return part;
+      }
+      put_box(hn, [](double v) { return __double_as_longlong(v); });
+      shell_rest(value);
+      __syncthreads();
+      acc_g = acc_d = 0.0;
+    }
+    each([&](const Own& n, double& r, double&, double&, double&, double& w) {
+      w = rs_stencil(reinterpret_cast<const double*>(RI) + n.e, EX, EX * EY, A, ONE);
       acc_g = fma(r, r, acc_g);
       acc_d = fma(w, r, acc_d);
       __stcg(Wn + n.o, w);
     });
-    RsSum part = rs_none();
-    if (E < 0) {
-      const double2 t = rs_block_sum2(acc_g, acc_d, s_park, nw_own);
-      part.v = __double_as_longlong((threadIdx.x & 31) < 8 ? t.x : t.y);
-      part.e = kRsRaw;
-      return part;
-    }
-    // the warp's sums, at the exponents of its largest terms
-    auto expo = [](double x) { return (__double2hiint(x) >> 20) & 0x7ff; };
-    const int xg = __reduce_max_sync(0xffffffffu, expo(acc_g)), xd = __reduce_max_sync(0xffffffffu, expo(acc_d));
-    const long long sg = rs_warp_sum(rs_fixed(acc_g, xg)), sd = rs_warp_sum(rs_fixed(acc_d, xd));
-    if ((threadIdx.x & 31) == 0) {
-      part.v = sg;
-      part.e = sg ? xg - 1022 - kRsBits : -kRsRaw;
-      s_warp[0][threadIdx.x >> 5] = part;
-      part.v = sd;
-      part.e = sd ? xd - 1022 - kRsBits : -kRsRaw;
-      s_warp[1][threadIdx.x >> 5] = part;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) part = rs_norm(rs_over_warps(s_warp));
+    const double2 t = rs_block_sum2(acc_g, acc_d, s_park, nw_own);
+    part.v = __double_as_longlong((threadIdx.x & 31) < 8 ? t.x : t.y);
+    part.e = kRsRaw;
     return part;
   };
   // the published r, w, s of up to kRsHB halo nodes per thread, loaded right after each
@@ -499,14 +544,9 @@ __global__ void __launch_bounds__(kRsThreads, 2)
     hr[u] = ho[u] >= 0 ? D.r[ho[u]] : 0.0;
     mag = max(mag, fx_mag(hr[u]));
   }
-  for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
-    int e, gi, gj, gk;
-    shell_node(h, e, gi, gj, gk);
-    const double v = interior(gi, gj, gk) ? D.r[gi + gj * g.sy + (long long)gk * g.sz] : 0.0;
-    RI[e] = __double_as_longlong(v);
-    mag = max(mag, fx_mag(v));
-  }
-  RsSum part = apply(fill(mag, hr), D.w0);
+  auto start = [&](long long o) { return D.r[o]; };
+  mag = max(mag, shell_rest(start));
+  RsSum part = apply(fill(mag, hr), hr, start, D.w0);
   // CG scalars: warp 0 keeps identical copies in all its lanes (and in every block)
   double gam = S->rr, alpha = 0.0, beta = 0.0, delta = 0.0;
   const double tol2 = S->tol2;
@@ -578,19 +618,11 @@ __global__ void __launch_bounds__(kRsThreads, 2)
       hn[u] = fma(-a, fma(bt, hs[u], hw[u]), hr[u]);  // 0 where there is no node: hr, hw, hs are
       mag = max(mag, fx_mag(hn[u]));
     }
-    for (int h = threadIdx.x + kRsHB * kRsThreads; h < nshell; h += kRsThreads) {
-      int e, gi, gj, gk;
-      shell_node(h, e, gi, gj, gk);
-      double rn = 0.0;
-      if (interior(gi, gj, gk)) {
-        const long long o = gi + gj * g.sy + (long long)gk * g.sz;
-        rn = fma(-a, fma(bt, __ldcg(Sg + o), __ldcg(Wg + o)), __ldcg(Rg + o));
-      }
-      RI[e] = __double_as_longlong(rn);
-      mag = max(mag, fx_mag(rn));
-    }
+    // (the arrays read here stay as they are until every block has arrived below)
+    auto value = [&](long long o) { return fma(-a, fma(bt, __ldcg(Sg + o), __ldcg(Wg + o)), __ldcg(Rg + o)); };
+    mag = max(mag, shell_rest(value));
     // 3. w = A r, gamma, delta; publish w
-    part = apply(fill(mag, hn), Wn);
+    part = apply(fill(mag, hn), hn, value, Wn);
     // 4. the grid reduction (it also orders every block's publications before the next
     // step's halo loads); the next halo's loads; scalars
     const bool ok = rs_arrive_wait(part, parts, counter, G, seq, err, &s_ok);

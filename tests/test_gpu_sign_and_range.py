@@ -156,11 +156,13 @@ def test_residual_is_accurate_where_values_are_small(X, kind, which):
     assert np.all(np.abs(got - want) <= tol)
 
 
+@pytest.mark.parametrize("N,engine", [(GROUPS_N, "cg_f64"), ((60, 90, 50), "cg_resident_f64"),
+                                      ((20, 24, 40), "cg_resident_f64")])
 @pytest.mark.parametrize("kind", KINDS)
-def test_streaming_cg_is_accurate_where_values_are_small(X, kind):
+def test_cg_is_accurate_where_values_are_small(X, kind, N, engine):
     """Two steps of CG on A u = 0 from an iterate with a large range: x_2 = x_0 + a_0 r_0 + a_1 (r_0 - a_0 A r_0 + b_1 r_0), node by node.  Sixteen
     roundings in a row and the scalars' (some 1e-13 of themselves) on each term."""
-    N, L = GROUPS_N, GROUPS_L
+    L = GROUPS_L
     u0 = ranged(kind, N, 10)
     for a in (u0[0], u0[-1], u0[:, 0], u0[:, -1], u0[:, :, 0], u0[:, :, -1]):
         a[...] = 0.0
@@ -185,7 +187,7 @@ def test_streaming_cg_is_accurate_where_values_are_small(X, kind):
     want = u0 + a0 * r0 + a1 * p1
     u = dev(u0)
     st = X.cg(dev(f), u, L, eps=0.0, fixed_iters=[2], profile=1)
-    assert "cg_f64" in st["profile"]
+    assert engine in st["profile"]
     c0 = 8 * sum(1.0 / v ** 2 for v in h)
     # r_0 is itself off by its neighbourhood's rounding; A r_0 likewise, one node further
     dr = 3 * c0 * near(u0, 4)
