@@ -207,7 +207,10 @@ __device__ void exp_finite_brick(const ProlongDesc& d, long long lb, BrickSmem& 
 constexpr int kBrickBits = 58;  // |w| <= 1.13 2^58, times (278 / 128)^3 after three passes: < 2^61.6
 
 struct BrickFx {
-  uint4 mag[kThreads / 128];      // a magnitude word per warp
+  // the largest magnitude word of each warp's grid-2h values in the brick's four cells, and of
+  // its grid-4h values
+  uint4 cell[kThreads / 32];
+  unsigned mag[kThreads / 32];
   long long w[BZ1 * BY1][BX1];    // u_2h, then the extrapolated values
   long long d[BZ0][BY0][BX0];     // u_2h - u_4h at the grid-4h nodes
   long long x[BZ1 * BY1][BXF];    // after the pass along x
@@ -272,29 +275,47 @@ __device__ bool exp_finite_brick_fx(const ProlongDesc& d, long long lb, BrickFx&
   // grid-2h and grid-4h values (bricks divide the grid in y and z; the last one in x may reach
   // past it: zeros there, in cells that no output takes)
   double v1[kU], v0 = 0.0;
-  unsigned mag = 0, low = 0;
+  unsigned c0 = 0, c1 = 0, c2 = 0, c3 = 0, low = 0;  // of the four cells along x
 #pragma unroll
   for (int u = 0; u < kU; ++u) {
     const int e = tid + u * kThreads, ix = e % BX1, r = e / BX1, jy = r % BY1, kz = r / BY1;
     const int I = 16 * bx + ix;
     v1[u] = e < N1 && I <= n1x ? __ldg(d.u2h + (I + (4 * by + jy) * s1y + (4 * bz + kz) * s1z)) : 0.0;
-    mag = max(mag, fx_mag(v1[u]));
+    const unsigned m = fx_mag(v1[u]);
+    c0 = max(c0, ix < 4 ? m : 0);  // (a node between two cells counts to one)
+    c1 = max(c1, ix >= 4 && ix < 8 ? m : 0);
+    c2 = max(c2, ix >= 8 && ix < 12 ? m : 0);
+    c3 = max(c3, ix >= 12 ? m : 0);
     low |= (unsigned)__double2loint(v1[u]);
   }
   const int i0 = tid % BX0, j0 = (tid / BX0) % BY0, k0 = tid / (BX0 * BY0);
   const bool has0 = tid < N0 && 8 * bx + i0 <= n0x;
   if (has0) v0 = __ldg(d.u4h + (8 * bx + i0 + (2 * by + j0) * s0y + (2 * bz + k0) * s0z));
-  mag = max(mag, fx_mag(v0));
+  unsigned mag = fx_mag(v0);
   low |= (unsigned)__double2loint(v0);
+  c0 = __reduce_max_sync(0xffffffffu, c0);
+  c1 = __reduce_max_sync(0xffffffffu, c1);
+  c2 = __reduce_max_sync(0xffffffffu, c2);
+  c3 = __reduce_max_sync(0xffffffffu, c3);
   mag = __reduce_max_sync(0xffffffffu, mag);
-  if (mag == 0) mag = __any_sync(0xffffffffu, low != 0);  // denormal below 2^-1042
+  if ((c0 | c1 | c2 | c3 | mag) == 0) mag = __any_sync(0xffffffffu, low != 0);  // denormal below 2^-1042
   __syncthreads();  // the brick before is done with the shared memory
-  if ((tid & 31) == 0) reinterpret_cast<unsigned*>(S.mag)[tid >> 5] = mag;
+  if ((tid & 31) == 0) {
+    S.cell[tid >> 5] = make_uint4(c0, c1, c2, c3);
+    S.mag[tid >> 5] = mag;
+  }
   __syncthreads();
-  const uint4 a = S.mag[0], b = S.mag[1];
-  mag = max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
+  // (a lane per warp and cell)
+  unsigned near = reinterpret_cast<const unsigned*>(S.cell)[tid & 31];
+  mag = __reduce_max_sync(0xffffffffu, max(near, S.mag[tid & 7]));
   const int E = mag == 0 ? kFxMinExp : (int)(mag >> 20);
   if (E < kFxMinExp || E > kFxMaxExp) return false;
+#pragma unroll
+  for (int o = 4; o < 32; o *= 2) near = max(near, __shfl_xor_sync(0xffffffffu, near, o));
+  // a cell of the grid (and all its values) far below the brick's scale
+  if (32 * bx + 8 * (tid & 3) >= g.nx) near = ~0u;
+  near = __reduce_min_sync(0xffffffffu, near);
+  if (mag != 0 && E - (int)(near >> 20) > kFxRange) return false;
 #pragma unroll
   for (int u = 0; u < kU; ++u) {
     const int e = tid + u * kThreads;
@@ -381,7 +402,8 @@ union BrickAny {
 };
 
 // A brick by fixed point, or in float64 where its values do not allow it (infinities, NaN,
-// extreme exponents).
+// extreme exponents, a cell of grid-2h values all more than 2^kFxRange below the brick's
+// largest: the interpolated values are within 2^-52 of the cell's largest, as in float64).
 __device__ __forceinline__ void exp_finite_any(const ProlongDesc& d, long long lb, BrickAny& S) {
   if (!exp_finite_brick_fx(d, lb, S.fx)) {
     __syncthreads();

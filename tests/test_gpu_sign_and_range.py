@@ -263,3 +263,24 @@ def test_resident_cg_scalars(X, kind, n):
     dr = alpha * dw + 2.0 ** -52 * (np.abs(r0[inner]) + np.abs(r1))
     got = np.longdouble(st["history"][1]) ** 2 * np.sum(r * r)
     assert abs(got - g1) <= 8 * 2.0 ** -50 * g1 + 2 * np.sum(np.abs(r1) * dr) + np.sum(dr * dr)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_exp_finite_is_accurate_where_values_are_small(X, kind):
+    """Every interpolated value within its cell's rounding (the tolerance of a brick of values
+    of one size, on the largest value of the cell and those that share a node with it)."""
+    N = (96, 48, 64)
+    u2 = ranged(kind, tuple(n // 2 for n in N), 13)
+    u4 = np.ascontiguousarray(u2[::2, ::2, ::2]) * (1 + 1e-3)
+    want = O.exp_finite(u2, u4)
+    got = X.exp_finite(dev(u2), dev(u4), (1.0, 1.0, 1.0)).cpu().numpy()
+    m = np.abs(u2)
+    for axis in range(3):  # the largest value of each cell (5 nodes, 4 apart), on its 9 fine nodes
+        m = np.moveaxis(m, axis, -1)
+        cells = np.max([m[..., s:s + m.shape[-1] - 4:4] for s in range(5)], axis=0)
+        fine = np.repeat(cells, 8, axis=-1)
+        last = fine[..., -1:]
+        low = np.concatenate([fine[..., :1], fine], axis=-1)   # a node between two cells: the larger
+        high = np.concatenate([fine, last], axis=-1)
+        m = np.moveaxis(np.maximum(low, high), -1, axis)
+    assert np.all(np.abs(got - want) <= 15 * 11.6 * m * 2.0 ** -53 * 2)
