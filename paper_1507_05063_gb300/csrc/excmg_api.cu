@@ -675,6 +675,7 @@ struct Item {
   CGDesc<float> d32;
   double* rhs_cache;    // MIXED: RHS(f) kept between refinement residuals (NULL: none)
   double eps;           // stop at ||r|| <= eps ||b||
+  int float64;          // 1: its 19-point sums in float64 (float64_sums)
   long long nodes;
   // results
   int iters, refs, status;
@@ -749,6 +750,7 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
     ResDesc r = it.res;
     r.t = make_fx_tiling(r.g, fx_tz);
     it.d64.t = make_fx_tiling(r.g, cg_tz);
+    r.float64 = it.d64.float64 = it.float64;
     r.tile_begin = rtiles;
     if (!it.d64.direct) rtiles += r.t.count();  // DSOLVE levels form their own b
     it.d64.tile_begin = tiles;
@@ -770,7 +772,6 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
       r.tol_b2 = it.eps * it.eps;
       r.tol_r2 = 0.0;
       r.fixed = fixed ? 1 : 0;
-      r.float64 = it.d64.float64 = !fixed && it.eps < kFloat64Eps;
       r.max_iter = fixed ? fixed[a] : o->max_iter;
     }
     it.res = r;
@@ -957,6 +958,24 @@ Shapes level_shapes(const Grid3& g, bool dsolve_level, const excmg_options* o) {
   return sh;
 }
 
+// The tolerance of level l.
+double level_eps(const Prob& p, int l, const excmg_options* o) {
+  const double ratio = o->eps_ratio > 0 ? o->eps_ratio : 1.0;
+  if (!p.cascade) return o->eps;
+  return l < 2 ? o->eps_coarse : o->eps * std::pow(ratio, (double)((int)p.lv.size() - 1 - l));
+}
+
+// Whether level l takes its 19-point sums in float64 (kFloat64Eps): decided once for the
+// levels that follow each other in a solve, by the tightest of their tolerances, so that one
+// solve has one arithmetic; levels 0 and 1 (DSOLVE by CG) also by their own.  Exact step
+// counts are no tolerance.
+bool float64_sums(const Prob& p, int l, const excmg_options* o) {
+  if (o->fixed_iters) return false;
+  double tight = level_eps(p, l, o);
+  for (int k = 2; k < (int)p.lv.size(); ++k) tight = std::min(tight, level_eps(p, k, o));
+  return tight < kFloat64Eps;
+}
+
 Item make_item(Prob& p, int l, int slot, const excmg_options* o) {
   const Grid3 g = p.grid(l);
   const Shapes sh = level_shapes(g, p.cascade && l < 2, o);
@@ -964,8 +983,8 @@ Item make_item(Prob& p, int l, int slot, const excmg_options* o) {
   const Tiling t = make_tiling(g, tz);
   Item it;
   memset(&it, 0, sizeof(it));
-  const double ratio = o->eps_ratio > 0 ? o->eps_ratio : 1.0;
-  it.eps = (l < 2) ? o->eps_coarse : o->eps * std::pow(ratio, (double)((int)p.lv.size() - 1 - l));
+  it.eps = level_eps(p, l, o);
+  it.float64 = float64_sums(p, l, o);
   it.nodes = g.nodes();
   it.res = make_res(g, slot, p.level_u(l), p.fview(l), nullptr);
   it.res.forcing = o->rhs_norm == EXCMG_RHS_NORM_FORCING;
@@ -1047,6 +1066,7 @@ excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
       c.level = l;
       CK(launch_boundary_init(g, p.gview(l), p.level_u(l), c.s));
       std::vector<Item> items{make_item(p, l, slot_of(0, l), &ot)};
+      items[0].float64 = float64_sums(p, l, o);  // (the tolerance of the run is no solve's)
       const int fixed = 3;
       excmg_status e = solve_items(c, items, &ot, state_slots(1), f32 ? nullptr : &fixed);
       if (e != EXCMG_OK) return e;
@@ -1586,7 +1606,6 @@ excmg_status excmg_cg(const excmg_grid* grid, const double* f, const excmg_optio
   p.L = prob_layout(lv, opt->precision == EXCMG_MIXED, false, mixed_min(opt));
   const int l = (int)lv.size() - 1;
   std::vector<Item> items{make_item(p, l, 0, opt)};
-  items[0].eps = opt->eps;
   if (opt->history) {
     c.hist = reinterpret_cast<double*>(p.base + p.L.bytes);
     items[0].res.hist = items[0].d64.hist = c.hist;
@@ -1693,7 +1712,6 @@ excmg_status excmg_adjoint(const excmg_grid* grid, const double* dLdu, const exc
   CK(cudaMemsetAsync(c.counters(), 0, sizeof(unsigned), c.s));
   CK(cudaMemsetAsync(lam, 0, sizeof(double) * nf, c.s));
   Item it = make_item(p, 0, 0, opt);
-  it.eps = opt->eps;
   // b = s = (dL/du) on interior nodes: r = LHS(lambda) + s = s - A lambda
   it.res.f = View{nullptr, 0, 0, 0};
   it.res.src = dLdu;

@@ -25,9 +25,10 @@ constexpr int kFxSlabY = 8;
 // 320 x 255 x 257 cells takes 375 us with three, 620 with four (64 registers, spills;
 // groups of four planes).
 constexpr int kFxBlocks = 3;
-// Float64 solves with a stopping tolerance below this take their sums in float64: the target
-// lies under the rounding of float64 sums, so the step counts and the last digits follow
-// that rounding, and stay float64's own.
+// Solves with a stopping tolerance below this (in either precision; on any of their levels) take
+// the 19-point sums of the residual and of the float64 CG in float64: the target lies under the
+// rounding of float64 sums, so the step counts and the last digits follow that rounding, and
+// stay float64's own.  The initial guess (EXP_finite) follows no tolerance.
 constexpr double kFloat64Eps = 1e-13;
 constexpr int kMaxGrid = 4096;   // cap on persistent grid size (partials per problem)
 #ifndef EXCMG_CLUSTER_MAX_NODES

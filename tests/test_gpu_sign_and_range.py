@@ -284,3 +284,30 @@ def test_exp_finite_is_accurate_where_values_are_small(X, kind):
         high = np.concatenate([fine, last], axis=-1)
         m = np.moveaxis(np.maximum(low, high), -1, axis)
     assert np.all(np.abs(got - want) <= 15 * 11.6 * m * 2.0 ** -53 * 2)
+
+
+def relres_of(X, f, u, L):
+    """||r|| / ||b|| of the iterate u with the sums of a tolerance below 1e-13 (float64)."""
+    return X.cg(f, u.clone(), L, eps=1e-15, max_iter=0, allow_not_converged=True)["relres"][0]
+
+
+def test_tight_mixed_residual_is_float64(X):
+    """MIXED at 1e-14: the outer residual that decides on convergence has the sums of an FP64
+    solve at that tolerance, to the last bit."""
+    N, L = (48, 40, 36), (1.0, 0.9, 1.1)
+    f, u = (dev(a) for a in fields(N, 14, "normal"))
+    st = X.cg(f, u, L, precision="mixed", mixed_min_nodes=1, eps=1e-14, max_refine=4, allow_not_converged=True)
+    assert st["refinements"][0] >= 2
+    assert st["relres"][0] == relres_of(X, f, u, L)
+
+
+def test_one_arithmetic_per_solve(X):
+    """A tolerance below 1e-13 on one level is the whole solve's: here level 2's (eps_ratio), the
+    finest level's start meets its own and is not changed."""
+    N, N0, L = (64, 48, 32), (8, 6, 4), (1.0, 0.9, 1.1)
+    i, j, k = np.meshgrid(*[np.arange(n + 1) / n for n in N], indexing="ij")
+    g = np.exp(i + j + k).transpose(2, 1, 0)
+    f, g = dev(3.1 * g), dev(g)
+    res = X.solve(f, g, L, N0, eps=0.5, eps_ratio=1e-14, max_iter=200, allow_not_converged=True)
+    assert res["stats"]["iters"][3] == 0
+    assert res["stats"]["relres"][3] == relres_of(X, f, res["u"], L)
