@@ -98,8 +98,7 @@ typedef struct {
   int max_refine;          /* MIXED: cap on refinement steps per level */
   const int* fixed_iters;  /* HOST array of `levels` counts or NULL: run exactly that
                               many CG iterations on each level (FP64 only; parity tests) */
-  int tile_z;              /* z-slab depth of the float32 stencil kernels (the float64 ones
-                              take their own model's); 0 = library default */
+  int tile_z;              /* z-slab depth of the stencil kernels; 0 = library default */
   int chunk;               /* CG iterations enqueued between convergence reads; 0 = auto */
   long long mixed_min_nodes; /* MIXED: grids with fewer nodes use float64 CG (latency-
                               bound there, float32 saves nothing); 0 = library default
@@ -138,12 +137,11 @@ typedef struct {
                               wait_timeout_ms, to check that the call returns
                               EXCMG_ERR_TIMEOUT and the context stays usable) */
   int autotune;            /* launch-shape tuning: 1 = before a single solve, time candidate
-                              slab depths of every level's float32 CG engine that the cache
-                              (per level grid, engine class and device, kept for the
-                              process) lacks, and keep the fastest (the float64 kernels
-                              follow their model: their entries hold its depth and times);
-                              0 (default) = use the cache where it holds the level, the
-                              models elsewhere; -1 = the models only.  options.tile_z > 0
+                              slab depths of every level's residual and tiled CG engine that
+                              the cache (per level grid, engine class and device, kept for
+                              the process) lacks, and keep the fastest; 0 (default) = single
+                              solves use the cache where it holds the level, the models
+                              elsewhere; -1 = the models only.  options.tile_z > 0
                               overrides both */
   int res_rows;            /* 0 (default), 1 or 4; other values are EXCMG_ERR_INVALID_ARG.
                               Rows per thread of an earlier residual kernel: accepted, and
@@ -155,9 +153,9 @@ typedef struct {
 typedef struct {
   int N[3];                     /* the level's cells */
   int f32;                      /* 1: its CG is the float32 engine of MIXED inner solves */
-  int res_tz, res_tz_model;     /* residual slab depth (the model's, both) */
+  int res_tz, res_tz_model;     /* residual slab depth: tuned, modelled */
   double res_ms, res_ms_model;  /* one residual launch at each (ms) */
-  int cg_tz, cg_tz_model;       /* slab depth of its CG engine (0: not a tuned engine) */
+  int cg_tz, cg_tz_model;       /* slab depth of its CG engine (0: the engine is not tiled) */
   double cg_ms, cg_ms_model;    /* one CG step at each (ms) */
   int res_rows, res_rows_model; /* rows per thread of its residual launch: 1 */
 } excmg_tuning;

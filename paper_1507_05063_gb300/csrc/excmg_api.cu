@@ -676,6 +676,7 @@ struct Item {
   double* rhs_cache;    // MIXED: RHS(f) kept between refinement residuals (NULL: none)
   double eps;           // stop at ||r|| <= eps ||b||
   int float64;          // 1: its 19-point sums in float64 (float64_sums)
+  int res_tz, cg_tz;    // slab depths of the residual and of the float64 CG; 0: the model's
   long long nodes;
   // results
   int iters, refs, status;
@@ -735,7 +736,8 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
   std::vector<CGState> hs;
   std::vector<ResDesc> hr;
   long long tiles = 0, rtiles = 0;  // CG tiles, residual tiles
-  // one launch serves every problem: they share the depth of their fixed-point slabs
+  // one launch serves every problem: they share the model's depth of their fixed-point slabs
+  // (a lone problem takes its own tuned ones, and the caller's tile_z goes before all)
   std::vector<Grid3> grids;
   for (const Item& it : items)
     if (!it.d64.direct) grids.push_back(it.res.g);
@@ -748,8 +750,9 @@ excmg_status solve_items_impl(const Ctx& c, std::vector<Item>& items, const excm
     it.status = EXCMG_OK;
     it.relres = 0.0;
     ResDesc r = it.res;
-    r.t = make_fx_tiling(r.g, fx_tz);
-    it.d64.t = make_fx_tiling(r.g, cg_tz);
+    const bool own = o->tile_z > 0 || grids.size() == 1;
+    r.t = make_fx_tiling(r.g, own && it.res_tz > 0 ? it.res_tz : fx_tz);
+    it.d64.t = make_fx_tiling(r.g, own && it.cg_tz > 0 ? it.cg_tz : cg_tz);
     r.float64 = it.d64.float64 = it.float64;
     r.tile_begin = rtiles;
     if (!it.d64.direct) rtiles += r.t.count();  // DSOLVE levels form their own b
@@ -937,23 +940,20 @@ bool level_f32(const Grid3& g, bool dsolve_level, const excmg_options* o) {
 // Launch shapes of a level: the caller's tile_z, else the tuned ones (options.autotune
 // >= 0 and a cache entry), else the models.
 struct Shapes {
-  int cg_tz, tma_tz;
+  int res_tz, cg_tz;   // of the fixed-point slabs, 0: their launch's model
+  int f32_tz, tma_tz;  // of the float32 engines: plain, tensor-copy
 };
 Shapes level_shapes(const Grid3& g, bool dsolve_level, const excmg_options* o) {
   Shapes sh;
-  const int tz = choose_tz(g, persistent_grid(1LL << 40), o->tile_z);
-  sh.cg_tz = tz;
-  sh.tma_tz = o->tile_z > 0 ? tz : tma_slab_depth(tz);
+  sh.res_tz = sh.cg_tz = o->tile_z;
+  sh.f32_tz = choose_tz(g, persistent_grid(1LL << 40), o->tile_z);
+  sh.tma_tz = o->tile_z > 0 ? o->tile_z : tma_slab_depth(sh.f32_tz);
+  const bool f32 = level_f32(g, dsolve_level, o);
   excmg_tuning t;
-  if (o->tile_z == 0 && o->autotune >= 0 && tune_lookup(g, level_f32(g, dsolve_level, o), &t)) {
-    // an entry's cg_tz is 0 where the single solve's engine for the grid is not tiled
-    // (resident or cluster): the model's depth stays for the tiled engines of a batch
-    if (t.cg_tz > 0) {
-      if (level_f32(g, dsolve_level, o))
-        sh.tma_tz = t.cg_tz;
-      else
-        sh.cg_tz = t.cg_tz;
-    }
+  if (o->tile_z == 0 && o->autotune >= 0 && tune_lookup(g, f32, &t)) {
+    sh.res_tz = t.res_tz;
+    // (cg_tz is 0 where the single solve's engine for the grid has no slabs)
+    if (t.cg_tz > 0) (f32 ? sh.tma_tz : sh.cg_tz) = t.cg_tz;
   }
   return sh;
 }
@@ -979,12 +979,13 @@ bool float64_sums(const Prob& p, int l, const excmg_options* o) {
 Item make_item(Prob& p, int l, int slot, const excmg_options* o) {
   const Grid3 g = p.grid(l);
   const Shapes sh = level_shapes(g, p.cascade && l < 2, o);
-  const int tz = sh.cg_tz;
-  const Tiling t = make_tiling(g, tz);
+  const Tiling t = make_tiling(g, sh.f32_tz);
   Item it;
   memset(&it, 0, sizeof(it));
   it.eps = level_eps(p, l, o);
   it.float64 = float64_sums(p, l, o);
+  it.res_tz = sh.res_tz;
+  it.cg_tz = sh.cg_tz;
   it.nodes = g.nodes();
   it.res = make_res(g, slot, p.level_u(l), p.fview(l), nullptr);
   it.res.forcing = o->rhs_norm == EXCMG_RHS_NORM_FORCING;
@@ -1030,11 +1031,12 @@ Item make_item(Prob& p, int l, int slot, const excmg_options* o) {
 }
 
 // The tuning pass of options.autotune = 1 (single solves): for every level from 2 up
-// without a cache entry, time the residual and, where the level's CG engine has a slab
-// depth (the float32 tensor-copy engine), three CG steps at candidate depths; each candidate runs on the level's own
-// solution array (overwritten by the solve afterwards: boundary = g, interior = 0 at every
-// start) with CUDA events around every launch.  The fastest depth, and the model's with its
-// time, go to the cache.
+// without a cache entry, time the residual at candidate slab depths and, where the level's CG
+// engine has slabs (the streaming float64 engine above kResidentMaxNodes nodes, or the float32
+// tensor-copy engine), three CG steps; each candidate runs on the level's own solution array
+// (overwritten by the solve afterwards: boundary = g, interior = 0 at every start) with CUDA
+// events around every launch.  The fastest of each, and the model's depth with its time, go to
+// the cache.
 excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
   for (int l = 2; l < (int)p.lv.size(); ++l) {
     const Grid3 g = p.grid(l);
@@ -1050,7 +1052,7 @@ excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
     om.max_refine = 1;
     om.inner_tol = 1e-30;
     const Shapes model = level_shapes(g, false, &om);
-    const bool cg_tiled = f32;
+    const bool cg_tiled = f32 || g.nodes() > kResidentMaxNodes;
     // one run: residual + three CG steps at slab depth tz; returns the mean residual launch
     // and the mean CG step (ms)
     auto run = [&](int tz, double& res_ms, double& step_ms) -> excmg_status {
@@ -1089,23 +1091,27 @@ excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
     t.N[1] = g.ny;
     t.N[2] = g.nz;
     t.f32 = f32 ? 1 : 0;
-    t.res_tz = t.res_tz_model = choose_fx_tz(&g, 1);  // one model for the fixed-point slabs
+    t.res_tz = t.res_tz_model = choose_fx_tz(&g, 1);
     t.res_rows = t.res_rows_model = 1;
-    t.cg_tz = t.cg_tz_model = cg_tiled ? (f32 ? model.tma_tz : model.cg_tz) : 0;
+    t.cg_tz = t.cg_tz_model = cg_tiled ? (f32 ? model.tma_tz : t.res_tz_model) : 0;
     double best_res = 1e300, best_cg = 1e300;
     std::vector<int> cands = {2, 4, 6, 8, 10, 12, 16, 20, 24, 32, 48};
     for (int& c : cands)
-      if (f32 && cg_tiled) c = tma_slab_depth(c);  // CG candidates for the tensor-copy engine
-    cands.push_back(f32 ? model.tma_tz : model.cg_tz);
+      if (f32) c = tma_slab_depth(c);  // CG candidates for the tensor-copy engine
+    cands.push_back(t.res_tz_model);
+    if (f32) cands.push_back(t.cg_tz_model);
     std::sort(cands.begin(), cands.end());
     cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
-    if (!cg_tiled) cands.resize(1);  // one run times the residual
     for (int tz : cands) {
-      if (cg_tiled && (tz < 1 || tz > g.nz + 1)) continue;
+      if (tz < 1 || tz > std::min(g.nz + 1, 256)) continue;
       double rm = 0.0, sm = 0.0;
       excmg_status e = run(tz, rm, sm);
       if (e != EXCMG_OK) return e;
-      if (rm > 0) best_res = std::min(best_res, rm);
+      if (rm > 0 && rm < best_res) {
+        best_res = rm;
+        t.res_tz = tz;
+      }
+      if (tz == t.res_tz_model) t.res_ms_model = rm;
       if (cg_tiled && sm > 0) {
         if (sm < best_cg) {
           best_cg = sm;
@@ -1114,7 +1120,8 @@ excmg_status tune_levels(Prob& p, const excmg_options* o, const Ctx& c0) {
         if (tz == t.cg_tz_model) t.cg_ms_model = sm;
       }
     }
-    t.res_ms = t.res_ms_model = best_res < 1e300 ? best_res : 0.0;
+    t.res_ms = best_res < 1e300 ? best_res : 0.0;
+    if (t.res_ms_model == 0.0) t.res_ms_model = t.res_ms;
     t.cg_ms = best_cg < 1e300 ? best_cg : 0.0;
     tune_store(g, f32, t);
   }

@@ -113,7 +113,7 @@ extern "C" excmg_status excmg_cg_noalloc(const excmg_grid* grid, const double* f
   double* partials = reinterpret_cast<double*>(base + L.partials);
 
   const Grid3 g = make_grid(grid->Nx, grid->Ny, grid->Nz, grid->Lx, grid->Ly, grid->Lz);
-  const Tiling t = make_fx_tiling(g, choose_fx_tz(&g, 1));
+  const Tiling t = make_fx_tiling(g, opt->tile_z > 0 ? opt->tile_z : choose_fx_tz(&g, 1));
   const int nblk = persistent_grid(t.count());
   ResDesc rd;
   memset(&rd, 0, sizeof(rd));

@@ -311,3 +311,33 @@ def test_one_arithmetic_per_solve(X):
     res = X.solve(f, g, L, N0, eps=0.5, eps_ratio=1e-14, max_iter=200, allow_not_converged=True)
     assert res["stats"]["iters"][3] == 0
     assert res["stats"]["relres"][3] == relres_of(X, f, res["u"], L)
+
+
+def test_slab_depth_reaches_the_float64_kernels(X):
+    """options.tile_z moves the slabs of the residual and of the streaming float64 CG (their
+    sums add in another order: other last bits, the same solution), and autotune = 1 times
+    them."""
+    N, L = GROUPS_N, GROUPS_L
+    f, start = (dev(a) for a in fields(N, 15, "normal"))
+    runs = []
+    for tz in (2, 3, 5, 8, 11, 23):
+        u = start.clone()
+        st = X.cg(f, u, L, eps=0.0, fixed_iters=[4], history=1, tile_z=tz, profile=1)
+        assert "cg_f64" in st["profile"]
+        runs.append((u, st["history"][0]))
+    a, ra = runs[0]
+    for b, rb in runs[1:]:
+        assert not torch.equal(a, b)
+        assert torch.max(torch.abs(a - b)) <= 1e-12 * torch.max(torch.abs(a)) and ra == pytest.approx(rb, rel=1e-13)
+    assert len({r for _, r in runs}) > 1
+    N, N0 = (128, 128, 128), (8, 8, 8)
+    i, j, k = np.meshgrid(*[np.arange(n + 1) / n for n in N], indexing="ij")
+    g = dev(np.exp(i + j + k))
+    X.excmg_tuning_clear()
+    X.solve(3.0 * g, g, (1.0, 1.0, 1.0), N0, eps=1e-9, autotune=1)
+    e = {tuple(t["N"]): t for t in X.tuning_entries()}
+    X.excmg_tuning_clear()
+    t = e[N]
+    assert t["cg_tz"] >= 1 and 0 < t["cg_ms"] <= t["cg_ms_model"] * 1.0001
+    assert any(v["res_tz"] != v["res_tz_model"] or v["res_ms"] == v["res_ms_model"] for v in e.values())
+    assert all(0 < v["res_ms"] <= v["res_ms_model"] * 1.0001 for v in e.values())
