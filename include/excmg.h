@@ -103,9 +103,9 @@ typedef struct {
   long long mixed_min_nodes; /* MIXED: grids with fewer nodes use float64 CG (latency-
                               bound there, float32 saves nothing); 0 = library default
                               2^21; 1 = float32 inner solves on every grid */
-  int profile;             /* nonzero: time every kernel launch of excmg_solve / excmg_cg
-                              with CUDA events on the caller's stream (stats.prof_*);
-                              single-problem calls only; adds two event records per launch */
+  int profile;             /* nonzero: time every kernel launch of excmg_solve, excmg_cg and
+                              excmg_solve_batched with CUDA events on the caller's stream
+                              (stats.prof_*); adds two event records per launch */
   int dsolve;              /* excmg_dsolve: how levels 0 and 1 are solved (DSOLVE of
                               Algorithm 1) */
   double eps_ratio;        /* per-level tolerance: level l >= 2 of L levels stops at
@@ -284,8 +284,9 @@ excmg_status excmg_grad(const excmg_grid* grid, const double* u, double* ux, dou
  * finest level.  Problems of 2^18 nodes and more share launches in groups of similar size, up
  * to 2^23 nodes a group; one or two that are left, and grids of 2^23 nodes, run first, one
  * after another, as single solves.  Smaller problems share one batch of launches.
- * With opt->profile every problem of 2^18 nodes and more runs as a single solve.  The results
- * are those of single solves up to rounding.  grids[nprob]: host array; f, g, u: host arrays of device pointers.
+ * The results are those of single solves up to rounding.  grids[nprob]: host array; f, g, u: host
+ * arrays of device pointers.  opt->profile: a launch that several problems share counts to the
+ * first of them in stats (without times per level).
  * opt: shared options (fixed_iters must be NULL).  stats: NULL or host array[nprob].
  * Workspace: excmg_workspace_size_batched().  1 <= nprob <= 128.
  */

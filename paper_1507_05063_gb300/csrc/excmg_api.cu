@@ -335,8 +335,9 @@ struct Prof {
     size_t e0, e1;   // indices into pool
     double nodes;
     bool real;
-    int iter_slot;   // >= 0: nodes are per CG step, times the steps of that state slot
     int level;       // level of the solve the launch worked on (-1: not known)
+    std::vector<std::pair<int, double>> steps;  // CG: a state slot and its problem's nodes, which
+                                                // count once per step (in place of nodes)
   };
   std::vector<cudaEvent_t> pool;
   std::vector<Rec> recs;
@@ -349,6 +350,19 @@ struct Prof {
     pool.push_back(e);
     return pool.size() - 1;
   }
+  static double count(const std::vector<std::pair<int, double>>& steps, const std::vector<CGState>& states) {
+    double n = 0.0;
+    for (const auto& sn : steps)
+      if (sn.first < (int)states.size()) n += sn.second * std::max(states[sn.first].iter, 0);
+    return n;
+  }
+  // The last record's steps, from states read now (a later residual resets them).
+  void settle(const std::vector<CGState>& states) {
+    Rec& r = recs.back();
+    r.nodes = count(r.steps, states);
+    r.real = r.nodes > 0.0;
+    r.steps.clear();
+  }
   // Sum the records into stats after the stream has been synchronised.
   void report(excmg_stats* st, const std::vector<CGState>& states) const {
     if (!st) return;
@@ -357,10 +371,9 @@ struct Prof {
       float ms = 0.f;
       if (cudaEventElapsedTime(&ms, pool[r.e0], pool[r.e1]) != cudaSuccess) continue;
       double nodes = r.nodes;
-      if (r.iter_slot >= 0) {
-        const int steps = r.iter_slot < (int)states.size() ? states[r.iter_slot].iter : 0;
-        if (steps <= 0) continue;
-        nodes *= steps;
+      if (!r.steps.empty()) {
+        nodes = count(r.steps, states);
+        if (nodes <= 0.0) continue;
       }
       st->prof_ms[r.kind] += ms;
       st->prof_launches[r.kind] += 1;
@@ -392,7 +405,7 @@ struct Ctx {
     if (prof->pool[a]) cudaEventRecord(prof->pool[a], s);
     cudaError_t e = fn();
     if (prof->pool[b]) cudaEventRecord(prof->pool[b], s);
-    prof->recs.push_back({kind, a, b, nodes, true, -1, level});
+    prof->recs.push_back({kind, a, b, nodes, true, level, {}});
     return e;
   }
   CGState* st() const { return reinterpret_cast<CGState*>(ws + H.st); }
@@ -515,19 +528,13 @@ excmg_status cg_loop(const Ctx& c, int n, CGDesc<T>* ddesc, long long tiles, int
         if (c.prof->pool[a]) cudaEventRecord(c.prof->pool[a], c.s);
         CK(launch_cg_resident(D, smem, c.st(), pairs, c.bar(), c.bar_err(), c.s));
         if (c.prof->pool[b]) cudaEventRecord(c.prof->pool[b], c.s);
-        c.prof->recs.push_back({EXCMG_K_CG_RESIDENT_F64, a, b, nodes, true, slots[0], c.level});
+        c.prof->recs.push_back({EXCMG_K_CG_RESIDENT_F64, a, b, 0.0, true, c.level, {{slots[0], nodes}}});
       } else {
         CK(launch_cg_resident(D, smem, c.st(), pairs, c.bar(), c.bar_err(), c.s));
       }
       if (c.defer) return EXCMG_OK;
       excmg_status e = read_states(c, nslots, hs);
-      if (e == EXCMG_OK && c.prof) {
-        // states are read now: count the steps before a later residual resets them
-        Prof::Rec& rec = c.prof->recs.back();
-        rec.nodes *= hs[slots[0]].iter;
-        rec.iter_slot = -1;
-        rec.real = hs[slots[0]].iter > 0;
-      }
+      if (e == EXCMG_OK && c.prof) c.prof->settle(hs);
       return e;
     }
   }
@@ -609,24 +616,20 @@ excmg_status cg_loop(const Ctx& c, int n, CGDesc<T>* ddesc, long long tiles, int
     const int kind = small ? (sizeof(T) == 8 ? EXCMG_K_CG_CLUSTER_F64 : EXCMG_K_CG_CLUSTER_F32)
                            : (sizeof(T) == 8 ? EXCMG_K_CG_F64 : EXCMG_K_CG_F32);
     if (c.launches) *c.launches += 1;
-    if (c.prof && n == 1) {
+    if (c.prof) {
       const size_t a = c.prof->event(), b = c.prof->event();
       if (c.prof->pool[a]) cudaEventRecord(c.prof->pool[a], c.s);
       CK(launch());
       if (c.prof->pool[b]) cudaEventRecord(c.prof->pool[b], c.s);
-      c.prof->recs.push_back({kind, a, b, nodes, true, slots[0], c.level});
+      Prof::Rec rec{kind, a, b, 0.0, true, c.level, {}};
+      for (int p = 0; p < n; ++p) rec.steps.push_back({slots[p], (double)((hd[p].g.nx + 1LL) * (hd[p].g.ny + 1) * (hd[p].g.nz + 1))});
+      c.prof->recs.push_back(rec);
     } else {
       CK(launch());
     }
     if (c.defer) return EXCMG_OK;
     excmg_status e = read_states(c, nslots, hs);
-    if (e == EXCMG_OK && c.prof && n == 1) {
-      // states are read now: count the steps before a later residual resets them
-      Prof::Rec& rec = c.prof->recs.back();
-      rec.nodes *= hs[slots[0]].iter;
-      rec.iter_slot = -1;
-      rec.real = hs[slots[0]].iter > 0;
-    }
+    if (e == EXCMG_OK && c.prof) c.prof->settle(hs);
     return e;
   }
   int chunk = chunk0 > 0 ? chunk0 : 4;
@@ -641,8 +644,8 @@ excmg_status cg_loop(const Ctx& c, int n, CGDesc<T>* ddesc, long long tiles, int
         const size_t e0 = prof->event(), e1 = prof->event(), e2 = prof->event();
         CK(launch_cg_step<T>(n, ddesc, tiles, grid, c.st(), c.partials(), c.counters(), c.s,
                              prof->pool[e0], prof->pool[e1], prof->pool[e2]));
-        prof->recs.push_back({kspmv, e0, e1, nodes, true, -1, c.level});
-        prof->recs.push_back({kupd, e1, e2, nodes, true, -1, c.level});
+        prof->recs.push_back({kspmv, e0, e1, nodes, true, c.level, {}});
+        prof->recs.push_back({kupd, e1, e2, nodes, true, c.level, {}});
       } else {
         CK(launch_cg_step<T>(n, ddesc, tiles, grid, c.st(), c.partials(), c.counters(), c.s));
       }
@@ -1138,7 +1141,7 @@ excmg_status run_excmg(std::vector<Prob>& P, const excmg_options* o, double* u_t
   Ctx c = c0;
   c.launches = &launches;
   Prof prof;
-  if (o->profile && np == 1) c.prof = &prof;
+  if (o->profile) c.prof = &prof;  // (a launch shared by a batch counts to its first problem)
   // one CG state per (problem, level); an FP64 solve reads them all once, at the end
   long long max_count = o->max_iter;
   if (o->fixed_iters)
@@ -1277,7 +1280,7 @@ excmg_status run_excmg(std::vector<Prob>& P, const excmg_options* o, double* u_t
   CK(cudaStreamSynchronize(c.s));
   CK(cudaGetLastError());
   std::vector<CGState> hs;
-  if (c.defer || c.prof) {
+  if (c.defer) {  // (else every launch's steps were read with its states)
     excmg_status e = read_states(c, state_slots(np), hs);
     if (e != EXCMG_OK) return e;
   }
@@ -1470,9 +1473,8 @@ excmg_status excmg_solve_batched(int nprob, const excmg_grid* grids, const doubl
   // The problems share the launches of one batch, where the CG of each runs as a team of
   // blocks.  One or two of kBatchSoloNodes nodes and more leave its blocks idle at the
   // barriers, and a grid of kBatchSoloMax fills the GPU: these run one after another with a
-  // single solve's engines (measured at the constants).  A profiled batch runs them so too:
-  // kernel times are a single solve's.  Each problem keeps its own workspace region; the
-  // runs share the header's states in stream order.  The larger problems form teams
+  // single solve's engines (measured at the constants).  Each problem keeps its own workspace
+  // region; the runs share the header's states in stream order.  The larger problems form teams
   // in groups of similar size and at most kBatchGroupNodes nodes: a team keeps its blocks to
   // its end, and in one launch over 64 problems of very different step counts the last ones
   // ran on a few blocks each.
@@ -1482,7 +1484,7 @@ excmg_status excmg_solve_batched(int nprob, const excmg_grid* grids, const doubl
     return (long long)(fl.nx + 1) * (fl.ny + 1) * (fl.nz + 1);
   };
   for (int i = 0; i < nprob; ++i)
-    (finest(i) < kBatchSoloNodes ? small : finest(i) < kBatchSoloMax && !opt->profile ? large : solo).push_back(i);
+    (finest(i) < kBatchSoloNodes ? small : finest(i) < kBatchSoloMax ? large : solo).push_back(i);
   std::stable_sort(large.begin(), large.end(), [&](int a, int b) { return finest(a) > finest(b); });
   std::vector<std::vector<int>> teams;
   for (size_t k = 0; k < large.size();) {

@@ -341,3 +341,28 @@ def test_slab_depth_reaches_the_float64_kernels(X):
     assert t["cg_tz"] >= 1 and 0 < t["cg_ms"] <= t["cg_ms_model"] * 1.0001
     assert any(v["res_tz"] != v["res_tz_model"] or v["res_ms"] == v["res_ms_model"] for v in e.values())
     assert all(0 < v["res_ms"] <= v["res_ms_model"] * 1.0001 for v in e.values())
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_profiled_batch_runs_as_it_does(X, precision):
+    """options.profile changes nothing about a batch: the same launches and the same bits, its
+    problems of 2^18 nodes in teams; a shared launch's time and node-steps count to the
+    group's first problem."""
+    N, N0, L = (64, 64, 64), (8, 8, 8), (1.0, 1.0, 1.0)
+    i, j, k = np.meshgrid(*[np.arange(n + 1) / n for n in N], indexing="ij")
+    batch = []
+    for a in (1.0, 1.3, 0.7):
+        g = np.exp(a * i + j + k)
+        batch.append(X.BatchedProblem(L, N, N0, dev((a * a + 2) * g), dev(g)))
+    kw = dict(eps=1e-9, precision=precision, mixed_min_nodes=1 << 15)
+    plain = X.solve_batched(batch, **kw)
+    prof = X.solve_batched(batch, profile=1, **kw)
+    for a, b in zip(plain["u"], prof["u"]):
+        assert torch.equal(a, b)
+    for a, b in zip(plain["stats"], prof["stats"]):
+        assert a["iters"] == b["iters"] and a["launches"] == b["launches"]
+    p = prof["stats"][0]["profile"]
+    assert not any(s["profile"] for s in prof["stats"][1:]) and not plain["stats"][0]["profile"]
+    steps = sum(st["iters"][l] * ((n := 8 << l) + 1) ** 3 for st in prof["stats"] for l in range(2, 4))
+    assert sum(v["nodes"] for name, v in p.items() if name.startswith("cg_")) == steps
+    assert ("cg_f64" if precision == "fp64" else "cg_f32") in p and "cg_resident_f64" not in p
