@@ -101,12 +101,12 @@ struct FinBeta {
 __device__ __forceinline__ double ldv(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ float ldv(const float* p) { return __ldcg(p); }
 
-// One stencil tile: p_new = r + beta p_old (p = r when first), q = A p_new on the tile's
-// nodes, returns this thread's share of p.q.  `sp` is the block's staging buffer and
-// `buf` its current half (advanced per plane).  All threads of the block must call.
+// One stencil tile of a float32 problem: p_new = r + beta p_old (p = r when first), q = A p_new
+// on the tile's nodes, returns this thread's share of p.q.  `sp` is the block's staging buffer
+// and `buf` its current half (advanced per plane).  All threads of the block must call.
 // The (kTX+2) x (kTY+2) halo plane is staged by the block's threads, at most two
-// elements each; the loads of plane k+1 are issued into registers before the barrier
-// and arithmetic of plane k, so global-memory latency overlaps the stencil work.
+// elements each; the loads of two planes ahead are issued into registers before the barrier
+// and arithmetic of a plane, so global-memory latency overlaps the stencil work.
 constexpr int kStage = (kTX + 2) * (kTY + 2);
 static_assert(kStage <= 2 * kThreads, "a staged plane must need at most two loads per thread");
 
@@ -168,20 +168,14 @@ __device__ __forceinline__ T spmv_tile(const CGDesc<T>& d, long long lt, bool fi
   const T exy = (T)d.A.exy, exz = (T)d.A.exz, eyz = (T)d.A.eyz;
   const T bta = first ? T(0) : beta;
   T Pm1 = T(0), Cm1 = T(0), Tm1 = T(0), Tm2 = T(0), tacc = T(0);
-  // float32 keeps two planes in flight (it is bound by load latency), float64 one (it is
-  // bound by the FP64 pipe and short of registers)
-  constexpr bool kDeep = sizeof(T) == 4;
+  static_assert(sizeof(T) == 4, "float64 takes spmv_slab");
   PlaneLoad<T> nxt, nxt2;
   load_plane(nxt, g, c, c.z0 - 1, first, r, pold);
-  if (kDeep) load_plane(nxt2, g, c, c.z0, first, r, pold);
+  load_plane(nxt2, g, c, c.z0, first, r, pold);
   for (int kk = c.z0 - 1; kk <= c.z1; ++kk) {
     store_plane(nxt, bta, sp[buf]);
-    if (kDeep) {
-      nxt = nxt2;
-      if (kk + 1 < c.z1) load_plane(nxt2, g, c, kk + 2, first, r, pold);
-    } else if (kk < c.z1) {
-      load_plane(nxt, g, c, kk + 1, first, r, pold);
-    }
+    nxt = nxt2;
+    if (kk + 1 < c.z1) load_plane(nxt2, g, c, kk + 2, first, r, pold);
     __syncthreads();
     const T P = sp[buf][ty + 1][tx + 1];
     const T SX = sp[buf][ty + 1][tx] + sp[buf][ty + 1][tx + 2];
