@@ -102,23 +102,25 @@ __device__ __forceinline__ long long fx_mad_s(int a, int b, long long c) {
 // signed, l2 = 2 l); |result| <= 96 2^56 < 2^62.6.  With X = x_h 2^32 + x_l (x_l signed) the sum
 // is t 2^63 + m 2^31 + n, every product one 32 x 32 multiply-add: t = sum x_h h, m = sum x_l h +
 // x_h l2 (< 2^62.9), n = sum x_l l (< 2^62.6).  The whole sum is formed and rounded once, to
-// odd: exact, or the odd one of its two neighbours, so that -X, -Y, -Z give the negative and
-// no rounding has a preferred side.  (A floor, half a unit the same way at every node, is a
-// smooth right-hand side: the solution of the level moved by 1e-14 with it; dropped low
-// products break the symmetry in sign.)
+// nearest, ties to even, so that -X, -Y, -Z give the negative and no rounding has a preferred
+// side.  (A floor, half a unit the same way at every node, is a smooth right-hand side: the
+// solution of the level moved by 1e-14 with it; dropped low products break the symmetry in
+// sign; the odd one of the two neighbours is off by up to a unit, which the residual of a smooth
+// field on unequal meshsizes shows: root mean square 7.7e-13 against 3.9e-13 for exp(x + y + z)
+// on 48 x 100 x 37 cells.)
 __device__ __forceinline__ long long fx_weigh(long long X, long long Y, long long Z, const FxWeights& W) {
   const int xl = (int)X, yl = (int)Y, zl = (int)Z;
   const int xh = (int)(X >> 32) - (xl >> 31), yh = (int)(Y >> 32) - (yl >> 31), zh = (int)(Z >> 32) - (zl >> 31);
   const long long n = fx_mad_s(zl, W.l[2], fx_mad_s(yl, W.l[1], (long long)xl * W.l[0]));
-  long long m = fx_mad_s(xl, W.h[0], n >> 31);
+  long long m = fx_mad_s(xl, W.h[0], (n >> 31) + (1 << 28));  // half a unit
   m = fx_mad_s(yl, W.h[1], m);
   m = fx_mad_s(zl, W.h[2], m);
   m = fx_mad_s(xh, W.l2[0], m);
   m = fx_mad_s(yh, W.l2[1], m);
   m = fx_mad_s(zh, W.l2[2], m);
   const long long t = fx_mad_s(zh, W.h[2], fx_mad_s(yh, W.h[1], (long long)xh * W.h[0]));
-  const unsigned rest = ((unsigned)m & 0x1fffffffu) | ((unsigned)n & 0x7fffffffu);
-  return ((t << 3) + (m >> 29)) | min(rest, 1u);
+  const unsigned rest = ((unsigned)m & 0x1fffffffu) | ((unsigned)n & 0x7fffffffu);  // 0: a tie
+  return ((t << 3) + (m >> 29)) & ~(long long)(rest == 0);
 }
 
 #endif  // __CUDACC__

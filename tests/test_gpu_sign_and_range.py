@@ -228,6 +228,34 @@ def stencil(v, h):
             - ((a + b) * exy + (a + c) * exz + (b + c) * eyz) / 2)
 
 
+def stencil_rhs(f):
+    """RHS(f) on the interior of a node array, in the array's own precision."""
+    c = f[1:-1, 1:-1, 1:-1]
+    return 3 * c + ((f[1:-1, 1:-1, :-2] + f[1:-1, 1:-1, 2:]) + (f[1:-1, :-2, 1:-1] + f[1:-1, 2:, 1:-1])
+                    + (f[:-2, 1:-1, 1:-1] + f[2:, 1:-1, 1:-1])) / 2
+
+
+@pytest.mark.parametrize("N", [(48, 100, 37), (20, 70, 23), (100, 24, 50)])
+def test_residual_of_a_smooth_field_rounds_to_nearest(X, N):
+    """Values within 2^3 of a slab's largest are exact as integers, so r is off by half a unit of
+    the weighted sum (2^-57 of the powers of two above the largest value and weight) and the
+    float64 roundings of the two sums and their difference."""
+    L = (1.0, 1.0, 1.0)
+    i, j, k = np.meshgrid(*[np.arange(n + 1) / n for n in N], indexing="ij")
+    u = np.exp(i + j + k).transpose(2, 1, 0)
+    f = 3.0 * u
+    r = X.residual(dev(f), dev(u), L)[0].cpu().numpy()[1:-1, 1:-1, 1:-1]
+    h = O.meshsizes(L, N)
+    # the weights 1/h^2 as float64 has them: stencil() squares and divides in long double
+    w = [1.0 / (t * t) for t in h]
+    lhs = -stencil(u.astype(np.longdouble), [1 / np.sqrt(np.longdouble(t)) for t in w])
+    rhs = -stencil_rhs(f.astype(np.longdouble))
+    unit = 2.0 ** (np.frexp(max(w))[1] + np.frexp(np.max(u))[1] - 57)
+    tol = 0.5 * unit * (1 + 2.0 ** -8) + 2.0 ** -52 * (np.abs(lhs) + np.abs(rhs))
+    tol += 32 * np.finfo(np.longdouble).eps * 8 * sum(w) * np.abs(u[1:-1, 1:-1, 1:-1])  # the reference's own
+    assert np.all(np.abs(r - (lhs + rhs)) <= tol)
+
+
 @pytest.mark.parametrize("n", [16, 32, 64])
 @pytest.mark.parametrize("kind", ["normal", "sine", "peak", "corner"])
 def test_resident_cg_scalars(X, kind, n):
