@@ -273,7 +273,7 @@ __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, 
       __syncthreads();
       const int was = R.scale;
       if (!R.next(S.mag[0])) return false;
-      held = R.near(S.mag[0]);
+      held = R.near(S.mag[0], kFxRangeCG);
       const int sc = R.scale;
       if (sc != was) M.rescale(was - sc);
       store_box(S.box, p, C, [&](double v) { return fx_from_double<kFxBits>(v, sc); });

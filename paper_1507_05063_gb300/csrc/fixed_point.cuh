@@ -38,6 +38,15 @@ constexpr int kFxMinExp = 200, kFxMaxExp = 1800;
 // 64^3 cells 2.1, 0.4 / 6e15, 5e14 / 1.9, 0.4; exp(-100 x) on 128 x 40 x 40 0.6, 0.3 / 2e9, 3e8 /
 // 0.6, 0.3; exp(4 (x + y + z)) on 48^3, 2 wide, 0.9, 0.24 / 69, 4.3 / 4.8, 0.33.
 constexpr int kFxRange = 6;
+// ... of the vectors of CG (p in slabs, r in the shared-memory boxes): held to 2^-46 of the largest
+// value near them then, below what a solve that takes integers can ask for (1e-13, kFloat64Eps),
+// and in norm the error stays 2^-57 of the largest value.  2^6 sent vectors of ordinary solves to
+// float64: they are small where boundary planes or zeros of the data meet, and r after EXP_finite
+// in the middle of a cell.  2^6 / 2^10: six solves of 128^3 cells with sums of sines, one batch,
+// 27.5 / 21.9 ms (20.0 without a check); 128^3 with u = exp(-100 x) 26.8 / 22.8 ms (16.0; 41.4 in
+// float64).  Shared-memory CG, the levels of a 512 x 256 x 128 solve at 1e-12: 3.7 ms with 2^6, 2.40
+// with 2^8, 2.31 with 2^10, 2.30 with 2^14.
+constexpr int kFxRangeCG = 10;
 
 #ifdef __CUDACC__
 

@@ -168,15 +168,15 @@ struct FxRange {
   }
   // (After next.)  Whether the group's and the previous group's values are held near their own
   // size: false, in every thread, if all values of a neighbourhood (of three columns, three rows and four
-  // planes) lie more than kFxRange powers of two below the scale, in a group that is not all
+  // planes) lie more than `range` powers of two below the scale, in a group that is not all
   // zero.
-  __device__ __forceinline__ bool near(const FxMags& S) {
+  __device__ __forceinline__ bool near(const FxMags& S, int range) {
     const unsigned l = S.low[threadIdx.x & 7], h = l == ~0u ? 0 : l;
     // a row's neighbourhoods, or those of a row beside it
     const unsigned h3 = max(h, max(__shfl_up_sync(0xffffffffu, h, 1, 8), __shfl_down_sync(0xffffffffu, h, 1, 8)));
     const int was = low;
     low = (int)(__reduce_min_sync(0xffffffffu, l == ~0u || E == 0 ? ~0u : h3) >> 20);
-    return scale - min(low, was) <= kFxRange;
+    return scale - min(low, was) <= range;
   }
 };
 

@@ -41,13 +41,6 @@ namespace {
 
 constexpr int kRsThreads = 256;
 constexpr unsigned long long kRsSpinLimit = 1ull << 25;
-// A node and its six neighbours may be this many powers of two below the box's scale: r is held
-// to 2^-57 of the scale, 2^-46 of the largest r near it then -- below what a solve that takes
-// integers can ask for (1e-13, kFloat64Eps), and in norm the error stays 2^-57 of the box's
-// largest r.  The residual's 2^6 would take boxes of ordinary solves to float64 in most steps
-// (r after EXP_finite is small in the middle of a cell): the levels of a 512 x 256 x 128 solve at
-// 1e-12 3.7 ms with 2^6, 2.40 with 2^8, 2.31 with 2^10, 2.30 with 2^14.
-constexpr int kRsRange = 10;
 constexpr int kRsHB = 6;  // halo nodes per thread whose loads are issued ahead
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
@@ -292,12 +285,12 @@ __device__ __forceinline__ long long rs_stencil_fx(const long long* P, int ey, i
   return fx_weigh((EXY + EXZ - Q) + 10 * SX, (EXY + EYZ - Q) + 10 * SY, (EXZ + EYZ - Q) + 10 * SZ, W);
 }
 
-// Whether a node and its six neighbours, integers of the box's scale, all lie more than kRsRange
-// powers of two below it (|v| < 2^(kFxBits - 1 - kRsRange), in either sign): by the high words,
+// Whether a node and its six neighbours, integers of the box's scale, all lie more than kFxRangeCG
+// powers of two below it (|v| < 2^(kFxBits - 1 - kFxRangeCG), in either sign): by the high words,
 // and by the low ones where those leave it open.  (With four neighbours white noise took a
 // block to float64 every few steps.)
 __device__ __forceinline__ bool rs_far_below(const long long* P, int ey, int ez) {
-  constexpr int T = 1 << (kFxBits - 1 - kRsRange - 32);
+  constexpr int T = 1 << (kFxBits - 1 - kFxRangeCG - 32);
   auto hi = [&](int o) { return (int)(P[o] >> 32); };
   const int top = max(hi(0), max(max(max(hi(-1), hi(1)), max(hi(-ey), hi(ey))), max(hi(-ez), hi(ez))));
   const int low = min(hi(0), min(min(min(hi(-1), hi(1)), min(hi(-ey), hi(ey))), min(hi(-ez), hi(ez))));

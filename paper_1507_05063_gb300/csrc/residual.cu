@@ -200,7 +200,7 @@ __device__ __noinline__ bool residual_slab(const ResDesc& d, const FxSlab c, Res
       } else {
         const int was = V.scale;
         if (!V.next(S.u.mag[1])) return false;
-        held = V.near(S.u.mag[1]);
+        held = V.near(S.u.mag[1], kFxRange);
         const int sf = V.scale;
         if (sf != was) {
           f1 = (FT)fx_shift((long long)f1, was - sf);
@@ -220,7 +220,7 @@ __device__ __noinline__ bool residual_slab(const ResDesc& d, const FxSlab c, Res
     } else {
       const int was = U.scale;
       if (!U.next(S.u.mag[0])) return false;
-      held = held & U.near(S.u.mag[0]);
+      held = held & U.near(S.u.mag[0], kFxRange);
       const int su = U.scale;
       if (su != was) M.rescale(was - su);
       store_box(S.u.box, v, C, [&](double x) { return fx_from_double<kFxBits>(x, su); });
