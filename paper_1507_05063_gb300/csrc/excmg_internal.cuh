@@ -327,6 +327,7 @@ cudaError_t launch_prolong_cmp(int points, int nprob, const ProlongDesc* descs,
 cudaError_t launch_exp_true(const Grid3& g, const double* uh, const double* u2h, double* ut,
                             cudaStream_t s);
 cudaError_t launch_boundary_init(const Grid3& g, View gb, double* u, cudaStream_t s);
+cudaError_t launch_timing_field(const Grid3& g, double* u, cudaStream_t s);
 cudaError_t launch_adjoint_finish(const Grid3& g, const Coef& A, const double* lam,
                                   const double* dLdu, double* dLdf, double* dLdg,
                                   cudaStream_t s);

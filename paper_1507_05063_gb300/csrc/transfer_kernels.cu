@@ -539,6 +539,13 @@ __global__ void __launch_bounds__(kThreads) k_boundary_init(Grid3 g, View gb, do
   }
 }
 
+// A field without zeros or layers, for timing: values in [1, 2) from a hash of the node's index.
+__global__ void __launch_bounds__(kThreads) k_timing_field(long long n, double* __restrict__ u) {
+  for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < n;
+       o += (long long)gridDim.x * blockDim.x)
+    u[o] = 1.0 + (double)(((unsigned)o * 2654435761u) >> 8) * 0x1p-24;
+}
+
 // Adjoint outputs from lambda (zero on boundary nodes):
 //   dL/df = -R^T lambda = -(3 lambda_m + (1/2) sum of lambda at the 6 face neighbours)
 //   dL/dg = LHS^T lambda + dL/du on boundary nodes, 0 inside (LHS weights = -A weights).
@@ -647,6 +654,11 @@ cudaError_t launch_exp_true(const Grid3& g, const double* uh, const double* u2h,
 
 cudaError_t launch_boundary_init(const Grid3& g, View gb, double* u, cudaStream_t s) {
   k_boundary_init<<<flat_grid(g.nodes()), kThreads, 0, s>>>(g, gb, u);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_timing_field(const Grid3& g, double* u, cudaStream_t s) {
+  k_timing_field<<<flat_grid(g.nodes()), kThreads, 0, s>>>(g.nodes(), u);
   return cudaGetLastError();
 }
 

@@ -371,6 +371,23 @@ def test_slab_depth_reaches_the_float64_kernels(X):
     assert all(0 < v["res_ms"] <= v["res_ms_model"] * 1.0001 for v in e.values())
 
 
+def test_tuning_times_no_layers_of_its_own(X):
+    """The tuning pass times the slabs on values of one size, whatever g: from a large g on the
+    boundary and zeros inside, slabs next to the boundary took the float64 form, more than twice
+    the time."""
+    N, N0, L = (256, 256, 128), (8, 8, 4), (1.0, 1.0, 1.0)
+    f = dev(np.random.default_rng(16).standard_normal([n + 1 for n in N[::-1]]))
+    times = []
+    for value in (0.0, 1e3):
+        X.excmg_tuning_clear()
+        X.solve(f, torch.full_like(f, value), L, N0, eps=1e-2, autotune=1)
+        times.append({tuple(t["N"]): t for t in X.tuning_entries()}[N])
+        X.excmg_tuning_clear()
+    for key in ("res_ms_model", "cg_ms_model"):
+        a, b = (t[key] for t in times)
+        assert 0 < max(a, b) <= 1.4 * min(a, b)
+
+
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_profiled_batch_runs_as_it_does(X, precision):
     """options.profile changes nothing about a batch: the same launches and the same bits, its
