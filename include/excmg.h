@@ -357,6 +357,12 @@ excmg_status excmg_cg(const excmg_grid* grid, const double* f, const excmg_optio
  * excmg_residual -- r = b - A u_I = LHS(u) - RHS(f) at interior nodes (0 on the
  * boundary), eq. (compact) / (FD), in float64; also returns ||r||_2 and ||b||_2 (b with
  * its Dirichlet lift taken from u's boundary entries) in *rnorm, *bnorm (host).
+ * Accuracy: the sums run on 64-bit integers of the power of two of the largest value of a block
+ * of nodes (34 x 10 x 12 at most) as long as every neighbourhood of 3 x 3 x 4 nodes holds a value
+ * within 2^6 of it, else in float64; a node's r is off by 2^-50 of the values near it times the
+ * weights at most, and residual(-f, -u) is the negative of residual(f, u) to the last bit.  The
+ * float64 CG forms A p likewise, with 2^10 in place of 2^6 (2^-46); solves with a tolerance below
+ * 1e-13 take float64 sums throughout.
  * Workspace: excmg_workspace_size_level().
  */
 excmg_status excmg_residual(const excmg_grid* grid, const double* f, const double* u,

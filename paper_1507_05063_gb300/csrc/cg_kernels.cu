@@ -212,7 +212,9 @@ __device__ __noinline__ double scale_pq(double v, int a, int b) { return v * fx_
 // F64: the sums in float64.  Returns false, in every thread, when a group is not for fixed
 // point (the caller then takes the slab again with F64).  All threads of the block must call.
 // Measured, a whole CG step: 385 x 201 x 121 cells 0.517 ms with the sums in float64 (19
-// float64 instructions per node and step), 0.195 ms here (7.5); 128^3 0.150 ms, 0.055 ms here.
+// float64 instructions per node and step), 0.190 to 0.207 ms here (7.5); 128^3 0.150 ms, 0.058 here.
+// A slab that is taken again in float64 costs both: 20 steps from zero on 385 x 201 x 121 (u = exp(x +
+// y + z): p large beside the boundary) 7.6 ms, 4.15 from an iterate, 10.3 in float64 alone.
 template <bool F64>
 __device__ __noinline__ bool spmv_slab(const CGDesc<double>& d, const FxSlab c, bool first, double beta,
                                        const double* __restrict__ pold, double* __restrict__ pnew, FxSmem& S,

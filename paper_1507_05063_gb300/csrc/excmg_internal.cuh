@@ -39,11 +39,19 @@ constexpr int kMaxGrid = 4096;   // cap on persistent grid size (partials per pr
 #endif
 // grids up to kClusterMaxNodes nodes can run all their CG steps in one thread-block
 // cluster; a single float64 grid of more than kResidentMinNodes nodes takes the resident
-// engine instead (measured faster from about 5,000 nodes: 8.2 vs 8.7 us per step)
+// engine instead.  us per step, cluster / resident: 16 x 8 x 4 cells 3.6 / 4.9, 16 x 8 x 8 3.8 /
+// 4.2, 10 x 12 x 12 (1,859 nodes) 4.2 / 4.5, 24 x 10 x 6 (1,925) 4.9 / 4.2, 12^3 (2,197) 6.1 / 4.5,
+// 16 x 16 x 8 4.9 / 4.4, 16^3 6.8 / 4.5, 32 x 16 x 8 7.9 / 4.5.
 constexpr long long kClusterMaxNodes = EXCMG_CLUSTER_MAX_NODES;
 constexpr long long kResidentMinNodes = EXCMG_RESIDENT_MIN_NODES;
 // MIXED mode solves grids below this many nodes in float64 by default: there CG is
-// latency-bound, float32 saves nothing and refinement would add host round trips.
+// latency-bound, float32 saves little and refinement adds a second residual and host round
+// trips.  What MIXED gains follows the number of steps on the grids above the line.  ms per
+// solve, FP64 / MIXED with the line at 2^19, 2^21, 2^22, 2^24 nodes: u = r^{5/3} on 256 x 128 x 128
+// cells at 1e-9 3.53 / 2.56, 2.53, 2.53, 3.59; 512 x 256 x 128 10.8 / 7.04, 7.08, 8.87, 8.83; the same
+// at 1e-12 84.1 / 35.6, 35.6, 52.3, 53.4; 256^3 at 1e-12 29.9 / 14.2, 14.2, 18.3, 18.5.  A solve whose
+// finest grids take no step loses the second residual: u = e^{x+y+z} at 1e-9, 512 x 256 x 128 1.36 /
+// 1.49 (2^21), 1024 x 512 x 512 7.83 / 8.91.
 constexpr long long kMixedMinNodes = 1LL << 21;
 
 struct Grid3 {
@@ -264,14 +272,14 @@ constexpr long long kResidentMaxNodes = EXCMG_RESIDENT_MAX_NODES;
 // excmg_solve_batched: one or two problems whose finest grid has kBatchSoloNodes nodes or
 // more, and any of kBatchSoloMax, run as single solves, one after another; the others share
 // the batch's launches.  ms for n equal problems of 64^3 / 128x64x32 / 128x128x64 / 128^3 /
-// 256x128x128 cells (eps 1e-8), as single solves: n = 2: 1.08 / 2.45 / 2.49 / 1.67 / 2.35, n =
-// 3: 1.57 / 3.65 / 3.67 / 2.46 / 3.51, n = 6: 3.11 / 7.50 / 7.44 / 4.85 / -; as teams: 1.01 /
-// 2.88 / 2.45 / 1.51 / 2.19, 1.09 / 3.29 / 2.99 / 1.77 / 2.64, 1.46 / 4.50 / 4.41 / 2.68 / -
-// (MIXED the same within 10%).
+// 256x128x128 cells (sums of sines, eps 1e-8), as single solves: n = 2: 2.06 / 3.71 / 7.46 / 7.82 /
+// 21.9, n = 3: 3.23 / 5.90 / 12.3 / 11.6 / 32.7, n = 6: 6.55 / 11.1 / 23.4 / 24.6 / 68.0; as teams:
+// 2.22 / 4.16 / 6.70 / 7.54 / 21.9, 2.86 / 5.78 / 10.7 / 10.2 / 32.7, 3.80 / 7.96 / 17.4 / 21.8 / 68.0.
+// Smooth data, n = 3: 0.78 / 1.04 / 1.03 / 1.15 / 1.47 and 0.43 / 0.69 / 0.67 / 0.68 / 1.48.
 constexpr long long kBatchSoloNodes = 1LL << 18, kBatchSoloMax = 1LL << 23;
 // Teams of one launch: at most this many nodes.  64 problems of 2^15 to 2^24 nodes and very
 // different step counts: 608 ms in one launch, 416 in groups of 2^24 nodes, 378 of 2^23 (377 one
-// by one); 16 of 2^15 to 2^20: 22.9 / 22.9 / 22.5 (30.3).
+// by one); 16 of 2^15 to 2^20: 22.9 / 22.9 / 22.5 (30.3).  (Before the check of small values.)
 constexpr long long kBatchGroupNodes = 1LL << 23;
 struct ResidentDesc {
   Grid3 g;

@@ -27,7 +27,7 @@ constexpr int kFxX = kTX, kFxY = kThreads / 32;
 // Planes per group: 84 rim nodes a plane go to 256 threads, so groups of 3 and 6 planes fill
 // the loads' rounds and others do not, and a deeper group has fewer barriers.  Residual at
 // 320 x 255 x 257 with 3 / 4 / 5 / 6 / 7 / 8 planes: 475 / 455 / 422 / 421 / 452 / 424 us; CG at
-// 385 x 201 x 121, 40 steps: 4.39 / 4.39 / 4.24 / 4.15 / 4.30 / 4.88 ms.
+// 385 x 201 x 121, 40 steps: 4.39 / 4.39 / 4.24 / 4.15 / 4.30 / 4.88 ms (without FxRange's check).
 constexpr int kFxG = 6;
 constexpr int kBoxX = kFxX + 2, kBoxY = kFxY + 2;
 constexpr int kPlane = kBoxX * kBoxY;

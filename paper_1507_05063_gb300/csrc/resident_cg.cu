@@ -26,9 +26,13 @@
 // largest.  A float64 warp instruction takes the pipe 64 clocks whatever its lanes do, so
 // the 19-point sums (fixed_point.cuh) and the reductions run on integers, and float64 is
 // left with the vector updates, the two products and the scalars: 8.5 instructions per node
-// and step instead of 25.  Measured per step, before and after: 16^3 cells 6.1 us, 3.8;
-// 32^3 7.3, 4.5; 64^3 21.9, 10.2; 128 x 128 x 32 36.4, 17.4.  The blocks' sums are read by
-// all warps (one or two per thread): read by one warp, ten per lane, they cost 1.5 us more.
+// and step instead of 25.  Measured per step, all in float64 and now: 16^3 cells 6.2 us, 4.5;
+// 32^3 7.5, 5.2; 64^3 22.0, 11.2; 128 x 64 x 64 37.7, 19.8 (3.8, 4.7, 9.8, 18.0 with sums of fewer
+// bits and no check of small values).  A field that falls off within its boxes has them in float64
+// too: 40 steps from zero on 64^3 with u = exp(-100 x) 1.29 ms, 1.12 in float64 alone (a box that stays
+// in float64 for 1, 3 or 7 steps after one: 1.23, 1.19, 1.17, and whole solves 0 to 4% slower).
+// The blocks' sums are read by all warps (one or two per thread): read by one warp, ten per
+// lane, they cost 1.5 us more.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -733,7 +737,8 @@ bool resident_box(const Grid3& g, ResidentDesc& D, size_t& smem) {
   const long long max_blocks = std::min<long long>((long long)g_rs_sms * g_rs_blocks_per_sm, 2 * kRsThreads);
   // per-step model in SM clocks: the busiest SM's float64 work (~12.5 clocks per node,
   // 2 DFMA per clock, plus ~400 per block for its reduction), the halo loads of a box
-  // (3 per shell node), and the grid reduction's share per block (arrival, partials)
+  // (3 per shell node), and the grid reduction's share per block (arrival, partials).  The
+  // constants are those of the sums in float64 and were not fitted anew to the integer ones.
   double best = 1e300;
   bool found = false;
   const int bxs[] = {32, 16, 8};

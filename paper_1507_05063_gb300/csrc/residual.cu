@@ -5,8 +5,11 @@
 // about 23 float64 instructions per node, 11.5 clocks of an SM at 2 lanes per clock, ten
 // times the 24 bytes a node moves.  Here five remain (the two conversions of the sums, the
 // difference, r.r and RHS.RHS).  Measured, one call on 320 x 255 x 257 cells: 1.11 ms in
-// float64, 0.42 ms here (the kernel 360 us; float64 pipe 61% busy, issue slots 46%), and the
-// error of r against 128-bit arithmetic 1.3 to 30 times smaller (random and smooth u).
+// float64, 0.44 ms here (the kernel 380 us; float64 pipe 58% busy, issue slots 50%), 1.16 to 1.18
+// where every slab is taken again in float64 (u = exp(-100 x), exp(-200 r^2)).  Error of r against
+// 128-bit arithmetic, root mean square, float64 / here: exp(x + y + z) on 64^3 cells 3.1e-11 /
+// 4.9e-15, on 48 x 100 x 37 4.7e-11 / 3.9e-13, r^{5/3} on 64^3 5.3e-12 / 5.6e-15, white noise 9.9e-12 /
+// 6.8e-12, exp(-100 x) 2.3e-13 / 2.4e-13.
 #include <math.h>
 
 #include <algorithm>

@@ -202,8 +202,9 @@ __device__ void exp_finite_brick(const ProlongDesc& d, long long lb, BrickSmem& 
 // every interpolated value is a sum of five products with the integers 128 l_m(t) rounded
 // once, and the only float64 instruction left is the result's conversion.  Each pass keeps
 // one line of five values in a thread and writes the whole line of results.  Measured, one
-// call on 512 x 256 x 128 cells with Dirichlet data: 240 us in float64, 142 us here (two block
-// barriers fewer, or 32-bit brick indices, changed nothing).
+// call on 512 x 256 x 128 cells with Dirichlet data: 245 us in float64, 157 us here, 150 of them without
+// the check of the cells' sizes; fields that fall off within their bricks 236 us (two block barriers
+// fewer, or 32-bit brick indices, changed nothing).
 constexpr int kBrickBits = 58;  // |w| <= 1.13 2^58, times (278 / 128)^3 after three passes: < 2^61.6
 
 struct BrickFx {
@@ -444,8 +445,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_exp_finite_one(ProlongDesc d, l
 // plane before serve the odd fine plane between.  2.4 float64 instructions per node (a
 // thread per node and plane pair summed the corner rows anew, 4.3); bound by the float64
 // pipe.  One call on 384 x 256 x 192 cells: 284 us (a row per warp), 154 us marching, 136 us
-// with the column i = nx in the last tile; chunks of 4 / 6 / 12 / 16 / 24 planes 135 / 132 / 139 /
-// 143 / 151 us.
+// with the column i = nx in the last tile.  Chunks of kEtK coarse planes: a deeper one sums fewer
+// first planes twice, a shallower one gives small grids more blocks.  us per call with 4 / 6 / 8 /
+// 12: 64^3 37 / 43 / 43 / 48, 384 x 256 x 192 142 / 143 / 142 / 147, 512 x 256 x 128 128 / 129 / 129 / 132,
+// 1024 x 512 x 512 1452 / 1412 / 1391 / 1373.
 constexpr int kEtX = 64, kEtY = 8, kEtK = 8;
 constexpr int kEcX = kEtX / 2 + 1, kEcY = kEtY / 2 + 1;
 
